@@ -156,26 +156,39 @@ cudaError_t launch_plan(const StageDims &d, const StageBufs &b, int tile_bins, i
 }
 
 // ---------------------------------------------------------------------------- finish
-// Per walker, the sums of its slot over its group's items, taken in item order so the
-// result does not depend on which block ran which item.  FP64: ln L = <d|h> - <h|h>/2 -
-// <d|d>/2 (Eq. (2)).  Split: the parts hold sum (|h|^2 - 2 Re(d h*)) and <h|h>, and
-// ln L = -sum/2 - <d|d>/2.  A device wait that gave up poisons every output with NaN.
-__global__ void finish_kernel(StageDims d, StageBufs b, int G, int split, double dd, double *lnL,
-                              double *dh, double *hh) {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+// Per walker, the sums of its slot over its group's items: one warp per walker, each lane a
+// stride of the items, then a fixed tree, so the result does not depend on which block ran
+// which item.  FP64: ln L = <d|h> - <h|h>/2 - <d|d>/2 (Eq. (2)).  Split: the parts hold sum
+// (|h|^2 - 2 Re(d h*)) and <h|h>, and ln L = -sum/2 - <d|d>/2.  A device wait that gave up
+// poisons every output with NaN.
+//
+// A walker of the 1-yr grid has up to 3082 items; one thread summing them in series was
+// bound by the latency of dependent loads (620 us for five walkers, 778 us for 1024);
+// a warp per walker takes 6 us for one walker and 29 us for
+// 1024.
+__global__ void __launch_bounds__(128) finish_kernel(StageDims d, StageBufs b, int G, int split,
+                                                     double dd, double *lnL, double *dh, double *hh) {
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (w >= d.B) return;
+    const bool ok = b.valid[w] != 0;
     double a = 0.0, c = 0.0;
-    double out;
-    if (b.valid[w]) {
+    if (ok) {
         const int i = b.slot_of[w], g = i / G, k = i % G;
-        for (int it = b.item_start[g]; it < b.item_start[g + 1]; it++) {
-            a += b.part[2 * ((size_t)it * G + k)];
-            c += b.part[2 * ((size_t)it * G + k) + 1];
+        const int end = b.item_start[g + 1];
+        const double2 *part = reinterpret_cast<const double2 *>(b.part);
+#pragma unroll 4
+        for (int it = b.item_start[g] + lane; it < end; it += 32) {
+            const double2 v = part[(size_t)it * G + k];
+            a += v.x;
+            c += v.y;
         }
-        out = split ? -0.5 * a - 0.5 * dd : a - 0.5 * c - 0.5 * dd;
-    } else {
-        out = -INFINITY;
     }
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        c += __shfl_down_sync(0xffffffffu, c, o);
+    }
+    if (lane) return;
+    double out = !ok ? -INFINITY : split ? -0.5 * a - 0.5 * dd : a - 0.5 * c - 0.5 * dd;
     double dhv = split ? 0.5 * (c - a) : a;
     if (*b.err) {
         out = NAN;
@@ -189,7 +202,7 @@ __global__ void finish_kernel(StageDims d, StageBufs b, int G, int split, double
 
 cudaError_t launch_finish(const StageDims &d, const StageBufs &b, int group, int split, double dd,
                           double *lnL, double *dh, double *hh, cudaStream_t s) {
-    finish_kernel<<<(d.B + 127) / 128, 128, 0, s>>>(d, b, group, split, dd, lnL, dh, hh);
+    finish_kernel<<<(d.B + 3) / 4, 128, 0, s>>>(d, b, group, split, dd, lnL, dh, hh);
     return cudaGetLastError();
 }
 
