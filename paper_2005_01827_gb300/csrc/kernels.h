@@ -5,7 +5,7 @@
 
 namespace lisa {
 
-constexpr int kScratchRows = 11;  // rows of K doubles per (walker, mode) in mscratch
+constexpr int kScratchRows = 9;   // rows of K doubles per (walker, mode) in mscratch
 
 // Device layout of one bin of the uploaded data: the FP64 dense kernel reads the
 // nine doubles w_A, w_E, w_T, (w d)_A re/im, (w d)_E re/im, (w d)_T re/im
@@ -32,9 +32,8 @@ struct StageBufs {
     double *fk;            // [B][L][K]
     int *kb;               // [B][L][K]: first dense bin with f_j >= f_k
     double *vals;          // [B][L][8][K]
-    double *mscratch;      // [B][L][11][K]: spline second derivatives of the 8 series, then
-                           // the shared factorisation: 1/h (row 8) and the normalised
-                           // super-diagonal (row 10); row 9 is spare
+    double *mscratch;      // [B][L][9][K]: spline second derivatives of the 8 series, then
+                           // 1/h (row 8)
     double *coef;          // [B][L][K-1][8][4]
     int *wrange;           // [B][2] union of the walker's active mode ranges
     int *order;            // [B] walkers sorted by band (groups are runs of G entries)
@@ -54,8 +53,8 @@ struct StageBufs {
 // derivatives in mscratch, as in FP64) and the seven other series in FP32 inside the same
 // per-(walker, mode) storage: series q' = 0 (A 2^64) and 1..6 (Re, Im of T^A, T^E, T^T)
 // as FP32 rows of K values from double row 2 of vals (knot values) and of mscratch
-// (second derivatives), and FP32 copies of 1/h, h, 1/pivot and the normalised
-// super-diagonal as four FP32 rows from double row 6 of mscratch.
+// (second derivatives), and FP32 copies of 1/h and h as two FP32 rows from double row 6
+// of mscratch.
 constexpr int kSplitSeries32 = 7;
 __host__ __device__ inline float *split_vals32(double *vals, size_t wm, int K) {
     return reinterpret_cast<float *>(vals + (wm * 8 + 2) * (size_t)K);

@@ -1,0 +1,310 @@
+// spline.cu -- not-a-knot cubic splines of the knot values (the Scipy-type tridiagonal
+// solve of Katz et al. 2020, Sec. II.A) and the FP64 cubic coefficients.
+//
+// One block per (walker, mode) system; the unknowns are the second derivatives
+// M_1 .. M_{K-2} of each of the 8 series, not-a-knot eliminating M_0 and M_{K-1}.  The
+// matrix (shared by the series) has diagonal 2 (h_{i-1} + h_i) and off-diagonals h_{i-1},
+// h_i, so whatever a sweep starts from is forgotten by a factor of at least
+// h / (2 (h + h') - h c) per row, about 0.27 on the nearly even steps of log-spaced knots
+// (and below 0.36 for a step ratio up to 1.2): a row's value depends on rows kHalo = 32
+// away by less than 1e-14 of them, of the size of a sweep's own rounding.  So every thread
+// sweeps a chunk of rows of its own after kHalo rows of run-in, and a sweep of 1022 rows
+// takes 64 steps instead of 1022.  The pivots forget twice as fast and take 16 rows of
+// run-in.  (Few knots have large step ratios, up to 0.5 per row; up to K = 34 every row is
+// within the run-in of the last.)
+//
+// What bounds it: with few systems the latency of the sweep steps, so the series are dealt
+// to several blocks; with many systems the FP64 pipe (2 lanes per clock per SM): slopes and
+// right-hand sides are independent and use full warps, a sweep step is two or three FP64
+// operations.  Measured on GB300 (solve and coefficient kernel) against one
+// system per lane of one warp with every row in series: 1 system of 256 knots 367 -> 39 us,
+// 148 systems of 509 knots 938 -> 82 us, 6144 systems of 1024 knots 3.66 -> 3.11 ms in FP64
+// and 2.29 -> 1.55 ms in split precision.
+#include "kernels.h"
+#include "model.cuh"
+
+namespace lisa {
+
+namespace {
+constexpr int kThreads = 256;
+constexpr int kHalo = 32;        // run-in rows of a sweep
+constexpr int kPivotHalo = 16;   // run-in rows of the pivots
+constexpr size_t kMaxSmem = 227 * 1024;
+}  // namespace
+
+// Row arrays in shared memory hold entry i at at(i): chunks of C = 2^cs entries with an odd
+// pitch, so that threads sweeping different chunks hit different banks.
+struct Rows {
+    int cs, mask, pitch;
+    __host__ __device__ __forceinline__ int at(int i) const { return (i >> cs) * pitch + (i & mask); }
+};
+
+// chunk layout for `tps` sweeping threads per series
+__host__ __device__ inline Rows rows_of(int K, int tps) {
+    Rows r;
+    r.cs = 0;
+    while ((tps << r.cs) < K - 1) r.cs++;
+    r.mask = (1 << r.cs) - 1;
+    r.pitch = r.cs ? (1 << r.cs) + 1 : 1;
+    return r;
+}
+
+// sweeping threads per series of a block that owns nq series
+__host__ __device__ inline int sweep_threads(int nq) {
+    return nq > 4 ? 32 : nq > 2 ? 64 : nq > 1 ? 128 : 256;
+}
+
+// Forward sweep of one chunk: rp_i = (rhs_i - sub_i rp_{i-1}) / pivot_i in place.  `run`
+// selects the run-in (nothing stored) or the chunk itself.
+template <typename T>
+__device__ __forceinline__ T sweep_forward(T *y, const T *h, const T *ih, const T *inv, const Rows R,
+                                           int from, int to, int n, T prev, bool store) {
+    for (int i = from; i < to; i++) {
+        const int o = R.at(i);
+        const T hi = h[o];
+        T sb = h[R.at(i - 1)];
+        if (i == n - 2) sb -= hi * hi * ih[R.at(i - 1)];
+        const T rhs = y[o], dv = inv[o];
+        prev = (i == 1) ? rhs * dv : (rhs - sb * prev) * dv;
+        if (store) y[o] = prev;
+    }
+    return prev;
+}
+
+// Backward sweep of one chunk: M_i = rp_i - c_i M_{i+1}, rows to-1 down to from.
+template <typename T>
+__device__ __forceinline__ T sweep_backward(T *y, const T *c, const Rows R, int from, int to, int n,
+                                            T next, bool store) {
+    for (int i = to - 1; i >= from; i--) {
+        const int o = R.at(i);
+        next = (i == n - 2) ? y[o] : y[o] - c[o] * next;
+        if (store) y[o] = next;
+    }
+    return next;
+}
+
+// One stage of a series' solve (a barrier follows each): run-in and chunk of the forward
+// sweep, run-in and chunk of the backward sweep, the not-a-knot ends.  The run-ins read
+// entries that the neighbours' chunks overwrite, hence stages of their own.
+template <typename T>
+__device__ __forceinline__ void solve_stage(int stage, T &v, T *y, const T *h, const T *ih,
+                                            const T *inv, const T *c, const Rows R, int t, int n) {
+    const int C = R.mask + 1;
+    const int i0 = 1 + t * C, i1 = min(i0 + C, n - 1);
+    if (stage == 4) {  // M_0 and M_{K-1} from their neighbours
+        if (t != 0) return;
+        const T h0 = h[R.at(0)], h1 = h[R.at(1)], ha = h[R.at(n - 3)], hb = h[R.at(n - 2)];
+        y[R.at(0)] = ((h0 + h1) * y[R.at(1)] - h0 * y[R.at(2)]) * ih[R.at(1)];
+        y[R.at(n - 1)] = ((ha + hb) * y[R.at(n - 2)] - hb * y[R.at(n - 3)]) * ih[R.at(n - 3)];
+        return;
+    }
+    if (i0 >= n - 1) return;
+    if (stage == 0) v = sweep_forward(y, h, ih, inv, R, max(1, i0 - kHalo), i0, n, T(0), false);
+    if (stage == 1) sweep_forward(y, h, ih, inv, R, i0, i1, n, v, true);
+    if (stage == 2) v = sweep_backward(y, c, R, i1, min(n - 1, i1 + kHalo), n, T(0), false);
+    if (stage == 3) sweep_backward(y, c, R, i0, i1, n, v, true);
+}
+
+// kSplit: the phase (series 1) in FP64, the other seven in FP32 from their FP32 knot values
+// (the interpolant depends on M only through terms of order h^2 M, far below the values).
+// Block (s, y) owns series [y, y + 1) 8 / gridDim.y of system s.
+template <bool kSplit>
+__global__ void __launch_bounds__(kThreads) spline_kernel(StageDims d, StageBufs b) {
+    extern __shared__ __align__(16) unsigned char spl_sm[];
+    const int K = d.K, n = K, tid = threadIdx.x;
+    const size_t wm = blockIdx.x;
+    if (!b.band[wm * 3]) return;  // inactive modes (and invalid walkers) have no splines
+    const int per = kNSeries / gridDim.y;
+    const int q0 = blockIdx.y * per;
+    const int tps = sweep_threads(per);
+    const Rows R = rows_of(K, tps);
+    const int NP = R.at(K - 1) + 1;
+    double *h = reinterpret_cast<double *>(spl_sm), *ih = h + NP, *inv = ih + NP, *c = inv + NP;
+    // FP64 series, then (split) the FP32 copies of the matrix and the FP32 series; a block of
+    // one series holds only the kind it owns
+    double *ys = c + NP;  // [1 or per][NP]
+    float *h32 = reinterpret_cast<float *>(ys + (!kSplit ? per : per == 1 && q0 != 1 ? 0 : 1) * NP);
+    float *ih32 = h32 + NP, *inv32 = ih32 + NP, *c32 = inv32 + NP;
+    float *ys32 = c32 + NP;  // split: [per][NP] (phase slot unused)
+    const bool own32 = kSplit && !(per == 1 && q0 == 1);
+    const double *x = b.fk + wm * K;
+    const double *yg = b.vals + wm * kNSeries * (size_t)K;
+    const float *y32g = split_vals32(b.vals, wm, K);
+
+    for (int i = tid; i < n - 1; i += kThreads) {
+        const double hi = x[i + 1] - x[i], v = 1.0 / hi;
+        const int o = R.at(i);
+        h[o] = hi;
+        ih[o] = v;
+        if (own32) {
+            h32[o] = (float)hi;
+            ih32[o] = (float)v;
+        }
+    }
+    __syncthreads();
+    // warp 0: pivots and super-diagonal of its chunk of rows; the others: right-hand sides
+    // 6 (slope_i - slope_{i-1}) of the block's series
+    if (tid < 32) {
+        const int F = (n - 2 + 31) / 32, i0 = 1 + tid * F, i1 = min(i0 + F, n - 1);
+        double cp = 0.0;
+        for (int i = max(1, i0 - kPivotHalo); i < i1; i++) {
+            const int o = R.at(i), om = R.at(i - 1);
+            const double hp = h[om], hc = h[o];
+            double dia = 2.0 * (hp + hc), sup = hc, sb = hp;
+            if (i == 1) {
+                dia += hp * (hp + hc) * ih[o];
+                sup -= hp * hp * ih[o];
+            }
+            if (i == n - 2) {
+                dia += hc * (hp + hc) * ih[om];
+                sb -= hc * hc * ih[om];
+            }
+            const double v = 1.0 / ((i == 1) ? dia : dia - sb * cp);
+            cp = sup * v;
+            if (i >= i0) {
+                inv[o] = v;
+                c[o] = cp;
+                if (own32) {
+                    inv32[o] = (float)v;
+                    c32[o] = (float)cp;
+                }
+            }
+        }
+    } else {
+        for (int q = q0; q < q0 + per; q++) {
+            if (kSplit && q != 1) {
+                const float *y = y32g + (size_t)(q == 0 ? 0 : q - 1) * K;
+                float *o32 = ys32 + (size_t)(q - q0) * NP;
+                for (int i = 1 + tid - 32; i < n - 1; i += kThreads - 32) {
+                    const float sl = (y[i + 1] - y[i]) * ih32[R.at(i)];
+                    const float sp = (y[i] - y[i - 1]) * ih32[R.at(i - 1)];
+                    o32[R.at(i)] = 6.0f * (sl - sp);
+                }
+            } else {
+                const double *y = yg + (size_t)q * K;
+                double *o64 = ys + (size_t)(kSplit ? 0 : q - q0) * NP;
+                for (int i = 1 + tid - 32; i < n - 1; i += kThreads - 32) {
+                    const double sl = (y[i + 1] - y[i]) * ih[R.at(i)];
+                    const double sp = (y[i] - y[i - 1]) * ih[R.at(i - 1)];
+                    o64[R.at(i)] = 6.0 * (sl - sp);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    // a series' threads lie in whole warps, so the FP64 / FP32 choice is uniform per warp
+    const int ql = tid / tps, t = tid % tps;
+    double v64 = 0.0;
+    float v32 = 0.0f;
+    for (int stage = 0; stage < 5; stage++) {
+        if (ql < per) {
+            if (kSplit && q0 + ql != 1)
+                solve_stage<float>(stage, v32, ys32 + (size_t)ql * NP, h32, ih32, inv32, c32, R, t, n);
+            else
+                solve_stage<double>(stage, v64, ys + (size_t)(kSplit ? 0 : ql) * NP, h, ih, inv, c, R, t, n);
+        }
+        __syncthreads();
+    }
+
+    // second derivatives, 1/h and (split) the FP32 copies, coalesced
+    double *Mg = b.mscratch + wm * kScratchRows * (size_t)K;
+    float *M32g = split_m32(b.mscratch, wm, K), *F32g = split_fac32(b.mscratch, wm, K);
+    for (int q = q0; q < q0 + per; q++) {
+        if (kSplit && q != 1) {
+            const float *y = ys32 + (size_t)(q - q0) * NP;
+            float *o = M32g + (size_t)(q == 0 ? 0 : q - 1) * K;
+            for (int i = tid; i < n; i += kThreads) o[i] = y[R.at(i)];
+        } else {
+            const double *y = ys + (size_t)(kSplit ? 0 : q - q0) * NP;
+            for (int i = tid; i < n; i += kThreads) Mg[(size_t)q * K + i] = y[R.at(i)];
+        }
+    }
+    if (q0 == 0) {
+        for (int i = tid; i < n - 1; i += kThreads) {
+            Mg[kNSeries * (size_t)K + i] = ih[R.at(i)];
+            if (kSplit) {
+                F32g[i] = ih32[R.at(i)];
+                F32g[K + i] = h32[R.at(i)];
+            }
+        }
+    }
+}
+
+// Cubic coefficients of every (system, segment, series) from the second derivatives, as
+// a grid-stride kernel of its own (full occupancy whatever the solve's blocks hold).
+// kSplit: only the FP64 phase series (the others stay as FP32 values and second
+// derivatives for the segment records).
+template <bool kSplit>
+__global__ void __launch_bounds__(256) spline_coef_kernel(StageDims d, StageBufs b) {
+    const int K = d.K;
+    const long long per_sys = (long long)(K - 1) * (kSplit ? 1 : kNSeries);
+    const long long total = (long long)d.B * d.L * per_sys;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
+         t += (long long)gridDim.x * blockDim.x) {
+        const long long w2 = t / per_sys;
+        const int rem = (int)(t - w2 * per_sys);
+        if (!b.band[w2 * 3]) continue;
+        const int sgm = kSplit ? rem : rem / kNSeries, q = kSplit ? 1 : rem % kNSeries;
+        const double *x2 = b.fk + (size_t)w2 * K;
+        const double *M2 = b.mscratch + (size_t)w2 * kScratchRows * K;
+        const double *yq = b.vals + ((size_t)w2 * kNSeries + q) * K;
+        const double *Mq = M2 + (size_t)q * K;
+        const double h = x2[sgm + 1] - x2[sgm], hi = M2[(size_t)kNSeries * K + sgm];
+        const double m0 = Mq[sgm], m1 = Mq[sgm + 1];
+        double *c = b.coef + ((size_t)w2 * (K - 1) + sgm) * 32 + q * 4;
+        c[0] = yq[sgm];
+        c[1] = (yq[sgm + 1] - yq[sgm]) * hi - h * (2.0 * m0 + m1) * (1.0 / 6.0);
+        c[2] = 0.5 * m0;
+        c[3] = (m1 - m0) * hi * (1.0 / 6.0);
+    }
+}
+
+namespace {
+
+template <bool kSplit>
+size_t spline_smem(int K, int per) {
+    const Rows R = rows_of(K, sweep_threads(per));
+    const size_t NP = R.at(K - 1) + 1;
+    if (!kSplit) return NP * 8 * (4 + per);
+    return per == 1 ? NP * (8 * 4 + 4 * 5) : NP * (8 * 5 + 4 * (4 + per));
+}
+
+// Blocks per system: one while the systems fill the chip, more (each with fewer series,
+// the pivots repeated) while they do not or while a block's rows would not fit in shared
+// memory (K above about 2300).
+template <bool kSplit>
+int spline_blocks(int nsys, int K) {
+    int y = 1;
+    while (y < kNSeries && nsys * y * 2 <= 152 * 2) y *= 2;
+    while (y < kNSeries && spline_smem<kSplit>(K, kNSeries / y) > kMaxSmem) y *= 2;
+    return y;
+}
+
+template <bool kSplit>
+cudaError_t launch_spline_t(const StageDims &d, const StageBufs &b, cudaStream_t s) {
+    const int nsys = d.B * d.L, y = spline_blocks<kSplit>(nsys, d.K);
+    const size_t smem = spline_smem<kSplit>(d.K, kNSeries / y);
+    cudaError_t e = cudaFuncSetAttribute(spline_kernel<kSplit>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    spline_kernel<kSplit><<<dim3(nsys, y), kThreads, smem, s>>>(d, b);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const long long total = (long long)nsys * (d.K - 1) * (kSplit ? 1 : kNSeries);
+    const long long want = (total + 255) / 256, cap = 152LL * 8;  // 8 blocks per SM
+    const int blocks = (int)(want < cap ? want : cap);
+    spline_coef_kernel<kSplit><<<blocks, 256, 0, s>>>(d, b);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_spline(const StageDims &d, const StageBufs &b, cudaStream_t s) {
+    return launch_spline_t<false>(d, b, s);
+}
+
+cudaError_t launch_spline_split(const StageDims &d, const StageBufs &b, cudaStream_t s) {
+    return launch_spline_t<true>(d, b, s);
+}
+
+}  // namespace lisa
