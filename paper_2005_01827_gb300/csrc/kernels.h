@@ -12,6 +12,9 @@ constexpr int kScratchRows = 9;   // rows of K doubles per (walker, mode) in msc
 // (w = 4 df / S, Eqs. (3) and (11)); 72 bytes, 16-byte aligned rows of 2 bins.
 constexpr int kBinDoubles = 9;
 
+struct WalkerConst;  // response.cuh
+struct ModeConst;
+
 struct StageDims {
     int B;       // walkers in this call
     int L;       // modes
@@ -29,6 +32,8 @@ struct StageBufs {
     double *xpk;           // [B] peak of f^2 A_22 in M f
     int *band;             // [B][L][3]: active, j_lo, j_hi
     double *fedge;         // [B][L][2]
+    WalkerConst *wconst;   // [B] waveform and response constants of valid walkers
+    ModeConst *mconst;     // [B][L] the same per active mode
     double *fk;            // [B][L][K]
     int *kb;               // [B][L][K]: first dense bin with f_j >= f_k
     double *vals;          // [B][L][8][K]
@@ -77,8 +82,8 @@ struct DenseTune {
 __host__ __device__ inline int n_groups(int B, int G) { return (B + G - 1) / G; }
 
 cudaError_t launch_knots(const StageDims &d, const StageBufs &b, cudaStream_t s);
-// the band kernel alone (walker constants, peak, bands; no knots)
-cudaError_t launch_band(const StageDims &d, const StageBufs &b, cudaStream_t s);
+// the first half of it alone: walker constants, peak, bands; no knots
+cudaError_t launch_source(const StageDims &d, const StageBufs &b, cudaStream_t s);
 cudaError_t launch_spline(const StageDims &d, const StageBufs &b, cudaStream_t s);
 // split precision: FP64 phase, FP32 amplitude and transfer (layout above)
 cudaError_t launch_knots_split(const StageDims &d, const StageBufs &b, cudaStream_t s);

@@ -17,6 +17,7 @@
 #include "internal.h"
 #include "kernels.h"
 #include "model.cuh"
+#include "response.cuh"
 #include "split.h"
 
 using namespace lisa;
@@ -54,6 +55,8 @@ struct lisa_like {
     // per-call buffers
     double *params = nullptr, *tc = nullptr, *xpk = nullptr, *fedge = nullptr, *fk = nullptr;
     double *vals = nullptr;
+    WalkerConst *wconst = nullptr;
+    ModeConst *mconst = nullptr;
     double *mscr = nullptr, *coef = nullptr, *part = nullptr, *out = nullptr;
     int *valid = nullptr, *band = nullptr, *kb = nullptr, *wrange = nullptr;
     int *order = nullptr, *slot_of = nullptr, *grange = nullptr;
@@ -109,7 +112,7 @@ cudaError_t dalloc(T **p, size_t n) {
 
 void free_batch(lisa_like_t *h) {
     void *ptrs[] = {h->params, h->tc,    h->xpk,    h->fedge,  h->fk,  h->vals,  h->mscr,
-                    h->coef,   h->out,   h->valid,  h->band,   h->kb,         h->wrange,
+                    h->coef,   h->out,   h->wconst, h->mconst, h->valid,  h->band,   h->kb,         h->wrange,
                     h->order,  h->slot_of, h->grange, h->item_start, h->counter, h->err_flag};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -120,6 +123,8 @@ void free_batch(lisa_like_t *h) {
     h->segs = nullptr;
     h->phases = nullptr;
     h->params = h->tc = h->fedge = h->fk = h->vals = h->mscr = h->coef = h->out = nullptr;
+    h->wconst = nullptr;
+    h->mconst = nullptr;
     h->valid = h->band = h->kb = h->wrange = h->item_start = h->counter = nullptr;
     if (h->h_params) cudaFreeHost(h->h_params);
     if (h->h_out) cudaFreeHost(h->h_out);
@@ -136,6 +141,8 @@ lisa_status alloc_batch(lisa_like_t *h) {
     LCK(dalloc(&h->valid, B), "device allocation (valid)");
     LCK(dalloc(&h->band, B * L * 3), "device allocation (band)");
     LCK(dalloc(&h->fedge, B * L * 2), "device allocation (fedge)");
+    LCK(dalloc(&h->wconst, B), "device allocation (walker constants)");
+    LCK(dalloc(&h->mconst, B * L), "device allocation (mode constants)");
     LCK(dalloc(&h->fk, B * L * K), "device allocation (knots)");
     LCK(dalloc(&h->kb, B * L * K), "device allocation (knot bins)");
     LCK(dalloc(&h->vals, B * L * kNSeries * K), "device allocation (knot values)");
@@ -168,6 +175,8 @@ StageBufs bufs_of(const lisa_like_t *h, const double *params) {
     b.xpk = h->xpk;
     b.band = h->band;
     b.fedge = h->fedge;
+    b.wconst = h->wconst;
+    b.mconst = h->mconst;
     b.fk = h->fk;
     b.kb = h->kb;
     b.vals = h->vals;
@@ -342,7 +351,7 @@ lisa_status enqueue(lisa_like_t *h, const double *dparams, int B, double *lnL, d
     LCK(launch_finish(d, b, h->tune.group, split ? 1 : 0, h->dd, lnL, dh, hh, s),
         "finish kernel launch");
     LCK(mark(6), "cudaEventRecord");
-    h->last_launches = 8;  // band, knots, spline solve + coefficients, segments, plan, dense, finish
+    h->last_launches = 8;  // source, knots, spline solve + coefficients, segments, plan, dense, finish
     return LISA_OK;
 }
 

@@ -15,6 +15,7 @@
 #include "../../include/lisa_like.h"
 #include "kernels.h"
 #include "model.cuh"
+#include "response.cuh"
 
 namespace lisa {
 void set_thread_error(const std::string &msg);  // defined in lisa_like.cu
@@ -43,7 +44,7 @@ void *g_addr[kMaxDevices] = {nullptr};
 size_t up256(size_t n) { return (n + 255) & ~(size_t)255; }
 
 struct Layout {
-    size_t valid, tc, xpk, band, fedge, fk, kb, vals, mscr, coef, phases, wrange, order, slot,
+    size_t valid, tc, xpk, band, fedge, wconst, mconst, fk, kb, vals, mscr, coef, phases, wrange, order, slot,
         grange, items,
         counter, err, part, end;
 };
@@ -66,6 +67,12 @@ Layout layout_for(size_t B, size_t L, size_t K, size_t items) {
     o.vals = take(sizeof(double) * B * L * kNSeries * K);
     o.mscr = take(sizeof(double) * B * L * kScratchRows * K);
     o.coef = take(sizeof(double) * B * L * (K - 1) * 32);
+    // the walker and mode constants are dead once the knots exist, before any coefficient is
+    // written: they share its space
+    o.wconst = o.coef;
+    o.mconst = o.coef + up256(sizeof(WalkerConst) * B);
+    static_assert(sizeof(WalkerConst) + sizeof(ModeConst) <= 3 * 256 - 176 && sizeof(WalkerConst) <= 512,
+                  "constants fit in the coefficients of a system of four knots");
     // the knot values are dead once the splines exist: the phase records reuse them
     o.phases = o.vals;
     static_assert(sizeof(unsigned long long) * kPhaseWords <= sizeof(double) * kNSeries,
@@ -160,6 +167,8 @@ extern "C" lisa_status lisa_like_loglike_noalloc(const lisa_like_config *cfg, do
     b.xpk = reinterpret_cast<double *>(s8 + o.xpk);
     b.band = reinterpret_cast<int *>(s8 + o.band);
     b.fedge = reinterpret_cast<double *>(s8 + o.fedge);
+    b.wconst = reinterpret_cast<WalkerConst *>(s8 + o.wconst);
+    b.mconst = reinterpret_cast<ModeConst *>(s8 + o.mconst);
     b.fk = reinterpret_cast<double *>(s8 + o.fk);
     b.kb = reinterpret_cast<int *>(s8 + o.kb);
     b.vals = reinterpret_cast<double *>(s8 + o.vals);

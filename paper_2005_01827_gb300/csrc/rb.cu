@@ -371,7 +371,7 @@ lisa_status enqueue_rb(lisa_like_t *h, const RbState *s, const double *d_params,
     StageBufs b = c.stage;
     b.params = d_params;
     const StageDims d = dims_of(c, B);
-    cudaError_t e = launch_band(d, b, st);
+    cudaError_t e = launch_source(d, b, st);
     if (e == cudaSuccess) {
         rb_walker_kernel<<<B, kRbThreads, walker_smem(s), st>>>(dev_of(c, s), d, b, lnL, dh, hh);
         e = cudaGetLastError();
@@ -400,7 +400,7 @@ lisa_status lisa_like_set_fiducial(lisa_like_t *h, const double *params, int n_r
     std::memcpy(c.h_params, params, sizeof(double) * kNPar);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c.params, c.h_params, sizeof(double) * kNPar, cudaMemcpyHostToDevice, s);
     const StageDims d1 = dims_of(c, 1);
-    if (e == cudaSuccess) e = launch_band(d1, c.stage, s);
+    if (e == cudaSuccess) e = launch_source(d1, c.stage, s);
     std::vector<int> band(3 * c.L);
     std::vector<double> fedge(2 * c.L);
     int valid = 0;

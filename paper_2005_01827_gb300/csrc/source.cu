@@ -1,0 +1,317 @@
+// source.cu -- everything that a walker's knots share, computed once per walker (Katz et al.
+// 2020, Sec. II): the waveform constants, the peak of f^2 A_22, the band of every mode
+// (the cut where t_lm(f) < 0 and the ringdown cut) with its integer dense-bin range, and
+// the coefficients of the response in the constellation's orbital harmonics.
+//
+// One warp per walker.  Both roots (the peak, and the frequency where the signal starts,
+// which is one mapped frequency x = 2 M f / m for all modes) are bracketed by two rounds
+// of 31 points, one per lane (five bisections a round), and finished by Newton steps.
+// What bounds it is the latency of one evaluation after another (about 2 us each: cube
+// root, divisions), so their number is what counts: about 16 against 94 of two bisections
+// to 1e-14 in one thread.  Source and knots together, one walker, one mode, 256 knots: 281 ->
+// 98 us.
+#include "kernels.h"
+#include "model.cuh"
+#include "response.cuh"
+
+namespace lisa {
+
+// f_j = f0 + j df, rounded as a separate product and sum (no fused multiply-add) so
+// that band edges and knot-to-bin boundaries are decided exactly as written.
+__device__ __forceinline__ double bin_freq(double f0, double df, int j) {
+    return __dadd_rn(f0, __dmul_rn((double)j, df));
+}
+
+// index in [0, 31] of the interval that five bisections on the sign (true: the root lies
+// above) of 31 interior points would end in; bit i of `above` belongs to point i, i = 1..31
+__device__ __forceinline__ int bisect32(unsigned above) {
+    int pos = 0;
+    for (int step = 16; step > 0; step >>= 1)
+        if ((above >> (pos + step)) & 1u) pos += step;
+    return pos;
+}
+
+// peak of f^2 A_22 (t_coal is reached there, Sec. II): the zero of its log-derivative over
+// [x_RD / 4, 2 x_RD], or the end of that range that it lies beyond
+__device__ double find_peak_warp(const Source &s, int lane) {
+    double lo = 0.25 * s.xrd, hi = 2.0 * s.xrd;
+    if (peak_equation(s, lo) <= 0.0) return lo;
+    if (peak_equation(s, hi) >= 0.0) return hi;
+    for (int round = 0; round < 2; round++) {
+        const double st = (hi - lo) * (1.0 / 32.0);
+        const unsigned up = __ballot_sync(0xffffffffu, peak_equation(s, lo + st * lane) > 0.0);
+        const int p = bisect32(up);
+        hi = (p == 31) ? hi : lo + st * (p + 1);
+        lo = lo + st * p;
+    }
+    double x = 0.5 * (lo + hi);
+    for (int it = 0; it < 6; it++) {
+        const double v = cbrt(kPi * x), r = x / s.xrd, r2 = r * r, r6 = r2 * r2 * r2;
+        const double q2 = s.al2 * v * v, q3 = s.al3 * v * v * v, den = 1.0 / (1.0 + r6);
+        const double g = 5.0 / 6.0 + (2.0 / 3.0) * q2 + q3 - 6.0 * r6 * den;
+        const double gx = (4.0 / 9.0) * q2 + q3 - 36.0 * r6 * den * den;  // x dg/dx
+        if (g > 0.0)
+            lo = fmax(lo, x);
+        else
+            hi = fmin(hi, x);
+        double nx = x - x * g / gx;
+        if (!(nx >= lo && nx <= hi)) nx = 0.5 * (lo + hi);
+        const double dx = fabs(nx - x);
+        x = nx;
+        if (dx <= 1e-15 * x) break;
+    }
+    return x;
+}
+
+// t_22 at the mapped frequency x
+__device__ __forceinline__ double time_at(const Source &s, double x) {
+    return s.tc - s.M / kTwoPi * (raw_slope(s, x) - s.dphpk);
+}
+
+// mapped frequency where t_22 = 0, inside [xa, xb] with t(xa) < 0 <= t(xb): t rises with x
+__device__ double find_start_warp(const Source &s, double xa, double xb, int lane) {
+    double lo = xa, hi = xb;
+    for (int round = 0; round < 2; round++) {
+        const double st = log(hi / lo) * (1.0 / 32.0);
+        const double x = lo * exp(st * lane);
+        const int p = bisect32(__ballot_sync(0xffffffffu, time_at(s, x) < 0.0));
+        const double l2 = __shfl_sync(0xffffffffu, x, p), h2 = __shfl_sync(0xffffffffu, x, (p + 1) & 31);
+        lo = p == 0 ? lo : l2;
+        hi = p == 31 ? hi : h2;
+    }
+    double x = 0.5 * (lo + hi);
+    for (int it = 0; it < 8; it++) {
+        const double t = time_at(s, x);
+        const double d2 = x <= kXJoin ? inspiral_phase(s, x).d2p : -2.0 * s.c2 / (x * x * x);
+        if (t < 0.0)
+            lo = fmax(lo, x);
+        else
+            hi = fmin(hi, x);
+        double nx = x + t / (s.M / kTwoPi * d2);
+        if (!(nx >= lo && nx <= hi)) nx = 0.5 * (lo + hi);
+        const double dx = fabs(nx - x);
+        x = nx;
+        if (dx <= 1e-15 * x) break;
+    }
+    return x;
+}
+
+// A vector's component along a combination of spacecraft positions, in units of the arm:
+// v . sum_i g_i q_i / L as {1, cos 2a, sin 2a, cos a, sin a} coefficients, with
+// cb = sum g_i cos b_i and sb = sum g_i sin b_i (b_i = 2 pi i / 3), a the orbital angle
+__device__ __forceinline__ void harmonics(const double v[3], double cb, double sb, double o[5]) {
+    const double p = 1.0 / (4.0 * sqrt(3.0));
+    o[0] = -3.0 * p * (v[0] * cb + v[1] * sb);
+    o[1] = p * (v[0] * cb - v[1] * sb);
+    o[2] = p * (v[0] * sb + v[1] * cb);
+    o[3] = -0.5 * v[2] * cb;
+    o[4] = -0.5 * v[2] * sb;
+}
+
+__global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (w >= d.B) return;
+    Source src;
+    const bool ok = make_source_core(b.params + (size_t)w * kNPar, d.t0, src);
+    const double fmn = d.f0, fmx = bin_freq(d.f0, d.df, d.N - 1);
+    if (ok) set_peak(src, find_peak_warp(src, lane));
+    // lanes 0 .. L-1: one mode each
+    const bool mode = lane < d.L;
+    Mode md = {2, 2};
+#pragma unroll
+    for (int i = 0; i < kMaxModes; i++)
+        if (i == lane && i < d.L) md = {d.ml[i], d.mm[i]};
+    bool act = false, whole = false;
+    double lo = 0.0, hi = 0.0;
+    if (ok && mode) {
+        const double fcut = 0.5 * md.m * kXCut / src.M;
+        hi = fmx < fcut ? fmx : fcut;
+        act = hi > fmn * (1.0 + 1e-12);
+        if (act) {
+            whole = mode_time(src, md, fmn) >= 0.0;
+            if (whole)
+                lo = fmn;
+            else if (mode_time(src, md, hi) < 0.0)
+                act = false;  // the mode ends before the observation starts
+        }
+    }
+    // the modes that start inside the observation share one mapped starting frequency
+    const bool inside = act && !whole;
+    if (__any_sync(0xffffffffu, inside)) {
+        double xa = inside ? mapped_x(src, md, fmn) : INFINITY, xb = inside ? mapped_x(src, md, hi) : 0.0;
+        for (int o = 16; o > 0; o >>= 1) {
+            xa = fmin(xa, __shfl_xor_sync(0xffffffffu, xa, o));
+            xb = fmax(xb, __shfl_xor_sync(0xffffffffu, xb, o));
+        }
+        const double x0 = find_start_warp(src, xa, xb, lane);
+        if (inside) lo = fmin(hi, fmax(fmn, 0.5 * md.m * x0 / src.M));
+    }
+    int jl = 0, jh = -1;
+    if (act && !(hi > lo * (1.0 + 1e-12))) act = false;
+    if (act) {
+        const double gl = ceil((lo - d.f0) / d.df - 1e-9);
+        const double gh = floor((hi - d.f0) / d.df + 1e-9);
+        jl = gl < 0.0 ? 0 : (int)gl;
+        jh = gh > (double)(d.N - 1) ? d.N - 1 : (int)gh;
+        if (jl > jh) act = false;
+    }
+    if (mode) {
+        const size_t wm = (size_t)w * d.L + lane;
+        int *bd = b.band + wm * 3;
+        bd[0] = act ? 1 : 0;
+        bd[1] = act ? jl : 0;
+        bd[2] = act ? jh : -1;
+        b.fedge[wm * 2] = lo;
+        b.fedge[wm * 2 + 1] = hi;
+    }
+    if (lane == 0) {
+        b.valid[w] = ok ? 1 : 0;
+        b.tc[w] = ok ? src.tc : 0.0;
+        b.xpk[w] = ok ? src.xpk : 0.0;
+    }
+    if (!ok) return;
+    if (act) {  // this lane's mode
+        ModeConst c;
+        cplx kp, kc;
+        pol_weights(src, md, kp, kc);
+        double s2, c2;
+        sincos(2.0 * src.psi, &s2, &c2);
+        c.are = kp.re * c2 - kc.re * s2;
+        c.aim = kp.im * c2 - kc.im * s2;
+        c.bre = 2.0 * (kp.re * s2 + kc.re * c2);
+        c.bim = 2.0 * (kp.im * s2 + kc.im * c2);
+        c.xf = 2.0 * src.M / md.m;
+        c.v0 = cbrt(kPi * (c.xf * lo));
+        c.x160 = sqrt(c.v0 * kInvCbrtPi);
+        c.s6 = log(hi / lo) / (6.0 * (double)(d.K - 1));
+        c.amp = src.amp0 * amp_ratio(src, md, 1.0);
+        c.off = phase_offset(md) - 0.5 * md.m * (src.phpk - src.dphpk * src.xpk);
+        c.half_m = 0.5 * md.m;
+        c.power = amp_power(md);
+        c.pad = 0;
+        b.mconst[(size_t)w * d.L + lane] = c;
+    }
+    if (lane == 0) {
+        WalkerConst c;
+        c.k128 = src.k128;
+        c.ps2 = src.ps2;
+        c.ps3 = src.ps3;
+        c.phj = src.phj - src.c1 * kXJoin + src.c2 / kXJoin;
+        c.c1 = src.c1;
+        c.c2 = src.c2;
+        c.dphpk = src.dphpk;
+        c.tc = src.tc;
+        c.m2pi = src.m2pi;
+        c.al2 = src.al2;
+        c.al3 = src.al3;
+        c.ixrd = 1.0 / src.xrd;
+        double sl, cl, sb, cb;
+        sincos(src.lam, &sl, &cl);
+        sincos(src.beta, &sb, &cb);
+        const double u[3] = {sl, -cl, 0.0}, p[3] = {-sb * cl, -sb * sl, cb};
+        const double k[3] = {-cb * cl, -cb * sl, -sb};
+        const double h = 0.8660254037844386467637;  // cos, sin of 0, 2 pi / 3, 4 pi / 3
+        // arms 0 -> 1 and 1 -> 2 (differences) and their sums
+        harmonics(k, -1.5, h, c.kn[0]);
+        harmonics(k, 0.0, -2.0 * h, c.kn[1]);
+        harmonics(k, 0.5, h, c.kq[0]);
+        harmonics(k, -1.0, 0.0, c.kq[1]);
+        harmonics(p, -1.5, h, c.wn[0]);
+        harmonics(p, 0.0, -2.0 * h, c.wn[1]);
+        double o[5];
+        harmonics(u, -1.5, h, o);
+        for (int i = 0; i < 3; i++) c.un[0][i] = o[i];
+        harmonics(u, 0.0, -2.0 * h, o);
+        for (int i = 0; i < 3; i++) c.un[1][i] = o[i];
+        const double R = kAuM / kClight;
+        c.dx = -kTwoPi * R * k[0];
+        c.dy = -kTwoPi * R * k[1];
+        b.wconst[w] = c;
+    }
+}
+
+cudaError_t launch_source(const StageDims &d, const StageBufs &b, cudaStream_t s) {
+    source_kernel<<<(d.B + 3) / 4, 128, 0, s>>>(d, b);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------- knots
+// One thread per knot, 128 knots of one (walker, mode) per block: log-spaced frequencies
+// (Sec. II.A: ~2^10 points) with A, phase + delay, and T, and the first dense bin at or
+// above each.  kSplit: the same FP64 values, A (times 2^64) and T stored as FP32 (the
+// split-precision layout).
+//
+// Bound by the FP64 pipe (2 lanes per clock per SM), so the count of FP64 operations per
+// knot is what matters (about 420 against 730): the powers of f come from one
+// exponential of the log-spaced step (f^(1/6) and its powers, no cube root or square root),
+// one division serves v, the amplitude and the three arms, and the response is in orbital
+// harmonics (response.cuh).  6144 systems of 1024 knots: 8.4 -> 5.4 ms with the
+// source kernel.  One block of 128 threads per system left all but a few SMs idle in small
+// calls (6 systems of 1024 knots: 246 us), hence one knot per thread.
+template <bool kSplit>
+__global__ void __launch_bounds__(128) knot_kernel(StageDims d, StageBufs b) {
+    const size_t wm = blockIdx.x;
+    if (!b.band[wm * 3]) return;  // inactive modes (and invalid walkers) have no knots
+    __shared__ WalkerConst wc;
+    __shared__ ModeConst mc;
+    {
+        const double *src = reinterpret_cast<const double *>(b.wconst + wm / d.L);
+        double *dst = reinterpret_cast<double *>(&wc);
+        if (threadIdx.x < sizeof(WalkerConst) / 8) dst[threadIdx.x] = src[threadIdx.x];
+        const double *msrc = reinterpret_cast<const double *>(b.mconst + wm);
+        double *mdst = reinterpret_cast<double *>(&mc);
+        if (threadIdx.x >= 96 && threadIdx.x - 96 < sizeof(ModeConst) / 8)
+            mdst[threadIdx.x - 96] = msrc[threadIdx.x - 96];
+    }
+    __syncthreads();
+    const int K = d.K, k = blockIdx.y * blockDim.x + threadIdx.x;
+    if (k >= K) return;
+    const double flo = b.fedge[wm * 2], fhi = b.fedge[wm * 2 + 1];
+    const double e6 = exp(mc.s6 * (double)k), e3 = e6 * e6;
+    const double f = (k == K - 1) ? fhi : flo * (e3 * e3 * e3);
+    b.fk[wm * K + k] = f;
+    // first dense bin at or above this knot: a guess, then exact by the bin frequencies
+    // themselves
+    const double g = ceil((f - d.f0) / d.df);
+    int j = g <= 0.0 ? 0 : (g >= (double)d.N ? d.N : (int)g);
+    while (j > 0 && bin_freq(d.f0, d.df, j - 1) >= f) j--;
+    while (j < d.N && bin_freq(d.f0, d.df, j) < f) j++;
+    b.kb[wm * K + k] = j;
+    double amp, ph;
+    cplx T[3];
+    mode_response(wc, mc, f, mc.v0 * e3, mc.x160 * e6, amp, ph, T);
+    double *vm = b.vals + wm * kNSeries * (size_t)K;
+    vm[1 * K + k] = ph;
+    if (kSplit) {
+        float *v32 = split_vals32(b.vals, wm, K);
+        v32[k] = (float)(amp * kAmpScale64);
+        for (int c = 0; c < 3; c++) {
+            v32[(1 + 2 * c) * K + k] = (float)T[c].re;
+            v32[(2 + 2 * c) * K + k] = (float)T[c].im;
+        }
+    } else {
+        vm[0 * K + k] = amp;
+        for (int c = 0; c < 3; c++) {
+            vm[(2 + 2 * c) * K + k] = T[c].re;
+            vm[(3 + 2 * c) * K + k] = T[c].im;
+        }
+    }
+}
+
+template <bool kSplit>
+static cudaError_t launch_knots_t(const StageDims &d, const StageBufs &b, cudaStream_t s) {
+    cudaError_t e = launch_source(d, b, s);
+    if (e != cudaSuccess) return e;
+    knot_kernel<kSplit><<<dim3(d.B * d.L, (d.K + 127) / 128), 128, 0, s>>>(d, b);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_knots(const StageDims &d, const StageBufs &b, cudaStream_t s) {
+    return launch_knots_t<false>(d, b, s);
+}
+
+cudaError_t launch_knots_split(const StageDims &d, const StageBufs &b, cudaStream_t s) {
+    return launch_knots_t<true>(d, b, s);
+}
+
+}  // namespace lisa
