@@ -174,8 +174,8 @@ lisa_status lisa_like_loglike_noalloc(const lisa_like_config *cfg, double f0, do
                                       double *d_dh, double *d_hh, void *stream);
 
 /* Test of the device-side timeout path (the paper has no counterpart).  With polls > 0
- * the dense kernels of later calls on this handle arm each data tile's barrier for the
- * tile's bytes but issue no copy, so every wait on it gives up after `polls` polls with
+ * the dense kernels of later calls on this handle arm the barrier of each staged copy for
+ * its bytes but issue no copy, so every wait on it gives up after `polls` polls with
  * no copy in flight: the call then returns LISA_ERR_TIMEOUT (loglike) or NaN outputs
  * (loglike_device), exactly as when a real staging copy never completes.  polls = 0
  * restores normal operation.  Errors: LISA_ERR_ARG for polls outside [0, 2^20]. */
@@ -188,8 +188,8 @@ lisa_status lisa_like_test_device_wait(lisa_like_t *h, int polls);
  * replays. */
 lisa_status lisa_like_set_graphs(lisa_like_t *h, int on);
 
-/* Tile shape of the fused dense kernel: `per_thread` consecutive bins per thread (the
- * tile is 128 x per_thread bins) and `group` walkers sharing one staged data tile.
+/* Tile shape of the fused dense kernel: tiles of 128 x per_thread bins and `group` walkers
+ * per work item.
  * Supported: (8,8), (4,8), (16,8) in split precision only, (8,1).  LISA_ERR_ARG
  * otherwise.  out[3] of get_tune: per_thread, group, persistent blocks. */
 lisa_status lisa_like_set_tune(lisa_like_t *h, int per_thread, int group);

@@ -1,60 +1,105 @@
-// dense.cu -- the fused FP64 dense kernel of the batched LISA likelihood (Katz et al.
-// 2020, Sec. II.A): spline interpolation of A, phase and T onto the dense bins, the mode
+// dense.cu -- the fused dense kernel of the FP64 path of the batched LISA likelihood (Katz et
+// al. 2020, Sec. II.A): spline interpolation of A, phase and T onto the dense bins, the mode
 // sum, and the noise-weighted inner products of Eqs. (3) and (11), reduced to one
 // (<d|h>, <h|h>) pair per (work item, walker).  The dense template is never stored.
 //
-// Work item = (walker group, tile of consecutive bins inside the group's union band).
-// One bulk copy (TMA) stages the tile's w and w d (72 bytes per bin) in shared memory;
-// every walker of the group then reads them from there.  Blocks are persistent and pull
-// items from a counter.
+// Arithmetic.  GB300's FP64 pipe does 2 operations per clock and SM, and a (walker, mode,
+// bin) takes 47 of them, so evaluated in FP64 this kernel ran at that pipe's speed (94 %
+// busy) and took 98 % of a call.  Here the per-bin work is in 64-bit fixed point on the
+// integer multiply-add units (28 times the rate; fixed.cuh), with as many bits as FP64 has:
+//   * the phase phi - 2 pi f t_coal advances from bin to bin by exact 64-bit forward
+//     differences (anchored per spline segment by an FP64 prologue), and e^{i phase} comes
+//     from a table and short polynomials, to 1e-16; modes with the same m have the same
+//     phase and share it;
+//   * the amplitude and the six transfer cubics are re-expanded in FP64 where a segment
+//     enters a warp's block of 128 bins, scaled by a power of two that bounds them over its
+//     bins there, and advance by 64-bit forward differences; A e^{i phase} T is summed over
+//     the modes in 64 bits, relative to the largest mode of the block and channel (2^-54 of
+//     it per term);
+//   * the integrand is summed in FP32 pairs (48 bits: products with their exact errors,
+//     two-sums) over a thread's bins, and in FP64 from there up.
+// Terms are thus exact to about 1e-14 of the largest mode's, and the knots' FP64 phases
+// (1e-12 to 1e-9 rad) set the error as they did: against 64-bit sums of the same splines the
+// errors of ln L, <d|h> and <h|h> are those of the FP64 evaluation (1024 walkers: 7.1e-11
+// both).  Where a warp's bins hold a segment of fewer than 8 bins or more than 14 segments
+// of one mode, or a value is infinite, NaN or beyond the exponents handled, they are
+// evaluated in FP64 (dense_direct).
 //
-// The phase phi - 2 pi f t_coal of each mode advances from bin to bin by exact 64-bit
-// fixed-point forward differences (anchored per spline segment by an FP64 prologue),
-// and e^{i phase} is a 1024-entry FP64 table entry rotated by a short polynomial in the
-// remaining angle (< 2 pi / 1024): every floating-point operation stays FP64.
+// Work.  An item is (walker group, tile of consecutive bins inside the group's union band);
+// blocks are persistent and pull items from a counter.  An item is split into units of 128
+// bins and two walkers, one warp each; a lane has 4 consecutive bins.  Nothing but the
+// phasor table (one TMA bulk copy per block) is shared between warps, so they meet only at
+// the end of an item.  The mode sums of a warp's bins are kept in shared memory (6 KB): the
+// loop over a lane's bins is then a loop in the code too, which stays within the
+// instruction cache, and 128 registers hold the 7 cubics and the phase (16 warps per SM).
+// With the sums in registers (the bins unrolled, 8 warps per SM, 255 registers) a third of
+// all issue slots waited for instructions: 428 ms against 219 (below).  The data rows (76 bytes
+// per bin, float pairs) are read from L2 by each walker.
+//
+// Bound by the multiply-add pipe (66 % busy: 143 integer multiply-adds per (walker, mode,
+// bin), 58 % of issue slots).  1024 walkers, six modes, 1-yr grid: 951 -> 219 ms; 37 walkers,
+// four modes, quarter-year grid: 2063 -> 917 us; one walker, (2,2), 30 days: 61 -> 35 us.
+#include "f32x2.cuh"
+#include "fixed.cuh"
 #include "kernels.h"
 #include "model.cuh"
 #include "tma.cuh"
 
 namespace lisa {
 
-__device__ __forceinline__ double bin_freq_d(double f0, double df, int j) {
-    return __dadd_rn(f0, __dmul_rn((double)j, df));
-}
+namespace {
 
-__device__ __forceinline__ int segment_of(const int *__restrict__ kb, int K, int j) {
-    int lo = 0, hi = K - 2;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(kb + mid) <= j)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
+constexpr int kC = kFxRows;    // consecutive bins of a thread
+constexpr int kBlk = 32 * kC;  // bins of a warp: one block of expansions
+constexpr int kWarps = 8;      // warps per block
+constexpr int kTasks = 14;     // expansions a warp holds at a time
+constexpr int kSer = 7;        // A, then Re/Im of T^A, T^E, T^T
+constexpr int kABits = 62, kTBits = 61;  // A is scaled below 2^62, T below 2^61
+constexpr int kNoScale = -10000;
+// Shortest segment for the expansions: over a bin or more per segment the differences no
+// longer fall with their order.
+constexpr int kMinSeg = 8;
 
-// Horner evaluation of the amplitude and transfer cubics (series 0, 2..7) of one segment
-// at offset x; the phase series is carried by the fixed-point recurrence instead.
-__device__ __forceinline__ void eval_segment(const double *__restrict__ c, double x,
-                                             double v[kNSeries]) {
-    const double2 *c2 = reinterpret_cast<const double2 *>(c);
-#pragma unroll
-    for (int q = 0; q < kNSeries; q++) {
-        if (q == 1) continue;
-        const double2 lo = __ldg(c2 + 2 * q);
-        const double2 hi = __ldg(c2 + 2 * q + 1);
-        v[q] = fma(x, fma(x, fma(x, hi.y, hi.x), lo.y), lo.x);
-    }
-}
+// One (mode, segment) in a warp's block of bins, at the block's first bin or 3 bins before
+// the segment's (a thread's 4 bins may begin there): value and forward differences of the
+// seven series in fixed point, and (index kSer) of the phase in fractions of a turn scaled by
+// 2^64; l2, l3 and low hold the next 32 bits of the differences.
+struct __align__(16) Expand {
+    i64 vd[kSer + 1][2];  // value, first difference
+    i64 d2[kSer + 1];
+    int2 d3[kSer];        // third difference, l2
+    i64 ph3;              // third difference of the phase
+    uint32_t l3[kSer], low[3];
+    int org, kb, next;    // origin, first bin of the segment and of the next one
+    int pad[3];
+};
+static_assert(sizeof(Expand) == 320, "16-byte loads of a series' value and first difference");
 
 struct Phase64 {
     unsigned long long ph, d1, d2, d3;
 };
 
+// shared memory of a warp
+struct WarpMem {
+    i64 H[kC][6][32];  // the mode sums of each thread's bins
+    i64 z[kC][2][32];  // e^{i phase} of each thread's bins, for modes with the same phase
+    Expand ex[kTasks];
+};
+
+struct SmemF64 {
+    FxTab tab[kFxTab];
+    WarpMem w[kWarps];
+};
+
+}  // namespace
+
+__device__ __forceinline__ double bin_freq_d(double f0, double df, int j) {
+    return __dadd_rn(f0, __dmul_rn((double)j, df));
+}
+
 // fixed-point forward differences of a segment's phase moved to bin n of the segment
 // (Newton's forward-difference formula in modular arithmetic; for n > 0 the low words
-// add the carries of the 128-bit products)
+// add the carries of the 128-bit products; n >= -8)
 __device__ __forceinline__ Phase64 phase64_at(const unsigned long long *__restrict__ r, int n) {
     const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2 *>(r));
     const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2 *>(r) + 1);
@@ -77,26 +122,15 @@ __device__ __forceinline__ Phase64 phase64_at(const unsigned long long *__restri
     return p;
 }
 
-// e^{2 pi i ph / 2^64} in FP64: the top 10 bits select e^{2 pi i k / 1024}, the next 52
-// bits give r < 2 pi / 1024 = R, sin r is its Taylor polynomial to r^5 (truncation below
-// 1e-19) and cos r = 1 - s/2 + c s^2 with s = r^2: the s^3 term of the Taylor series is
-// absorbed into c, chosen so that the error c s^2 - (1/24 - s/720 + ...) s^2 equioscillates
-// over s in [0, R^2] (c = 1/24 - k R^2 with 76800 k^3 + k = 1/720; truncation below 8e-18)
-constexpr double kStep64 = 6.1359231515425647e-03;  // 2 pi / 1024
-constexpr double kCos2 = 0.041666619912852754;
-
-__device__ __forceinline__ void phasor64(unsigned long long ph, const double2 *__restrict__ tab,
-                                         double &zr, double &zi) {
-    const double2 t = tab[ph >> 54];
-    // x in [1, 2) carries the next 52 bits; fma(x, step, -step) = (x - 1) step exactly
-    // rounded once, as (x - 1) is exact
-    const double x = __longlong_as_double(0x3ff0000000000000ull | ((ph << 10) >> 12));
-    const double r = fma(x, kStep64, -kStep64);
-    const double r2 = r * r;
-    const double sn = r * fma(r2, fma(r2, 1.0 / 120.0, -1.0 / 6.0), 1.0);
-    const double cs = fma(r2, fma(r2, kCos2, -0.5), 1.0);
-    zr = fma(t.x, cs, -t.y * sn);
-    zi = fma(t.x, sn, t.y * cs);
+// segment of bin j: kb[s] <= j < kb[s + 1] (the last one open), from the log spacing of the
+// knots moved by the integer knot-to-bin boundaries
+__device__ __forceinline__ int segment_at(const int *__restrict__ kb, int K, int j, float f, float l0,
+                                          float scale) {
+    int s = (int)fmaf(__log2f(f), scale, -l0);
+    s = min(max(s, 0), K - 2);
+    while (s > 0 && __ldg(kb + s) > j) s--;
+    while (s < K - 2 && __ldg(kb + s + 1) <= j) s++;
+    return s;
 }
 
 // group of a work item: largest g with item_start[g] <= item
@@ -112,222 +146,714 @@ __device__ __forceinline__ int group_of(const int *__restrict__ item_start, int 
     return lo;
 }
 
-constexpr int kTab64 = 1024;
-
-template <int C, int G>
-__global__ void __launch_bounds__(128) dense_f64_kernel(StageDims d, StageBufs b,
-                                                        const unsigned long long *__restrict__ segs,
-                                                        const double *__restrict__ bins,
-                                                        int tile_bins) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    double2 *tab = reinterpret_cast<double2 *>(smem);                       // [1024]
-    double *sbin = reinterpret_cast<double *>(smem + sizeof(double2) * kTab64);  // [tile][9]
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + sizeof(double2) * kTab64 +
-                                                 sizeof(double) * kBinDoubles * tile_bins);
-    __shared__ int s_item, s_walker[G], s_lo[G][kMaxModes], s_hi[G][kMaxModes];
-    __shared__ double red[2][4];
-    const int tid = threadIdx.x;
-    for (int k = tid; k < kTab64; k += blockDim.x) {
-        double sn, cs;
-        sincospi((double)k / (kTab64 / 2), &sn, &cs);
-        tab[k] = make_double2(cs, sn);
+// ------------------------------------------------------------------ FP64 evaluation
+// Bins [j0, j1) of one walker in FP64 from the staged rows in global memory: segments too
+// short for the expansions, and values outside them.
+__device__ __noinline__ double2 dense_direct(const StageDims &d, const StageBufs &b,
+                                             const unsigned long long *__restrict__ segs,
+                                             const double *__restrict__ bins, int w, int j0, int j1,
+                                             const int *slo, const int *shi) {
+    double dh = 0.0, hh = 0.0;
+    const int K = d.K;
+    for (int j = j0; j < j1; j++) {
+        const double f = bin_freq_d(d.f0, d.df, j);
+        double h[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        for (int mi = 0; mi < d.L; mi++) {
+            if (j < slo[mi] || j > shi[mi]) continue;
+            const size_t wm = (size_t)w * d.L + mi;
+            const int *kb = b.kb + wm * K;
+            int lo = 0, hi = K - 2;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (kb[mid] <= j)
+                    lo = mid;
+                else
+                    hi = mid - 1;
+            }
+            const unsigned long long *rec = segs + kPhaseWords * (wm * (K - 1) + lo);
+            const double *c = b.coef + (wm * (K - 1) + lo) * 32;
+            const double x = f - b.fk[wm * K + lo];
+            double sn, cs;
+            sincospi((double)(long long)phase64_at(rec, j - kb[lo]).ph * 0x1p-63, &sn, &cs);
+            const double amp = fma(x, fma(x, fma(x, c[3], c[2]), c[1]), c[0]);
+            const double zr = amp * cs, zi = amp * sn;
+            for (int ch = 0; ch < 3; ch++) {
+                const double *r = c + 8 + 8 * ch, *m = r + 4;
+                const double tr = fma(x, fma(x, fma(x, r[3], r[2]), r[1]), r[0]);
+                const double ti = fma(x, fma(x, fma(x, m[3], m[2]), m[1]), m[0]);
+                h[2 * ch] = fma(tr, zr, fma(-ti, zi, h[2 * ch]));
+                h[2 * ch + 1] = fma(tr, zi, fma(ti, zr, h[2 * ch + 1]));
+            }
+        }
+        const double *o = bins + (size_t)j * kBinDoubles;
+        for (int ch = 0; ch < 3; ch++) {
+            const double hr = h[2 * ch], hi = h[2 * ch + 1];
+            hh = fma(o[ch], fma(hr, hr, hi * hi), hh);
+            dh = fma(o[3 + 2 * ch], hr, fma(o[4 + 2 * ch], hi, dh));
+        }
     }
-    if (tid == 0) mbar_init(bar, 1);
+    return make_double2(dh, hh);
+}
+
+// ------------------------------------------------------------------ data rows
+// A double scaled by 2^-e as a pair of floats, hi truncated to 24 bits and lo the next 24
+// (|v| < 2^e; values below 2^-76 are dropped)
+__device__ __forceinline__ void split_double(double v, int e, float &hi, float &lo) {
+    const long long b = __double_as_longlong(v);
+    const int de = (int)((b >> 52) & 0x7ff) - 1022 - e;  // <= 0; v = m 2^(de - 53) 2^e
+    const unsigned int mh = (unsigned int)(b >> 29) & 0x7fffffu;
+    const unsigned int ml = (unsigned int)b & 0x1fffffffu;
+    const unsigned int sign = (unsigned int)(b >> 32) & 0x80000000u;
+    const bool keep = de > -76 && ((b >> 52) & 0x7ff) != 0;
+    hi = keep ? __uint_as_float(sign | (unsigned int)(126 + de) << 23 | mh) : 0.0f;
+    const float l = (float)ml * __uint_as_float((unsigned int)max(126 + 1 + de - 53, 0) << 23);
+    lo = keep ? __uint_as_float(__float_as_uint(l) | sign) : 0.0f;
+}
+
+// Rows of kFxRows bins of 9 doubles (w_A, w_E, w_T, (w d)_A re, im, ...) in the form the dense
+// kernel uses: per row 18 floats, (w hi, w lo) of the three channels, then (re hi, im hi, re
+// lo, im lo) of each w d, channel c scaled by 2^-ew[c] and 2^-ed[c], the largest exponents of
+// the rows; and the exponents.  Rows past the data become zero.
+struct FxRows {
+    float v[kFxRows][2 * kBinDoubles];
+    int ew[3], ed[3];
+    bool ok;  // false: a value is infinite, NaN or out of range
+};
+
+__device__ __forceinline__ FxRows split_rows(const double *__restrict__ row, int rows) {
+    FxRows f;
+    f.ok = true;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        f.ew[c] = f.ed[c] = -2000;
+#pragma unroll
+        for (int r = 0; r < kFxRows; r++) {
+            if (r >= rows) break;
+            const double *o = row + r * kBinDoubles;
+            f.ew[c] = max(f.ew[c], exponent_of(o[c]));
+            f.ed[c] = max(f.ed[c], max(exponent_of(o[3 + 2 * c]), exponent_of(o[4 + 2 * c])));
+        }
+        f.ok = f.ok && max(f.ew[c], f.ed[c]) < 1025 && (f.ew[c] > -900 || f.ew[c] == -2000) &&
+               (f.ed[c] > -900 || f.ed[c] == -2000);
+    }
+#pragma unroll
+    for (int r = 0; r < kFxRows; r++)
+#pragma unroll
+        for (int q = 0; q < kBinDoubles; q++) {
+            const int c = q < 3 ? q : (q - 3) >> 1, im = (q - 3) & 1;
+            float h = 0.0f, l = 0.0f;
+            if (f.ok && r < rows) split_double(row[r * kBinDoubles + q], q < 3 ? f.ew[c] : f.ed[c], h, l);
+            if (q < 3) {
+                f.v[r][2 * q] = h;
+                f.v[r][2 * q + 1] = l;
+            } else {
+                f.v[r][6 + 4 * c + im] = h;
+                f.v[r][6 + 4 * c + 2 + im] = l;
+            }
+        }
+    return f;
+}
+
+// exponents as six signed 16-bit numbers and the flag, in one 16-byte word
+__device__ __forceinline__ int4 pack_exponents(const FxRows &f) {
+    auto two = [](int a, int b) { return (a & 0xffff) | (int)((unsigned int)b << 16); };
+    return make_int4(two(f.ew[0], f.ew[1]), two(f.ew[2], f.ed[0]), two(f.ed[1], f.ed[2]), f.ok ? 1 : 0);
+}
+
+// One thread per kFxRows bins; 16-byte word u of rows c goes to ((c / 32) kFxWords + u) 32 + c % 32,
+// so that a warp whose threads take consecutive rows reads every word coalesced.
+__global__ void __launch_bounds__(128) prep_fx_kernel(const double *__restrict__ bins, int N,
+                                                      float4 *__restrict__ out) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = c * kFxRows;
+    if (c >= fx_chunks(N)) return;
+    const FxRows f = split_rows(bins + (size_t)j * kBinDoubles, min(max(N - j, 0), kFxRows));
+    const float *v = &f.v[0][0];
+    float4 *o = out + (size_t)(c >> 5) * kFxWords * 32 + (c & 31);
+#pragma unroll
+    for (int u = 0; u < kFxWords - 1; u++) o[u * 32] = make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+    const int4 e = pack_exponents(f);
+    o[(kFxWords - 1) * 32] = make_float4(__int_as_float(e.x), __int_as_float(e.y), __int_as_float(e.z),
+                                         __int_as_float(e.w));
+}
+
+cudaError_t launch_prep_fx(const double *bins, int N, float4 *out, cudaStream_t s) {
+    prep_fx_kernel<<<(fx_chunks(N) + 127) / 128, 128, 0, s>>>(bins, N, out);
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------ expansions
+// A cubic of a segment, in x from its knot, and its forward differences over one bin at x
+__device__ __forceinline__ void differences(const double2 *__restrict__ c2, int row, double x, double df,
+                                            double d[4]) {
+    const double2 lo = __ldg(c2 + 2 * row), hi = __ldg(c2 + 2 * row + 1);
+    const double t = 3.0 * hi.y, df2 = df * df;
+    const double p1 = fma(x, fma(x, t, hi.x + hi.x), lo.y) * df;
+    const double p2 = fma(x, t, hi.x) * df2, p3 = hi.y * (df2 * df);
+    d[0] = fma(x, fma(x, fma(x, hi.y, hi.x), lo.y), lo.x);
+    d[1] = p1 + p2 + p3;
+    d[2] = 2.0 * fma(3.0, p3, p2);
+    d[3] = 6.0 * p3;
+}
+
+// m with |v| < 2^m over 2^n1 bins, |v| <= |d0| + n |d1| + n^2/2 |d2| + n^3/6 |d3|; large enough
+// for the third difference to fit 32 bits
+__device__ __forceinline__ int bound_of(const double d[4], int n1) {
+    return max(max(exponent_of(d[0]), exponent_of(d[1]) + n1),
+               max(exponent_of(d[2]) + 2 * n1 - 1, exponent_of(d[3]) + max(3 * n1 - 2, 30))) +
+           2;
+}
+
+// series q of an expansion, left as the doubles of differences() and their bound, in fixed
+// point scaled by 2^s
+__device__ __forceinline__ void series_put(Expand *e, int q, const double d[4], int bound) {
+    e->vd[q][0] = __double_as_longlong(d[0]);
+    e->vd[q][1] = __double_as_longlong(d[1]);
+    e->d2[q] = __double_as_longlong(d[2]);
+    e->d3[q] = make_int2(__double2loint(d[3]), __double2hiint(d[3]));
+    e->l3[q] = (uint32_t)bound;
+}
+
+__device__ __forceinline__ void series_fix(Expand *e, int q, int s) {
+    uint32_t l2, l3;
+    e->vd[q][0] = to_fixed(__longlong_as_double(e->vd[q][0]), s);
+    e->vd[q][1] = to_fixed(__longlong_as_double(e->vd[q][1]), s);
+    e->d2[q] = to_fixed96(__longlong_as_double(e->d2[q]), s, l2);
+    e->d3[q] = make_int2((int)to_fixed96(__hiloint2double(e->d3[q].y, e->d3[q].x), s, l3), (int)l2);
+    e->l3[q] = l3;
+}
+
+struct Diff {
+    i64 v, d1, d2;
+    int d3;
+};
+
+// series q n >= 0 bins from its origin; c2 = n(n-1)/2, c3 = n(n-1)(n-2)/6
+__device__ __forceinline__ Diff series_at(const Expand *__restrict__ e, int q, uint32_t n, uint32_t c2,
+                                          uint32_t c3) {
+    const longlong2 a = *reinterpret_cast<const longlong2 *>(e->vd[q]);
+    const i64 d2 = e->d2[q];
+    const int2 t = e->d3[q];
+    Diff r;
+    i64 v = mad_u((uint32_t)a.y, n, a.x);
+    v = mad_u((uint32_t)d2, c2, v);
+    v = mad_s(t.x, (int)c3, v);
+    v += (i64)(__umulhi(c2, (uint32_t)t.y) + __umulhi(c3, e->l3[q]));
+    r.v = add_hi(v, (uint32_t)(a.y >> 32) * n + (uint32_t)(d2 >> 32) * c2);
+    i64 d1 = mad_u((uint32_t)d2, n, a.y);
+    d1 = mad_s(t.x, (int)c2, d1);
+    r.d1 = add_hi(d1, (uint32_t)(d2 >> 32) * n);
+    r.d2 = mad_s(t.x, (int)n, d2);
+    r.d3 = t.x;
+    return r;
+}
+
+// the phase n >= 0 bins from its origin
+__device__ __forceinline__ void phase_at(const Expand *__restrict__ e, uint32_t n, uint32_t c2, uint32_t c3,
+                                         i64 p[4]) {
+    const longlong2 a = *reinterpret_cast<const longlong2 *>(e->vd[kSer]);
+    const i64 d2 = e->d2[kSer], d3 = e->ph3;
+    i64 v = mad_u((uint32_t)a.y, n, a.x);
+    v = mad_u((uint32_t)d2, c2, v);
+    v = mad_u((uint32_t)d3, c3, v);
+    v += (i64)__umulhi(n, e->low[0]) + (i64)(__umulhi(c2, e->low[1]) + __umulhi(c3, e->low[2]));
+    p[0] = add_hi(v, (uint32_t)(a.y >> 32) * n + (uint32_t)(d2 >> 32) * c2 + (uint32_t)(d3 >> 32) * c3);
+    i64 d1 = mad_u((uint32_t)d2, n, a.y);
+    d1 = mad_u((uint32_t)d3, c2, d1);
+    p[1] = add_hi(d1, (uint32_t)(d2 >> 32) * n + (uint32_t)(d3 >> 32) * c2);
+    p[2] = add_hi(mad_u((uint32_t)d3, n, d2), (uint32_t)(d3 >> 32) * n);
+    p[3] = d3;
+}
+
+__device__ __forceinline__ void diff_next(Diff &r) {
+    r.v += r.d1;
+    r.d1 += r.d2;
+    r.d2 += r.d3;
+}
+
+// ------------------------------------------------------------------ integrand
+// x as two floats: x 2^-29 = a + b 2^-23 to 48 significant bits, |x| < 2^60
+__device__ __forceinline__ void fixed_pair(i64 x, float &a, float &b) {
+    const int hi = (int)(x >> 29);
+    a = __int2float_rn(hi);
+    const int rest = hi - __float2int_rn(a);  // |rest| <= 64
+    // (rest 2^29 + low 29 bits) 2^-6, below 2^30
+    const int r = (int)(((unsigned int)rest << 23) | (((unsigned int)x & 0x1fffffffu) >> 6));
+    b = __int2float_rn(r);
+}
+
+// q + e added to the pair sum + comp: the error of the sum is exact (two-sum)
+__device__ __forceinline__ void add_pair(float2 &sum, float2 &comp, float2 q, float2 e) {
+    const float2 t = add2(sum, q);
+    const float2 z = sub2(t, sum);
+    const float2 err = add2(sub2(sum, sub2(t, z)), sub2(q, z));
+    comp = add2(comp, add2(err, e));
+    sum = t;
+}
+
+// the two halves of a pair sum together, times 2^k
+__device__ __forceinline__ double scaled_sum(float2 sum, float2 comp, int k) {
+    const float t = sum.x + sum.y, z = t - sum.x;
+    const float err = (sum.x - (t - z)) + (sum.y - z);
+    const double v = (double)t + (double)(err + (comp.x + comp.y));
+    return abs(k) < 1000 ? v * __hiloint2double((1023 + k) << 20, 0) : ldexp(v, k);
+}
+
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// a thread's rows in shared memory, padded to an odd number of 16-byte units
+// G walkers per group; kRaw: data rows converted from the FP64 rows as they are used (callers
+// that bring their own rows) instead of read in the dense kernel's form.
+template <int G, bool kRaw>
+__global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, StageBufs b,
+                                                                const unsigned long long *__restrict__ segs,
+                                                                const double *__restrict__ bins,
+                                                                const float4 *__restrict__ rows,
+                                                                int tile_bins) {
+    constexpr int NS = G == 1 ? 1 : 2;  // walkers expanded together: their modes share a warp
+    extern __shared__ __align__(128) unsigned char smem[];
+    SmemF64 &sm = *reinterpret_cast<SmemF64 *>(smem);
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ int s_item, s_walker[G], s_wlo[G], s_whi[G], s_lo[G][kMaxModes], s_hi[G][kMaxModes];
+    __shared__ float s_g0[G][kMaxModes], s_g1[G][kMaxModes];
+    __shared__ int s_task[kWarps][kTasks];
+    __shared__ int s_first[kWarps][kMaxModes * NS];  // first expansion of a (walker, mode), its count
+    __shared__ double s_sum[kWarps][G][2];           // <d|h>, <h|h> of the item by each warp
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    WarpMem &wm_ = sm.w[warp];
+    Expand *ex = wm_.ex;
+    if (tid == 0) mbar_init(&bar, 1);
     __syncthreads();
     const int ng = n_groups(d.B, G);
     const int total = b.item_start[ng];
-    const int K = d.K;
-    uint32_t parity = 0;
+    const int K = d.K, L = d.L;
+    const float f0f = (float)d.f0, dff = (float)d.df;
+    bool staged = false;
     for (;;) {
         __syncthreads();
         if (tid == 0) s_item = atomicAdd(b.counter, 1);
         __syncthreads();
         const int item = s_item;
         if (item >= total) return;
+        if (!staged) {
+            // the phasor table by one bulk copy; every thread waits, and the block leaves
+            // together if the copy never completed
+            if (tid == 0) {
+                if (b.wait_test_polls == 0)
+                    tma_load_1d(sm.tab, b.fxtab, sizeof(sm.tab), &bar);
+                else
+                    mbar_expect_tx(&bar, sizeof(sm.tab));  // test of the give-up path: no copy is issued
+            }
+            const uint32_t polls = b.wait_test_polls ? b.wait_test_polls : kWaitPolls;
+            if (!__syncthreads_and(mbar_wait_bounded(&bar, 0, b.err, polls))) return;
+            staged = true;
+        }
         const int g = group_of(b.item_start, ng, item);
         const int J0 = b.grange[2 * g] + (item - b.item_start[g]) * tile_bins;
-        const int Jend = min(J0 + tile_bins, b.grange[2 * g + 1] + 1);
-        // whole groups of 4 rows (16-byte multiples) by one bulk copy, the last <= 3 rows
-        // by plain loads, so nothing past the end of the data is read
-        const int full = (Jend - J0) & ~3, tail = Jend - J0 - full;
-        if (tid == 0 && full > 0) {
-            const uint32_t bytes = (uint32_t)(full * kBinDoubles * sizeof(double));
-            fence_proxy_async();
-            if (b.wait_test_polls == 0)
-                tma_load_1d(sbin, bins + (size_t)J0 * kBinDoubles, bytes, bar);
-            else
-                mbar_expect_tx(bar, bytes);  // test of the give-up path: no copy is issued
-        }
-        if (tid < tail * kBinDoubles)
-            sbin[full * kBinDoubles + tid] = bins[((size_t)J0 + full) * kBinDoubles + tid];
+        const int Jitem = min(J0 + tile_bins, b.grange[2 * g + 1] + 1);
         if (tid < G) {
-            const int i = g * G + tid;
-            s_walker[tid] = i < d.B ? b.order[i] : -1;
+            const int i = g * G + tid, w = i < d.B ? b.order[i] : -1;
+            s_walker[tid] = w;
+            s_wlo[tid] = w < 0 ? 0 : b.wrange[2 * w];
+            s_whi[tid] = w < 0 ? -1 : b.wrange[2 * w + 1];
         }
         if (tid < G * kMaxModes) {
             const int k = tid / kMaxModes, mi = tid % kMaxModes;
             const int i = g * G + k;
             int lo = 1, hi = 0;
-            if (i < d.B && mi < d.L) {
+            float g0 = 0.0f, g1 = 0.0f;
+            if (i < d.B && mi < L) {
                 const int w = b.order[i];
-                const int *bd = b.band + ((size_t)w * d.L + mi) * 3;
+                const size_t wm = (size_t)w * L + mi;
+                const int *bd = b.band + wm * 3;
                 if (b.valid[w] && bd[0]) {
                     lo = bd[1];
                     hi = bd[2];
+                    const unsigned long long *r = segs + kPhaseWords * (wm * (K - 1)) + 7;
+                    g0 = __uint_as_float((unsigned int)(__ldg(r) >> 32));
+                    g1 = __uint_as_float((unsigned int)(__ldg(r + kPhaseWords) >> 32));
                 }
             }
             s_lo[k][mi] = lo;
             s_hi[k][mi] = hi;
+            s_g0[k][mi] = g0;
+            s_g1[k][mi] = g1;
+        }
+        if (lane < G) s_sum[warp][lane][0] = s_sum[warp][lane][1] = 0.0;
+        __syncthreads();
+
+        const int nblk = (Jitem - J0 + kBlk - 1) / kBlk;
+        for (int unit0 = warp; unit0 < nblk * (G / NS); unit0 += kWarps) {
+            const int Jw = J0 + (unit0 % nblk) * kBlk, kp = unit0 / nblk * NS;
+            const int Jend = min(Jw + kBlk, Jitem);
+            const int j0 = Jw + lane * kC;
+            {
+                // lanes 0 .. NS L - 1: the segments that a walker's mode has in the warp's bins
+                int s0 = 0, cnt = 0;
+                if (lane < NS * L) {
+                    const int k = kp + lane / L, mi = d.ord[lane % L];
+                    const int ja = max(Jw, s_lo[k][mi]), jb = min(Jend, s_hi[k][mi] + 1);
+                    if (ja < jb) {
+                        const int *kb = b.kb + ((size_t)s_walker[k] * L + mi) * K;
+                        s0 = segment_at(kb, K, ja, fmaf((float)ja, dff, f0f), s_g0[k][mi], s_g1[k][mi]);
+                        int s1 = s0;
+                        while (s1 < K - 2 && __ldg(kb + s1 + 1) < jb) s1++;
+                        cnt = s1 - s0 + 1;
+                    }
+                }
+                int upto = cnt;
+                for (int o = 1; o < kMaxModes * NS; o <<= 1) {
+                    const int u = __shfl_up_sync(0xffffffffu, upto, o);
+                    if (lane >= o) upto += u;
+                }
+                int have = 0;  // (walker, mode) units expanded so far
+                // scale of each channel's sums (units of 2^(E - 55)), of this walker and the next;
+                // and whether a walker's bins here go to the FP64 evaluation
+                int E[3] = {kNoScale, kNoScale, kNoScale}, En[3] = {kNoScale, kNoScale, kNoScale};
+                bool direct = false, directn = false;
+#pragma unroll 1
+                for (int sub = 0; sub < NS; sub++) {
+                    const int k = kp + sub, w = s_walker[k];
+                    if (s_whi[k] < Jw || s_wlo[k] >= Jend) {  // nothing of this walker here
+                        have = max(have, (sub + 1) * L);
+                        continue;
+                    }
+#pragma unroll
+                    for (int i = 0; i < kC; i++)
+#pragma unroll
+                        for (int q = 0; q < 6; q++) wm_.H[i][q][lane] = 0;
+#pragma unroll 1
+                    for (int pos = 0; pos < L; pos++) {
+                        const int unit = sub * L + pos, mi = d.ord[pos];
+                        if (direct) break;
+                        if (unit >= have) {
+                            // expand as many units from here on as fit
+                            const int base = __shfl_sync(0xffffffffu, upto - cnt, unit);
+                            const unsigned fit =
+                                __ballot_sync(0xffffffffu, lane >= unit && lane < NS * L && upto - base <= kTasks);
+                            if (!fit) {  // one mode alone has too many segments here
+                                direct = true;
+                                break;
+                            }
+                            have = unit + __popc(fit);
+                            const int tasks = __shfl_sync(0xffffffffu, upto, have - 1) - base;
+                            __syncwarp();
+                            if (lane >= unit && lane < have) {
+                                const int first = upto - cnt - base;
+                                for (int i = 0; i < cnt; i++) s_task[warp][first + i] = lane | (s0 + i) << 4;
+                                s_first[warp][lane] = first | cnt << 8;
+                            }
+                            __syncwarp();
+                            if (lane < tasks) {
+                                const int t = s_task[warp][lane], u = t & 15, seg = t >> 4;
+                                const size_t wm = (size_t)s_walker[kp + u / L] * L + d.ord[u % L];
+                                Expand *e = ex + lane;
+                                const int *kb = b.kb + wm * K;
+                                const int k0 = __ldg(kb + seg);
+                                const int k1 =
+                                    seg < K - 2 ? __ldg(kb + seg + 1) : s_hi[kp + u / L][d.ord[u % L]] + 1;
+                                const int org = max(Jw, k0 - (kC - 1)), nn = org - k0;
+                                e->org = org;
+                                e->kb = k0;
+                                e->next = k1;
+                                const unsigned long long *r = segs + kPhaseWords * (wm * (K - 1) + seg);
+                                const Phase64 p = phase64_at(r, nn);
+                                const i64 c2 = (i64)nn * (nn - 1) / 2;
+                                e->vd[kSer][0] = p.ph;
+                                e->vd[kSer][1] = p.d1;
+                                e->d2[kSer] = p.d2;
+                                e->ph3 = p.d3;
+                                e->low[0] = (uint32_t)((r[4] + (i64)nn * r[5] + c2 * r[6]) >> 32);
+                                e->low[1] = (uint32_t)((r[5] + (i64)nn * r[6]) >> 32);
+                                e->low[2] = (uint32_t)(r[6] >> 32);
+                            }
+                            __syncwarp();
+                            // every lane one (expansion, series) at a time: FP64 instructions cost a
+                            // full warp's time however few lanes take part
+                            for (int i = lane; i < tasks * kSer; i += 32) {
+                                Expand *e = ex + i / kSer;
+                                const int q = i % kSer;
+                                const int t = s_task[warp][i / kSer], u = t & 15, seg = t >> 4;
+                                const size_t wm = (size_t)s_walker[kp + u / L] * L + d.ord[u % L];
+                                const double x = bin_freq_d(d.f0, d.df, e->org) - __ldg(b.fk + wm * K + seg);
+                                const double2 *cf =
+                                    reinterpret_cast<const double2 *>(b.coef + (wm * (size_t)(K - 1) + seg) * 32);
+                                double dd[4];
+                                differences(cf, q == 0 ? 0 : q + 1, x, d.df, dd);  // series 1 is the phase
+                                const int n1 = 32 - __clz(max(min(e->next, Jw + kBlk) - e->org - 1, 15));
+                                series_put(e, q, dd, bound_of(dd, n1));
+                            }
+                            __syncwarp();
+                            int ea = -5000, et[3] = {-5000, -5000, -5000}, ts = 0;
+                            bool bad = false;
+                            if (lane < tasks) {
+                                const Expand *e = ex + lane;
+                                ts = (s_task[warp][lane] & 15) / L;
+                                ea = (int)e->l3[0];
+                                int top = ea;
+#pragma unroll
+                                for (int c = 0; c < 3; c++) {
+                                    et[c] = max((int)e->l3[1 + 2 * c], (int)e->l3[2 + 2 * c]);
+                                    top = max(top, et[c]);
+                                }
+                                // a short segment, or an infinite or NaN coefficient
+                                bad = e->next - e->kb < kMinSeg || top > 900;
+                            }
+                            const unsigned wrong = __ballot_sync(0xffffffffu, bad);
+                            const unsigned of_next = __ballot_sync(0xffffffffu, lane < tasks && ts > sub);
+                            directn = directn || (wrong & of_next);
+                            if (wrong & ~of_next) {
+                                direct = true;
+                                break;
+                            }
+                            int sc[3];
+#pragma unroll
+                            for (int c = 0; c < 3; c++) {
+                                const int v = ea + et[c];
+                                const int m = __reduce_max_sync(0xffffffffu, lane < tasks && ts == sub ? v : kNoScale);
+                                const int mn = __reduce_max_sync(0xffffffffu, lane < tasks && ts > sub ? v : kNoScale);
+                                if (m > E[c]) {
+                                    if (pos > 0 && E[c] > kNoScale)
+                                        for (int i = 0; i < kC; i++)
+                                            for (int q = 2 * c; q < 2 * c + 2; q++)
+                                                wm_.H[i][q][lane] >>= min(m - E[c], 63);
+                                    E[c] = m;
+                                }
+                                En[c] = max(En[c], mn);
+                                sc[c] = ts > sub ? En[c] : E[c];
+                            }
+                            if (lane < tasks) {  // the binary scale of every series
+                                Expand *e = ex + lane;
+                                e->l3[0] = (uint32_t)(kABits - ea);
+#pragma unroll
+                                for (int q = 1; q < kSer; q++)
+                                    e->l3[q] = (uint32_t)(kTBits - (sc[(q - 1) >> 1] - ea));
+                            }
+                            __syncwarp();
+                            for (int i = lane; i < tasks * kSer; i += 32)
+                                series_fix(ex + i / kSer, i % kSer, (int)ex[i / kSer].l3[i % kSer]);
+                            __syncwarp();
+                        }
+                        const int fc = s_first[warp][unit];
+                        const Expand *e = ex + (fc & 0xff), *eend = e + (fc >> 8);
+                        const int ja = max(j0, s_lo[k][mi]), jb = min(min(j0 + kC, Jend), s_hi[k][mi] + 1);
+                        if (ja >= jb) continue;
+                        while (e->next <= ja) e++;
+                        int from = ja;
+                        for (; from < jb && e < eend; e++) {  // usually one segment
+                            const int to = min(jb, e->next), ka = from - j0, kz = to - j0;
+                            if (ka >= kz) continue;  // a segment without bins
+                            from = to;
+                            const uint32_t n0 = j0 - e->org, c2 = n0 * (n0 - 1) / 2, c3 = c2 * (n0 - 2) / 3;
+                            i64 ph[4] = {0, 0, 0, 0};
+                            const bool same = d.same[pos] != 0;  // the phase of the mode before
+                            if (!same) phase_at(e, n0, c2, c3, ph);
+                            Diff s[kSer];
+#pragma unroll
+                            for (int q = 0; q < kSer; q++) s[q] = series_at(e, q, n0, c2, c3);
+#pragma unroll 1
+                            for (int i = 0; i < kC; i++) {
+                                if (i >= ka && i < kz) {
+                                    i64 pr, pi;
+                                    if (same) {
+                                        pr = wm_.z[i][0][lane];
+                                        pi = wm_.z[i][1][lane];
+                                    } else {
+                                        fx_rotate(ph[0], sm.tab[fx_cell(ph[0])], pr, pi);
+                                        wm_.z[i][0][lane] = pr;
+                                        wm_.z[i][1][lane] = pi;
+                                    }
+                                    const Bal a = bal(s[0].v);
+                                    const i64 ar = mulhi(a, bal(pr)), ai = mulhi(a, bal(pi));
+                                    const Bal zr = bal(ar), zi = bal(ai), zn = bal(-ai);  // A e^{i phase}
+#pragma unroll
+                                    for (int c = 0; c < 3; c++) {
+                                        const Bal r = bal(s[1 + 2 * c].v), m = bal(s[2 + 2 * c].v);
+                                        i64 h0 = wm_.H[i][2 * c][lane], h1 = wm_.H[i][2 * c + 1][lane];
+                                        i64 x0 = (i64)r.h * zr.l, x1 = (i64)r.h * zi.l;
+                                        x0 = mad_s(r.l, zr.h, x0);
+                                        x1 = mad_s(r.l, zi.h, x1);
+                                        x0 = mad_s(m.h, zn.l, x0);
+                                        x1 = mad_s(m.h, zr.l, x1);
+                                        x0 = mad_s(m.l, zn.h, x0);
+                                        x1 = mad_s(m.l, zr.h, x1);
+                                        h0 += x0 >> 32;
+                                        h1 += x1 >> 32;
+                                        h0 = mad_s(r.h, zr.h, h0);
+                                        h1 = mad_s(r.h, zi.h, h1);
+                                        h0 = mad_s(m.h, zn.h, h0);
+                                        h1 = mad_s(m.h, zr.h, h1);
+                                        wm_.H[i][2 * c][lane] = h0;
+                                        wm_.H[i][2 * c + 1][lane] = h1;
+                                    }
+                                }
+                                ph[0] += ph[1];
+                                ph[1] += ph[2];
+                                ph[2] += ph[3];
+#pragma unroll
+                                for (int q = 0; q < kSer; q++) diff_next(s[q]);
+                            }
+                        }
+                    }
+
+                    double dh = 0.0, hh = 0.0;
+                    const int mine = min(max(Jend - j0, 0), kC);  // this thread's rows
+                    bool here = !direct && mine > 0;
+                    float2 hs[3], hc[3], ds[3], dc[3];
+                    int ew[3] = {0, 0, 0}, ed[3] = {0, 0, 0};
+                    FxRows raw;
+                    const float4 *src = rows + (size_t)(j0 >> 7) * kFxWords * 32 + ((j0 >> 2) & 31);
+                    if (here) {
+                        if (kRaw) {
+                            raw = split_rows(bins + (size_t)j0 * kBinDoubles, mine);
+                            here = raw.ok;
+#pragma unroll
+                            for (int c = 0; c < 3; c++) {
+                                ew[c] = raw.ew[c];
+                                ed[c] = raw.ed[c];
+                            }
+                        } else {
+                            const int4 e4 = __ldg(reinterpret_cast<const int4 *>(src) + (kFxWords - 1) * 32);
+                            here = e4.w != 0;
+                            ew[0] = (e4.x << 16) >> 16;
+                            ew[1] = e4.x >> 16;
+                            ew[2] = (e4.y << 16) >> 16;
+                            ed[0] = e4.y >> 16;
+                            ed[1] = (e4.z << 16) >> 16;
+                            ed[2] = e4.z >> 16;
+                        }
+                    }
+                    if (here) {
+#pragma unroll
+                        for (int c = 0; c < 3; c++) hs[c] = hc[c] = ds[c] = dc[c] = make_float2(0.0f, 0.0f);
+#pragma unroll(kRaw ? 2 : 1)
+                        for (int i2 = 0; i2 < kC / 2; i2++) {
+                            // two rows: nine 16-byte words
+                            float o[4 * kBinDoubles];
+#pragma unroll
+                            for (int q = 0; q < kBinDoubles; q++) {
+                                if (kRaw) {
+#pragma unroll
+                                    for (int u = 0; u < 4; u++) o[4 * q + u] = (&raw.v[0][0])[36 * i2 + 4 * q + u];
+                                } else {
+                                    const float4 v = __ldg(src + (kBinDoubles * i2 + q) * 32);
+                                    o[4 * q] = v.x;
+                                    o[4 * q + 1] = v.y;
+                                    o[4 * q + 2] = v.z;
+                                    o[4 * q + 3] = v.w;
+                                }
+                            }
+#pragma unroll
+                            for (int ii = 0; ii < 2; ii++) {
+                                const float *q = o + 2 * kBinDoubles * ii;
+                                const int i = 2 * i2 + ii;
+#pragma unroll
+                                for (int c = 0; c < 3; c++) {
+                                    float2 x, y;  // h = x + y
+                                    fixed_pair(wm_.H[i][2 * c][lane], x.x, y.x);
+                                    fixed_pair(wm_.H[i][2 * c + 1][lane], x.y, y.y);
+                                    const float s23 = 1.1920928955078125e-7f;  // 2^-23
+                                    y = mul2(y, make_float2(s23, s23));
+                                    const float2 wh = make_float2(q[2 * c], q[2 * c]);
+                                    const float2 wl = make_float2(q[2 * c + 1], q[2 * c + 1]);
+                                    const float2 eh = make_float2(q[6 + 4 * c], q[7 + 4 * c]);
+                                    const float2 el = make_float2(q[8 + 4 * c], q[9 + 4 * c]);
+                                    // w |h|^2
+                                    const float2 p = mul2(x, x);
+                                    const float2 pe = fma2(add2(add2(x, x), y), y, fma2(x, x, neg2(p)));
+                                    const float2 u = mul2(wh, p);
+                                    float2 ue = fma2(wh, p, neg2(u));
+                                    ue = fma2(wl, p, ue);
+                                    add_pair(hs[c], hc[c], u, fma2(wh, pe, ue));
+                                    // Re((w d)* h)
+                                    const float2 v = mul2(eh, x);
+                                    float2 ve = fma2(eh, x, neg2(v));
+                                    ve = fma2(el, x, ve);
+                                    add_pair(ds[c], dc[c], v, fma2(eh, y, ve));
+                                }
+                            }
+                        }
+                        // h = (x + y) 2^(E - 26)
+#pragma unroll
+                        for (int c = 0; c < 3; c++) {
+                            if (E[c] == kNoScale) continue;
+                            hh += scaled_sum(hs[c], hc[c], ew[c] + 2 * (E[c] - 26));
+                            dh += scaled_sum(ds[c], dc[c], ed[c] + E[c] - 26);
+                        }
+                    } else if (mine > 0) {
+                        const double2 r = dense_direct(d, b, segs, bins, w, j0, j0 + mine, s_lo[k], s_hi[k]);
+                        dh = r.x;
+                        hh = r.y;
+                    }
+                    for (int o = 16; o > 0; o >>= 1) {
+                        dh += __shfl_down_sync(0xffffffffu, dh, o);
+                        hh += __shfl_down_sync(0xffffffffu, hh, o);
+                    }
+                    if (lane == 0) {
+                        s_sum[warp][k][0] += dh;
+                        s_sum[warp][k][1] += hh;
+                    }
+                    // after an early end the next walker's expansions are not in fixed point yet
+                    have = direct ? (sub + 1) * L : max(have, (sub + 1) * L);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        E[c] = direct ? kNoScale : En[c];
+                        En[c] = kNoScale;
+                    }
+                    direct = directn;
+                    directn = false;
+                }
+            }
         }
         __syncthreads();
-        if (full > 0) {
-            // every thread waits; the block leaves together if the copy never completed
-            const uint32_t polls = b.wait_test_polls ? b.wait_test_polls : kWaitPolls;
-            if (!__syncthreads_and(mbar_wait_bounded(bar, parity, b.err, polls))) return;
-            parity ^= 1u;
-        }
-
-        for (int k = 0; k < G; k++) {
-            const int w = s_walker[k];
-            if (w < 0) continue;
-            const size_t slot = (size_t)item * G + k;
-            if (b.wrange[2 * w + 1] < J0 || b.wrange[2 * w] >= Jend) {
-                if (tid == 0) {
-                    b.part[2 * slot] = 0.0;
-                    b.part[2 * slot + 1] = 0.0;
-                }
-                continue;
-            }
-            const int j0 = J0 + tid * C;
-            int seg[kMaxModes], knext[kMaxModes];
-            Phase64 ph[kMaxModes];
-#pragma unroll
-            for (int mi = 0; mi < kMaxModes; mi++) {
-                seg[mi] = 0;
-                knext[mi] = 0x7fffffff;
-                ph[mi] = Phase64{0, 0, 0, 0};
-                const int jj = max(j0, s_lo[k][mi]);
-                if (mi < d.L && jj <= s_hi[k][mi] && jj < min(j0 + C, Jend)) {
-                    const size_t wm = (size_t)w * d.L + mi;
-                    const int *kbm = b.kb + wm * K;
-                    const int s = segment_of(kbm, K, jj);
-                    seg[mi] = s;
-                    knext[mi] = (s < K - 2) ? __ldg(kbm + s + 1) : 0x7fffffff;
-                    ph[mi] = phase64_at(segs + kPhaseWords * (wm * (K - 1) + s), jj - __ldg(kbm + s));
-                }
-            }
-            double dh = 0.0, hh = 0.0;
-            for (int i = 0; i < C; i++) {
-                const int j = j0 + i;
-                if (j >= Jend) break;
-                const double f = bin_freq_d(d.f0, d.df, j);
-                double hr0 = 0.0, hi0 = 0.0, hr1 = 0.0, hi1 = 0.0, hr2 = 0.0, hi2 = 0.0;
-#pragma unroll
-                for (int mi = 0; mi < kMaxModes; mi++) {
-                    if (mi >= d.L || j < s_lo[k][mi] || j > s_hi[k][mi]) continue;
-                    const size_t wm = (size_t)w * d.L + mi;
-                    if (j >= knext[mi]) {  // into the next segment: new anchor
-                        const int *kbm = b.kb + wm * K;
-                        int s = seg[mi];
-                        while (s < K - 2 && j >= __ldg(kbm + s + 1)) s++;
-                        seg[mi] = s;
-                        knext[mi] = (s < K - 2) ? __ldg(kbm + s + 1) : 0x7fffffff;
-                        ph[mi] = phase64_at(segs + kPhaseWords * (wm * (K - 1) + s), j - __ldg(kbm + s));
-                    }
-                    const int s = seg[mi];
-                    const double x = f - __ldg(b.fk + wm * K + s);
-                    double v[kNSeries];
-                    eval_segment(b.coef + (wm * (K - 1) + s) * 32, x, v);
-                    double cs, sn;
-                    phasor64(ph[mi].ph, tab, cs, sn);
-                    ph[mi].ph += ph[mi].d1;
-                    ph[mi].d1 += ph[mi].d2;
-                    ph[mi].d2 += ph[mi].d3;
-                    const double zr = v[0] * cs, zi = v[0] * sn;
-                    hr0 = fma(v[2], zr, fma(-v[3], zi, hr0));
-                    hi0 = fma(v[2], zi, fma(v[3], zr, hi0));
-                    hr1 = fma(v[4], zr, fma(-v[5], zi, hr1));
-                    hi1 = fma(v[4], zi, fma(v[5], zr, hi1));
-                    hr2 = fma(v[6], zr, fma(-v[7], zi, hr2));
-                    hi2 = fma(v[6], zi, fma(v[7], zr, hi2));
-                }
-                const double *o = sbin + (size_t)(j - J0) * kBinDoubles;
-                hh = fma(o[0], fma(hr0, hr0, hi0 * hi0), hh);
-                hh = fma(o[1], fma(hr1, hr1, hi1 * hi1), hh);
-                hh = fma(o[2], fma(hr2, hr2, hi2 * hi2), hh);
-                dh = fma(o[3], hr0, fma(o[4], hi0, dh));
-                dh = fma(o[5], hr1, fma(o[6], hi1, dh));
-                dh = fma(o[7], hr2, fma(o[8], hi2, dh));
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                dh += __shfl_down_sync(0xffffffffu, dh, o);
-                hh += __shfl_down_sync(0xffffffffu, hh, o);
-            }
-            if ((tid & 31) == 0) {
-                red[0][tid >> 5] = dh;
-                red[1][tid >> 5] = hh;
-            }
-            __syncthreads();
-            if (tid == 0) {
-                double a = 0.0, c = 0.0;
-                for (int q = 0; q < (int)(blockDim.x >> 5); q++) {
-                    a += red[0][q];
-                    c += red[1][q];
-                }
-                b.part[2 * slot] = a;
-                b.part[2 * slot + 1] = c;
-            }
-            __syncthreads();
+        if (tid < 2 * G && s_walker[tid >> 1] >= 0) {
+            const int k = tid >> 1, q = tid & 1;
+            double t = 0.0;
+            for (int i = 0; i < kWarps; i++) t += s_sum[i][k][q];
+            b.part[2 * ((size_t)item * G + k) + q] = t;
         }
     }
 }
 
-template <int C>
-constexpr size_t f64_smem() {
-    return sizeof(double2) * kTab64 + sizeof(double) * kBinDoubles * 128 * C + 16;
+template <int G, bool kRaw>
+cudaError_t f64_attr() {
+    return cudaFuncSetAttribute(dense_f64_kernel<G, kRaw>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(SmemF64));
 }
 
-template <int C, int G>
+template <int G, bool kRaw>
 cudaError_t launch_f64(const StageDims &d, const StageBufs &b, const unsigned long long *segs,
-                       const double *bins, int blocks, cudaStream_t s) {
-    const int tile = 128 * C;
-    const size_t smem = f64_smem<C>();
-    cudaError_t e = cudaFuncSetAttribute(dense_f64_kernel<C, G>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                       const double *bins, const float4 *rows, const DenseTune &t, cudaStream_t s) {
+    cudaError_t e = f64_attr<G, kRaw>();
     if (e != cudaSuccess) return e;
-    dense_f64_kernel<C, G><<<blocks, 128, smem, s>>>(d, b, segs, bins, tile);
+    dense_f64_kernel<G, kRaw><<<t.blocks, 32 * kWarps, sizeof(SmemF64), s>>>(d, b, segs, bins, rows,
+                                                                             t.threads * t.per_thread);
     return cudaGetLastError();
 }
 
-template <int C, int G>
+template <int G, bool kRaw>
 int occ_f64() {
-    const size_t smem = f64_smem<C>();
-    if (cudaFuncSetAttribute(dense_f64_kernel<C, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
-        return 0;
+    if (f64_attr<G, kRaw>() != cudaSuccess) return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dense_f64_kernel<C, G>, 128, smem) !=
-        cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dense_f64_kernel<G, kRaw>, 32 * kWarps,
+                                                      sizeof(SmemF64)) != cudaSuccess)
         return 0;
     return n;
 }
 
+// Blocks per SM of a tile shape: tiles of 512 or 1024 bins, groups of 1 or 8 walkers.
 int dense_f64_occupancy(int per_thread, int group) {
-    if (per_thread == 8 && group == 8) return occ_f64<8, 8>();
-    if (per_thread == 8 && group == 1) return occ_f64<8, 1>();
-    if (per_thread == 4 && group == 8) return occ_f64<4, 8>();
-    if (per_thread == 4 && group == 1) return occ_f64<4, 1>();
-    return 0;
+    if ((per_thread != 4 && per_thread != 8) || (group != 1 && group != 8)) return 0;
+    return group == 8 ? occ_f64<8, false>() : occ_f64<1, false>();
 }
 
 cudaError_t launch_dense_f64(const StageDims &d, const StageBufs &b,
-                             const unsigned long long *segs, const double *bins,
+                             const unsigned long long *segs, const double *bins, const float4 *rows,
                              const DenseTune &t, cudaStream_t s) {
-    if (t.threads != 128) return cudaErrorInvalidValue;
-    if (t.per_thread == 8 && t.group == 8) return launch_f64<8, 8>(d, b, segs, bins, t.blocks, s);
-    if (t.per_thread == 8 && t.group == 1) return launch_f64<8, 1>(d, b, segs, bins, t.blocks, s);
-    if (t.per_thread == 4 && t.group == 8) return launch_f64<4, 8>(d, b, segs, bins, t.blocks, s);
-    if (t.per_thread == 4 && t.group == 1) return launch_f64<4, 1>(d, b, segs, bins, t.blocks, s);
+    if (t.threads != 128 || (t.per_thread != 4 && t.per_thread != 8)) return cudaErrorInvalidValue;
+    if (!rows) return t.group == 1 ? launch_f64<1, true>(d, b, segs, bins, rows, t, s) : cudaErrorInvalidValue;
+    if (t.group == 8) return launch_f64<8, false>(d, b, segs, bins, rows, t, s);
+    if (t.group == 1) return launch_f64<1, false>(d, b, segs, bins, rows, t, s);
     return cudaErrorInvalidValue;
 }
 

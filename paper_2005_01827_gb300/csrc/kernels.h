@@ -15,6 +15,15 @@ constexpr int kBinDoubles = 9;
 struct WalkerConst;  // response.cuh
 struct ModeConst;
 
+// The same rows in the form the FP64 dense kernel uses (dense.cu): kFxRows bins as kFxWords
+// 16-byte words, interleaved over 32 neighbours.
+constexpr int kFxRows = 4;
+constexpr int kFxWords = 19;
+__host__ __device__ inline int fx_chunks(int N) { return ((N + kFxRows - 1) / kFxRows + 31) & ~31; }
+
+struct FxTab;  // fixed.cuh
+constexpr size_t kFxTabBytes = 8192;
+
 struct StageDims {
     int B;       // walkers in this call
     int L;       // modes
@@ -22,7 +31,28 @@ struct StageDims {
     int N;       // dense bins
     double f0, df, t0;
     int ml[6], mm[6];  // (l, m) of each mode
+    // Modes with the same m share their band, knots and phase: phi_lm = (m/2) phi_22(2f/m) and
+    // a constant that depends on m alone for the six modes.  ord lists the modes with equal m
+    // next to each other; same[i]: ord[i] has the m of ord[i - 1].
+    int ord[6], same[6];
 };
+
+__host__ inline void order_modes(StageDims &d) {
+    int n = 0;
+    for (int i = 0; i < d.L; i++) {
+        bool first = true;
+        for (int j = 0; j < i; j++) first = first && d.mm[j] != d.mm[i];
+        if (!first) continue;
+        const int start = n;
+        for (int j = i; j < d.L; j++)
+            if (d.mm[j] == d.mm[i]) {
+                d.ord[n] = j;
+                d.same[n] = n > start ? 1 : 0;
+                n++;
+            }
+    }
+    for (; n < 6; n++) d.ord[n] = d.same[n] = 0;
+}
 
 // Per-call device buffers (sized for max_batch by the host).
 struct StageBufs {
@@ -46,11 +76,12 @@ struct StageBufs {
     int *grange;           // [groups][2] union range of each group (start a multiple of 4)
     int *item_start;       // [groups+1] exclusive prefix of the dense work items
     int *counter;          // dense work-queue counter
+    const FxTab *fxtab;    // phasor table of the FP64 dense kernel, written by the source kernel
     int *err;              // set by a device wait that gave up
     double *part;          // [items][G][2] per-item, per-slot partial sums
-    // Test only (0 in normal operation): when > 0 the dense kernels arm each tile's
-    // barrier for the tile's bytes but issue no copy, so every wait on it gives up after
-    // this many polls, with no copy in flight, and takes the error path.
+    // Test only (0 in normal operation): when > 0 the dense kernels arm the barrier of each
+    // staged copy for its bytes but issue no copy, so every wait on it gives up after this
+    // many polls, with no copy in flight, and takes the error path.
     unsigned wait_test_polls = 0;
 };
 
@@ -72,10 +103,10 @@ __host__ __device__ inline float *split_fac32(double *mscratch, size_t wm, int K
 }
 
 struct DenseTune {
-    int threads;     // threads per block
-    int per_thread;  // consecutive bins per thread
+    int threads;     // a tile is threads x per_thread bins
+    int per_thread;
     int blocks;      // persistent grid size
-    int group;       // walkers sharing one staged data tile
+    int group;       // walkers per work item
 };
 
 // groups of a call with B walkers
@@ -95,15 +126,20 @@ cudaError_t launch_plan(const StageDims &d, const StageBufs &b, int tile_bins, i
 // segment's first bin, as fractions of a turn scaled by 2^64 (words 0..3), and the next
 // 64 fractional bits of the three differences (words 4..6), which keep anchors deep
 // inside long segments exact to the FP64 value of the differences; the low 32 bits of
-// word 7 hold the first bin of the next segment (0x7fffffff for the last one).
+// word 7 hold the first bin of the next segment (0x7fffffff for the last one), and in the
+// FP64 path its high 32 bits hold the FP32 segment-guess constants: sc log2 f_lo in segment
+// 0, sc = (K - 1) / log2(f_hi / f_lo) in segment 1 (0 beyond).
 constexpr int kPhaseWords = 8;
 
 // FP64 path: the phase records of all segments ([B][L][K-1][kPhaseWords]).
 cudaError_t launch_phaseprep(const StageDims &d, const StageBufs &b, unsigned long long *phases,
                              cudaStream_t s);
+// rows: launch_prep_fx's, or NULL to convert them as they are used (group 1 only)
 cudaError_t launch_dense_f64(const StageDims &d, const StageBufs &b,
                              const unsigned long long *phases, const double *bins,
-                             const DenseTune &t, cudaStream_t s);
+                             const float4 *rows, const DenseTune &t, cudaStream_t s);
+// rows of the FP64 dense kernel from the staged data: fx_chunks(N) kFxWords float4
+cudaError_t launch_prep_fx(const double *bins, int N, float4 *out, cudaStream_t s);
 // split = 0: parts hold (<d|h>, <h|h>); split = 1: (sum |h|^2 - 2 Re(d h*), <h|h>)
 cudaError_t launch_finish(const StageDims &d, const StageBufs &b, int group, int split, double dd,
                           double *lnL, double *dh, double *hh, cudaStream_t s);

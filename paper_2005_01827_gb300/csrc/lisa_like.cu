@@ -48,6 +48,8 @@ struct lisa_like {
     double f0 = 0.0, df = 0.0, dd = 0.0;
     int N = 0;
     double *bins = nullptr;   // [N][9] FP64 staged data
+    float4 *rows = nullptr;   // the same in the FP64 dense kernel's form (FP64 precision)
+    FxTab *fxtab = nullptr;   // its phasor table
     float *bins32 = nullptr;  // [N][kBinFloats] FP32 whitened data (split precision)
     SegRec *segs = nullptr;   // [max_batch][L][K-1] split-precision segment records
     unsigned long long *phases = nullptr;  // [max_batch][L][K-1][8] FP64-path phase records
@@ -112,7 +114,7 @@ cudaError_t dalloc(T **p, size_t n) {
 
 void free_batch(lisa_like_t *h) {
     void *ptrs[] = {h->params, h->tc,    h->xpk,    h->fedge,  h->fk,  h->vals,  h->mscr,
-                    h->coef,   h->out,   h->wconst, h->mconst, h->valid,  h->band,   h->kb,         h->wrange,
+                    h->coef,   h->out,   h->wconst, h->mconst, h->fxtab, h->valid,  h->band,   h->kb,         h->wrange,
                     h->order,  h->slot_of, h->grange, h->item_start, h->counter, h->err_flag};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -125,6 +127,7 @@ void free_batch(lisa_like_t *h) {
     h->params = h->tc = h->fedge = h->fk = h->vals = h->mscr = h->coef = h->out = nullptr;
     h->wconst = nullptr;
     h->mconst = nullptr;
+    h->fxtab = nullptr;
     h->valid = h->band = h->kb = h->wrange = h->item_start = h->counter = nullptr;
     if (h->h_params) cudaFreeHost(h->h_params);
     if (h->h_out) cudaFreeHost(h->h_out);
@@ -159,8 +162,10 @@ lisa_status alloc_batch(lisa_like_t *h) {
     LCK(dalloc(&h->out, 3 * B), "device allocation (outputs)");
     if (h->precision == LISA_PREC_SPLIT)
         LCK(dalloc(&h->segs, B * L * (K - 1)), "device allocation (split segments)");
-    else
+    else {
         LCK(dalloc(&h->phases, B * L * (K - 1) * kPhaseWords), "device allocation (phase anchors)");
+        LCK(dalloc((unsigned char **)&h->fxtab, kFxTabBytes), "device allocation (phasor table)");
+    }
     LCK(cudaMallocHost(&h->h_params, sizeof(double) * B * kNPar), "pinned allocation");
     LCK(cudaMallocHost(&h->h_out, sizeof(double) * 3 * B), "pinned allocation");
     LCK(cudaMallocHost(&h->h_err, sizeof(int)), "pinned allocation");
@@ -178,6 +183,7 @@ StageBufs bufs_of(const lisa_like_t *h, const double *params) {
     b.wconst = h->wconst;
     b.mconst = h->mconst;
     b.fk = h->fk;
+    b.fxtab = h->fxtab;
     b.kb = h->kb;
     b.vals = h->vals;
     b.mscratch = h->mscr;
@@ -207,6 +213,7 @@ StageDims dims_of(const lisa_like_t *h, int B) {
         d.ml[i] = h->ml[i];
         d.mm[i] = h->mm[i];
     }
+    order_modes(d);
     return d;
 }
 
@@ -327,6 +334,7 @@ lisa_status enqueue(lisa_like_t *h, const double *dparams, int B, double *lnL, d
                 n++;
             }
         d.L = n;
+        order_modes(d);
     }
     const StageBufs b = bufs_of(h, dparams);
     const int tile = h->tune.threads * h->tune.per_thread;
@@ -346,7 +354,7 @@ lisa_status enqueue(lisa_like_t *h, const double *dparams, int B, double *lnL, d
     if (split)
         LCK(launch_dense_split(d, b, h->segs, h->bins32, h->tune, s), "dense kernel launch");
     else
-        LCK(launch_dense_f64(d, b, h->phases, h->bins, h->tune, s), "dense kernel launch");
+        LCK(launch_dense_f64(d, b, h->phases, h->bins, h->rows, h->tune, s), "dense kernel launch");
     LCK(mark(5), "cudaEventRecord");
     LCK(launch_finish(d, b, h->tune.group, split ? 1 : 0, h->dd, lnL, dh, hh, s),
         "finish kernel launch");
@@ -604,30 +612,33 @@ lisa_status lisa_like_set_data(lisa_like_t *h, double f0, double df, int64_t n_b
     const int64_t items = max_items(h->max_batch, N, h->min_tile);
     double *part = nullptr;
     float *bins32 = nullptr;
+    float4 *rows = nullptr;
+    const bool split = h->precision == LISA_PREC_SPLIT;
     if ((e = dalloc(&part, (size_t)items * 2)) != cudaSuccess ||
-        (h->precision == LISA_PREC_SPLIT &&
-         (e = dalloc(&bins32, (size_t)kBinFloats * N)) != cudaSuccess)) {
+        (split && (e = dalloc(&bins32, (size_t)kBinFloats * N)) != cudaSuccess) ||
+        (!split && (e = dalloc(&rows, (size_t)fx_chunks(N) * kFxWords)) != cudaSuccess)) {
         if (part) cudaFree(part);
         cudaFree(bins);
-        return cuda_fail(h, e, "device allocation (partial sums / FP32 data)");
+        return cuda_fail(h, e, "device allocation (partial sums / dense data)");
     }
-    if (bins32) {
-        if ((e = launch_prep_split(bins, N, bins32, s)) != cudaSuccess) {
-            cudaFree(part);
-            cudaFree(bins32);
-            cudaFree(bins);
-            return cuda_fail(h, e, "FP32 data preparation");
-        }
-        st = wait_for(h, s);
-        if (st != LISA_OK) {
-            h->deferred.push_back(part);
-            h->deferred.push_back(bins32);
-            h->deferred.push_back(bins);
-            return st;
-        }
+    if ((e = split ? launch_prep_split(bins, N, bins32, s) : launch_prep_fx(bins, N, rows, s)) != cudaSuccess) {
+        cudaFree(part);
+        if (bins32) cudaFree(bins32);
+        if (rows) cudaFree(rows);
+        cudaFree(bins);
+        return cuda_fail(h, e, "dense data preparation");
+    }
+    st = wait_for(h, s);
+    if (st != LISA_OK) {
+        h->deferred.push_back(part);
+        if (bins32) h->deferred.push_back(bins32);
+        if (rows) h->deferred.push_back(rows);
+        h->deferred.push_back(bins);
+        return st;
     }
     if (h->bins) cudaFree(h->bins);
     if (h->bins32) cudaFree(h->bins32);
+    if (h->rows) cudaFree(h->rows);
     if (h->part) cudaFree(h->part);
     if (h->rb) {  // summary data belong to the previous data
         lisa::rb_free(h->rb);
@@ -635,6 +646,7 @@ lisa_status lisa_like_set_data(lisa_like_t *h, double f0, double df, int64_t n_b
     }
     h->bins = bins;
     h->bins32 = bins32;
+    h->rows = rows;
     h->part = part;
     h->part_items = items;
     h->f0 = f0;
@@ -970,6 +982,7 @@ void lisa_like_destroy(lisa_like_t *h) {
     }
     if (h->bins) cudaFree(h->bins);
     if (h->bins32) cudaFree(h->bins32);
+    if (h->rows) cudaFree(h->rows);
     if (h->part) cudaFree(h->part);
     lisa::rb_free(h->rb);
     drop_graph(h);

@@ -44,7 +44,7 @@ void *g_addr[kMaxDevices] = {nullptr};
 size_t up256(size_t n) { return (n + 255) & ~(size_t)255; }
 
 struct Layout {
-    size_t valid, tc, xpk, band, fedge, wconst, mconst, fk, kb, vals, mscr, coef, phases, wrange, order, slot,
+    size_t fxtab, valid, tc, xpk, band, fedge, wconst, mconst, fk, kb, vals, mscr, coef, phases, wrange, order, slot,
         grange, items,
         counter, err, part, end;
 };
@@ -57,6 +57,7 @@ Layout layout_for(size_t B, size_t L, size_t K, size_t items) {
         p += up256(bytes);
         return at;
     };
+    o.fxtab = take(kFxTabBytes);
     o.valid = take(sizeof(int) * B);
     o.tc = take(sizeof(double) * B);
     o.xpk = take(sizeof(double) * B);
@@ -162,6 +163,7 @@ extern "C" lisa_status lisa_like_loglike_noalloc(const lisa_like_config *cfg, do
     unsigned char *s8 = static_cast<unsigned char *>(base);
     StageBufs b;
     b.params = d_params;
+    b.fxtab = reinterpret_cast<const FxTab *>(s8 + o.fxtab);
     b.valid = reinterpret_cast<int *>(s8 + o.valid);
     b.tc = reinterpret_cast<double *>(s8 + o.tc);
     b.xpk = reinterpret_cast<double *>(s8 + o.xpk);
@@ -195,6 +197,7 @@ extern "C" lisa_status lisa_like_loglike_noalloc(const lisa_like_config *cfg, do
         d.ml[i] = i < L ? cfg->modes[i][0] : 0;
         d.mm[i] = i < L ? cfg->modes[i][1] : 0;
     }
+    order_modes(d);
     const DenseTune tune = {kThreads, kPerThread, nsm * 2, kGroup};
     cudaStream_t s = (cudaStream_t)stream;
     // Every buffer is written before it is read within the call; the work counter and the
@@ -207,7 +210,7 @@ extern "C" lisa_status lisa_like_loglike_noalloc(const lisa_like_config *cfg, do
     unsigned long long *phases = reinterpret_cast<unsigned long long *>(s8 + o.phases);
     if ((e = launch_phaseprep(d, b, phases, s)) != cudaSuccess)
         return cuda_error(e, "segment kernel launch");
-    if ((e = launch_dense_f64(d, b, phases, d_bins, tune, s)) != cudaSuccess)
+    if ((e = launch_dense_f64(d, b, phases, d_bins, nullptr, tune, s)) != cudaSuccess)
         return cuda_error(e, "dense kernel launch");
     if ((e = launch_finish(d, b, tune.group, 0, dd, d_lnL, d_dh, d_hh, s)) != cudaSuccess)
         return cuda_error(e, "finish kernel launch");

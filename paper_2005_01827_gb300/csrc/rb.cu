@@ -356,6 +356,7 @@ StageDims dims_of(const LikeCore &c, int B) {
         d.ml[i] = c.ml[i];
         d.mm[i] = c.mm[i];
     }
+    order_modes(d);
     return d;
 }
 

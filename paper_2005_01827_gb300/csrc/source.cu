@@ -10,11 +10,14 @@
 // root, divisions), so their number is what counts: about 16 against 94 of two bisections
 // to 1e-14 in one thread.  Source and knots together, one walker, one mode, 256 knots: 281 ->
 // 98 us.
+#include "fixed.cuh"
 #include "kernels.h"
 #include "model.cuh"
 #include "response.cuh"
 
 namespace lisa {
+
+static_assert(sizeof(FxTab) * kFxTab == kFxTabBytes, "table size");
 
 // f_j = f0 + j df, rounded as a separate product and sum (no fused multiply-add) so
 // that band edges and knot-to-bin boundaries are decided exactly as written.
@@ -108,7 +111,17 @@ __device__ __forceinline__ void harmonics(const double v[3], double cb, double s
     o[4] = -0.5 * v[2] * sb;
 }
 
+// One block more than the walkers need writes the phasor table of the FP64 dense kernel.
 __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
+    if (blockIdx.x == gridDim.x - 1) {
+        FxTab *tab = const_cast<FxTab *>(b.fxtab);
+        for (int k = threadIdx.x; tab && k < kFxTab; k += blockDim.x) {
+            double sn, cs;
+            sincospi((double)k / (kFxTab / 2), &sn, &cs);
+            tab[k] = FxTab{bal(to_fixed(cs, 62)), bal(to_fixed(sn, 62))};
+        }
+        return;
+    }
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (w >= d.B) return;
     Source src;
@@ -231,7 +244,7 @@ __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
 }
 
 cudaError_t launch_source(const StageDims &d, const StageBufs &b, cudaStream_t s) {
-    source_kernel<<<(d.B + 3) / 4, 128, 0, s>>>(d, b);
+    source_kernel<<<(d.B + 3) / 4 + 1, 128, 0, s>>>(d, b);
     return cudaGetLastError();
 }
 

@@ -16,6 +16,7 @@
 // Packed FP32: each channel's (Re, Im) transfer pair is one Horner evaluation in
 // Blackwell's f32x2 FMA (one instruction for both lanes, each rounded as the scalar
 // FMA), and the per-bin integrand runs on (re, im) pairs the same way.
+#include "f32x2.cuh"
 #include "kernels.h"
 #include "model.cuh"
 #include "split.h"
@@ -152,18 +153,21 @@ __global__ void __launch_bounds__(256) segprep_kernel(StageDims d, StageBufs b, 
                 r.ph[7] = (unsigned int)((s < K - 2) ? kb[s + 1] : 0x7fffffff);
             }
         }
+        int guess0 = 0, guess1 = 0;
+        if (s <= 1) {  // the (walker, mode)'s segment-guess constants, read once per tile
+            const double f_lo = b.fedge[2 * wm], f_hi = b.fedge[2 * wm + 1];
+            const double scl = (double)(K - 1) / log2(f_hi / f_lo);
+            guess0 = __float_as_int((float)(log2(f_lo) * scl));
+            guess1 = __float_as_int((float)scl);
+        }
         if (kFull) {
             r.kb0 = kb0;
             r.invw = 1.0f / (float)W;
-            r.pad[0] = r.pad[1] = 0;
-            if (s == 0) {  // the (walker, mode)'s segment-guess constants, read once per tile
-                const double f_lo = b.fedge[2 * wm], f_hi = b.fedge[2 * wm + 1];
-                const double scl = (double)(K - 1) / log2(f_hi / f_lo);
-                r.pad[0] = __float_as_int((float)(log2(f_lo) * scl));
-                r.pad[1] = __float_as_int((float)scl);
-            }
+            r.pad[0] = s == 0 ? guess0 : 0;
+            r.pad[1] = s == 0 ? guess1 : 0;
             segs[g] = r;
         } else {
+            r.ph[7] |= (unsigned long long)(unsigned int)(s == 0 ? guess0 : guess1) << 32;
             ulonglong2 *o = reinterpret_cast<ulonglong2 *>(phases + (size_t)kPhaseWords * g);
             for (int q = 0; q < kPhaseWords / 2; q++)
                 o[q] = make_ulonglong2(r.ph[2 * q], r.ph[2 * q + 1]);
@@ -202,41 +206,6 @@ __device__ __forceinline__ int seg_guess(const int *__restrict__ kb, int K, int 
     while (s < K - 2 && __ldg(kb + s + 1) <= j) s++;
     return s;
 }
-
-// packed FP32 pairs (Blackwell f32x2): one instruction, each lane rounded as its scalar
-// counterpart
-#define LISA_F32X2(op, ...)                                                                  \
-    asm("{\n.reg .b64 ra, rb, rc, rd;\n"                                                      \
-        "mov.b64 ra, {%2, %3};\nmov.b64 rb, {%4, %5};\nmov.b64 rc, {%6, %7};\n" op         \
-        "\nmov.b64 {%0, %1}, rd;\n}"                                                          \
-        : "=f"(d.x), "=f"(d.y)                                                              \
-        : __VA_ARGS__)
-
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-    float2 d;
-    LISA_F32X2("fma.rn.f32x2 rd, ra, rb, rc;", "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x),
-               "f"(c.y));
-    return d;
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-    float2 d;
-    LISA_F32X2("mul.rn.f32x2 rd, ra, rb;", "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(0.0f),
-               "f"(0.0f));
-    return d;
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-    float2 d;
-    LISA_F32X2("add.rn.f32x2 rd, ra, rb;", "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(0.0f),
-               "f"(0.0f));
-    return d;
-}
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
-    float2 d;
-    LISA_F32X2("sub.rn.f32x2 rd, ra, rb;", "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(0.0f),
-               "f"(0.0f));
-    return d;
-}
-#undef LISA_F32X2
 
 // phase and forward differences at one bin as 32-bit fractions of a turn; the phase is
 // offset by half a table cell so that its top 8 bits name the nearest table entry
