@@ -16,6 +16,7 @@
 #include "internal.h"
 #include "kernels.h"
 #include "model.cuh"
+#include "response.cuh"
 
 namespace lisa {
 
@@ -26,10 +27,12 @@ constexpr int kRbTile = 256;  // grid bins per tile of the summary kernel
 struct RbState {
     int ne = 0, nb = 0, L = 0, P = 0;
     int *edges = nullptr;    // [ne] grid indices
-    double *fe = nullptr;    // [ne] edge frequencies
-    double *h0e = nullptr;   // [L][3][ne] complex: the fiducial's modes at the edges
-    double *A = nullptr;     // [2][L][3][nb] complex: A0, A1
-    double *Bs = nullptr;    // [2][P][3][nb] complex: B0, B1 for the mode pairs a <= a2
+    double *fe = nullptr;    // [3][ne] edge frequencies f, f^(1/3), f^(1/6)
+    double *h0e = nullptr;   // [L][3][ne] complex: 1 / the fiducial's modes at the edges (0 for 0)
+    // [L][3][nb] complex pairs: A0 and A1 / (width of the bin)
+    double *A = nullptr;
+    // [P][3][nb] complex pairs: B0 and B1 / width of the mode pairs a <= a2, twice that for a < a2
+    double *Bs = nullptr;
     double *fid = nullptr;   // [11] fiducial parameters
     double *flo = nullptr;   // [L] fiducial band edges
     double *fhi = nullptr;
@@ -82,7 +85,7 @@ __device__ inline void response(const Source &src, const Frame &fr, const Mode &
     }
 }
 
-// the fiducial's modes at the edges: one block per mode
+// the inverse of the fiducial's modes at the edges: one block per mode
 __global__ void rb_fid_kernel(RbDev r, const double *fid, double xpk, const double *flo,
                               const double *fhi, double *h0e) {
     const int a = blockIdx.x;
@@ -102,8 +105,10 @@ __global__ void rb_fid_kernel(RbDev r, const double *fid, double xpk, const doub
         cplx h[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
         if (f >= flo[a] && f <= fhi[a]) response(src, fr, md, kp, kc, f, h);
         for (int c = 0; c < 3; c++) {
-            h0e[2 * ((a * 3 + c) * r.ne + e)] = h[c].re;
-            h0e[2 * ((a * 3 + c) * r.ne + e) + 1] = h[c].im;
+            const double n = h[c].re * h[c].re + h[c].im * h[c].im;
+            const bool nz = h[c].re != 0.0 || h[c].im != 0.0;
+            h0e[2 * ((a * 3 + c) * r.ne + e)] = nz ? h[c].re / n : 0.0;
+            h0e[2 * ((a * 3 + c) * r.ne + e) + 1] = nz ? -h[c].im / n : 0.0;
         }
     }
 }
@@ -194,16 +199,17 @@ __global__ void __launch_bounds__(kRbThreads) rb_summary_kernel(RbDev r, const d
         }
         __syncthreads();
     }
+    if (q >= Q) return;
+    const double width = kind ? r.fe[b + 1] - r.fe[b] : 1.0, sc = a == a2 || q < 6 * L ? 1.0 : 2.0;
+    double *o;
     if (q < 6 * L) {
-        double *o = A + 2 * (((size_t)(kind * L + a) * 3 + c) * r.nb + b);
-        o[0] = accr;
-        o[1] = acci;
-    } else if (q < Q) {
+        o = A + 4 * (((size_t)a * 3 + c) * r.nb + b) + 2 * kind;
+    } else {
         const int p = ((q - 6 * L) % (3 * r.P)) / 3;
-        double *o = Bs + 2 * (((size_t)(kind * r.P + p) * 3 + c) * r.nb + b);
-        o[0] = accr;
-        o[1] = acci;
+        o = Bs + 4 * (((size_t)p * 3 + c) * r.nb + b) + 2 * kind;
     }
+    o[0] = sc * accr / width;
+    o[1] = sc * acci / width;
 }
 
 __device__ inline double block_sum(double v, double *red) {
@@ -217,17 +223,24 @@ __device__ inline double block_sum(double v, double *red) {
     return s;
 }
 
-// ln L of one walker per block
-__global__ void __launch_bounds__(kRbThreads) rb_walker_kernel(RbDev r, StageDims d, StageBufs b,
-                                                               double *lnL, double *dh, double *hh) {
+// ln L of one walker per block.  Bound by the FP64 pipe (2 lanes per clock and SM; 84 % busy
+// before the operations were cut), so what counts is the number of FP64 operations, and shared
+// memory and the loads of the summary data cost nothing beside them: the modes of equal m share
+// the response but for their polarisation weights (response.cuh), powers of the edge frequencies
+// are tabulated, divisions by the fiducial and by the bin widths are in the stored
+// data, each ratio is formed once, and the pairs of a mode are summed before its ratio
+// multiplies them (12 operations a pair).  1024 walkers, 128 bins, six modes: 3.67 -> 1.7 ms.
+__global__ void __launch_bounds__(kRbThreads, 2) rb_walker_kernel(RbDev r, StageDims d, StageBufs b,
+                                                                  double *lnL, double *dh,
+                                                                  double *hh) {
     extern __shared__ double sm[];
     const int w = blockIdx.x, L = r.L, ne = r.ne, nb = r.nb;
-    double *rr = sm;                                               // [L][3][ne] complex
-    unsigned char *ok = reinterpret_cast<unsigned char *>(rr + (size_t)L * 3 * ne * 2);  // [L][3][ne]
-    __shared__ Source src;
-    __shared__ Frame fr;
-    __shared__ cplx kp[6], kc[6];
+    cplx *rr = reinterpret_cast<cplx *>(sm);                                  // [L][3][ne]
+    unsigned char *ok = reinterpret_cast<unsigned char *>(rr + (size_t)L * 3 * ne);  // [L][3][ne]
+    __shared__ WalkerConst wc;
+    __shared__ ModeConst mc[kMaxModes];
     __shared__ double red[32];
+    __shared__ int first[kMaxModes], ngroup;
     if (!b.valid[w]) {
         if (threadIdx.x == 0) {
             lnL[w] = -INFINITY;
@@ -236,81 +249,94 @@ __global__ void __launch_bounds__(kRbThreads) rb_walker_kernel(RbDev r, StageDim
         }
         return;
     }
+    const double *src = reinterpret_cast<const double *>(b.wconst + w);
+    for (int i = threadIdx.x; i < (int)(sizeof(WalkerConst) / 8); i += blockDim.x)
+        reinterpret_cast<double *>(&wc)[i] = src[i];
+    if (threadIdx.x < L) {
+        const int a = threadIdx.x;
+        if (b.band[((size_t)w * L + a) * 3]) {
+            ModeConst m = b.mconst[(size_t)w * L + a];
+            m.v0 = cbrt(kPi * m.xf);  // for f^(1/3) of the edge itself
+            m.x160 = sqrt(m.v0 * kInvCbrtPi);
+            mc[a] = m;
+        }
+    }
     if (threadIdx.x == 0) {
-        make_source_core(b.params + (size_t)w * kNPar, d.t0, src);
-        set_peak(src, b.xpk[w]);
-        make_frame(src, fr);
+        int n = 0;
+        for (int i = 0; i < L; i++)
+            if (!d.same[i]) first[n++] = i;
+        ngroup = n;
     }
     __syncthreads();
-    if (threadIdx.x < L) pol_weights(src, Mode{r.ml[threadIdx.x], r.mm[threadIdx.x]}, kp[threadIdx.x], kc[threadIdx.x]);
-    __syncthreads();
-    for (int i = threadIdx.x; i < L * ne; i += blockDim.x) {
-        const int a = i / ne, e = i % ne;
-        const int *bd = b.band + ((size_t)w * L + a) * 3;
-        const double flo = b.fedge[((size_t)w * L + a) * 2], fhi = b.fedge[((size_t)w * L + a) * 2 + 1];
+    // r = h / h0 at the edges
+    for (int i = threadIdx.x; i < ngroup * ne; i += blockDim.x) {
+        const int i0 = first[i / ne], e = i % ne, a0 = d.ord[i0];
+        const size_t wm = (size_t)w * L + a0;
         const double f = r.fe[e];
-        cplx h[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
-        if (bd[0] && f >= flo && f <= fhi) response(src, fr, Mode{r.ml[a], r.mm[a]}, kp[a], kc[a], f, h);
-        for (int c = 0; c < 3; c++) {
-            const double *g = r.h0e + 2 * ((size_t)(a * 3 + c) * ne + e);
-            const bool nz = g[0] != 0.0 || g[1] != 0.0;
-            double qr = 0.0, qi = 0.0;
-            if (nz) {  // h / h0
-                const double den = g[0] * g[0] + g[1] * g[1];
-                qr = (h[c].re * g[0] + h[c].im * g[1]) / den;
-                qi = (h[c].im * g[0] - h[c].re * g[1]) / den;
+        const bool in = b.band[wm * 3] && f >= b.fedge[wm * 2] && f <= b.fedge[wm * 2 + 1];
+        ModeBase base;
+        double sn = 0.0, cs = 0.0;
+        if (in) {
+            mode_base(wc, mc[a0], f, mc[a0].v0 * r.fe[ne + e], mc[a0].x160 * r.fe[2 * ne + e], base);
+            sincos(base.phase - 2.0 * kPi * f * wc.tc, &sn, &cs);
+        }
+        for (int q = i0; q < L && (q == i0 || d.same[q]); q++) {
+            const int a = d.ord[q];
+            cplx T[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
+            cplx z = {0.0, 0.0};
+            if (in) {
+                double amp;
+                mode_channels(base, mc[a], amp, T);
+                z = {amp * cs, amp * sn};
             }
-            rr[2 * ((size_t)(a * 3 + c) * ne + e)] = qr;
-            rr[2 * ((size_t)(a * 3 + c) * ne + e) + 1] = qi;
-            ok[(a * 3 + c) * ne + e] = nz ? 1 : 0;
+            for (int c = 0; c < 3; c++) {
+                const double2 g = reinterpret_cast<const double2 *>(r.h0e)[(size_t)(a * 3 + c) * ne + e];
+                rr[(a * 3 + c) * ne + e] = cmul(cmul(T[c], z), cplx{g.x, g.y});
+                ok[(a * 3 + c) * ne + e] = g.x != 0.0 || g.y != 0.0 ? 1 : 0;
+            }
         }
     }
     __syncthreads();
-    // r0, r1 of (mode a, channel c, bin k) by the edge rule
-    auto ratios = [&](int a, int c, int k, double &r0r, double &r0i, double &r1r, double &r1i) {
-        const int base = (a * 3 + c) * ne;
-        const bool okL = ok[base + k], okR = ok[base + k + 1];
-        const double *pL = rr + 2 * ((size_t)base + k), *pR = pL + 2;
-        r1r = r1i = 0.0;
-        if (okL) {
-            r0r = pL[0];
-            r0i = pL[1];
-            if (okR) {
-                const double inv = 1.0 / (r.fe[k + 1] - r.fe[k]);
-                r1r = (pR[0] - pL[0]) * inv;
-                r1i = (pR[1] - pL[1]) * inv;
-            }
-        } else if (okR) {
-            r0r = pR[0];
-            r0i = pR[1];
-        } else {
-            r0r = r0i = 0.0;
-        }
-    };
+    // r0 and r1 times the bin's width of every (mode, channel, bin) by the edge rule
     double sdh = 0.0, shh = 0.0;
-    for (int i = threadIdx.x; i < L * 3 * nb; i += blockDim.x) {
-        const int a = i / (3 * nb), c = (i / nb) % 3, k = i % nb;
-        double r0r, r0i, r1r, r1i;
-        ratios(a, c, k, r0r, r0i, r1r, r1i);
-        const double *A0 = r.A + 2 * (((size_t)a * 3 + c) * nb + k);
-        const double *A1 = r.A + 2 * (((size_t)(L + a) * 3 + c) * nb + k);
-        sdh += A0[0] * r0r + A0[1] * r0i + A1[0] * r1r + A1[1] * r1i;  // Re(A conj(r))
-    }
-    for (int i = threadIdx.x; i < r.P * 3 * nb; i += blockDim.x) {
-        const int p = i / (3 * nb), c = (i / nb) % 3, k = i % nb;
-        int a, a2;
-        pair_of(p, L, a, a2);
-        double x0r, x0i, x1r, x1i, y0r, y0i, y1r, y1i;
-        ratios(a, c, k, x0r, x0i, x1r, x1i);
-        ratios(a2, c, k, y0r, y0i, y1r, y1i);
-        const double *B0 = r.Bs + 2 * (((size_t)p * 3 + c) * nb + k);
-        const double *B1 = r.Bs + 2 * (((size_t)(r.P + p) * 3 + c) * nb + k);
-        // Re(B0 x0 conj(y0) + B1 (x0 conj(y1) + x1 conj(y0)))
-        const double u0r = x0r * y0r + x0i * y0i, u0i = x0i * y0r - x0r * y0i;
-        const double u1r = x0r * y1r + x0i * y1i + x1r * y0r + x1i * y0i;
-        const double u1i = x0i * y1r - x0r * y1i + x1i * y0r - x1r * y0i;
-        const double t = B0[0] * u0r - B0[1] * u0i + B1[0] * u1r - B1[1] * u1i;
-        shh += (a == a2) ? t : 2.0 * t;
+    for (int i = threadIdx.x; i < 3 * nb; i += blockDim.x) {
+        const int c = i / nb, k = i % nb;
+        cplx x0[kMaxModes], x1[kMaxModes];
+#pragma unroll
+        for (int a = 0; a < kMaxModes; a++) {
+            x0[a] = x1[a] = {0.0, 0.0};
+            if (a >= L) continue;
+            const int at = (a * 3 + c) * ne + k;
+            const bool okL = ok[at], okR = ok[at + 1];
+            const cplx pL = rr[at], pR = rr[at + 1];
+            if (okL)
+                x0[a] = pL;
+            else if (okR)
+                x0[a] = pR;
+            if (okL && okR) x1[a] = csub(pR, pL);
+            const double2 *A = reinterpret_cast<const double2 *>(r.A) + 2 * (((size_t)a * 3 + c) * nb + k);
+            const double2 A0 = __ldg(A), A1 = __ldg(A + 1);
+            sdh += A0.x * x0[a].re + A0.y * x0[a].im + A1.x * x1[a].re + A1.y * x1[a].im;  // Re(A conj(r))
+        }
+        // Re(B0 x0 conj(y0) + B1 (x0 conj(y1) + x1 conj(y0))) over the pairs (x, y)
+        const double2 *B = reinterpret_cast<const double2 *>(r.Bs) + 2 * ((size_t)c * nb + k);
+#pragma unroll
+        for (int a = 0; a < kMaxModes; a++) {
+            if (a >= L) continue;
+            cplx z0 = {0.0, 0.0}, z1 = {0.0, 0.0};  // sums of B0 conj(y0) + B1 conj(y1), B1 conj(y0)
+#pragma unroll
+            for (int a2 = a; a2 < kMaxModes; a2++) {
+                if (a2 >= L) continue;
+                const double2 B0 = __ldg(B), B1 = __ldg(B + 1);
+                B += (size_t)6 * nb;
+                const cplx y0 = x0[a2], y1 = x1[a2];
+                z0.re += B0.x * y0.re + B0.y * y0.im + B1.x * y1.re + B1.y * y1.im;
+                z0.im += B0.y * y0.re - B0.x * y0.im + B1.y * y1.re - B1.x * y1.im;
+                z1.re += B1.x * y0.re + B1.y * y0.im;
+                z1.im += B1.y * y0.re - B1.x * y0.im;
+            }
+            shh += x0[a].re * z0.re - x0[a].im * z0.im + x1[a].re * z1.re - x1[a].im * z1.im;
+        }
     }
     const double tdh = block_sum(sdh, red);
     const double thh = block_sum(shh, red);
@@ -446,8 +472,13 @@ lisa_status lisa_like_set_fiducial(lisa_like_t *h, const double *params, int n_r
     r->L = c.L;
     r->P = c.L * (c.L + 1) / 2;
     r->xpk = xpk;
-    std::vector<double> fe(r->ne);
-    for (int i = 0; i < r->ne; i++) fe[i] = c.f0 + (double)ed[i] * c.df;
+    std::vector<double> fe(3 * r->ne);
+    for (int i = 0; i < r->ne; i++) {
+        const double f = c.f0 + (double)ed[i] * c.df;
+        fe[i] = f;
+        fe[r->ne + i] = std::cbrt(f);
+        fe[2 * r->ne + i] = std::sqrt(std::cbrt(f));
+    }
     std::vector<double> flo(c.L), fhi(c.L);
     for (int a = 0; a < c.L; a++) {
         flo[a] = band[3 * a] ? fedge[2 * a] : 1.0;   // inactive: an empty interval
@@ -455,7 +486,7 @@ lisa_status lisa_like_set_fiducial(lisa_like_t *h, const double *params, int n_r
     }
     const size_t nA = (size_t)2 * r->L * 3 * r->nb * 2, nB = (size_t)2 * r->P * 3 * r->nb * 2;
     if ((e = cudaMalloc(&r->edges, sizeof(int) * r->ne)) != cudaSuccess ||
-        (e = cudaMalloc(&r->fe, sizeof(double) * r->ne)) != cudaSuccess ||
+        (e = cudaMalloc(&r->fe, sizeof(double) * 3 * r->ne)) != cudaSuccess ||
         (e = cudaMalloc(&r->h0e, sizeof(double) * r->L * 3 * r->ne * 2)) != cudaSuccess ||
         (e = cudaMalloc(&r->A, sizeof(double) * nA)) != cudaSuccess ||
         (e = cudaMalloc(&r->Bs, sizeof(double) * nB)) != cudaSuccess ||
@@ -467,7 +498,7 @@ lisa_status lisa_like_set_fiducial(lisa_like_t *h, const double *params, int n_r
                          std::string("relative-binning allocation: ") + cudaGetErrorString(e));
     }
     e = cudaMemcpy(r->edges, ed.data(), sizeof(int) * r->ne, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(r->fe, fe.data(), sizeof(double) * r->ne, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(r->fe, fe.data(), sizeof(double) * 3 * r->ne, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(r->fid, params, sizeof(double) * kNPar, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(r->flo, flo.data(), sizeof(double) * c.L, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(r->fhi, fhi.data(), sizeof(double) * c.L, cudaMemcpyHostToDevice);

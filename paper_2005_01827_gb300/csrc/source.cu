@@ -249,26 +249,29 @@ cudaError_t launch_source(const StageDims &d, const StageBufs &b, cudaStream_t s
 }
 
 // ---------------------------------------------------------------------------- knots
-// One thread per knot, 128 knots of one (walker, mode) per block: log-spaced frequencies
+// One thread per knot of the modes of one m, 128 knots per block: log-spaced frequencies
 // (Sec. II.A: ~2^10 points) with A, phase + delay, and T, and the first dense bin at or
 // above each.  kSplit: the same FP64 values, A (times 2^64) and T stored as FP32 (the
 // split-precision layout).
 //
 // Bound by the FP64 pipe (2 lanes per clock per SM), so the count of FP64 operations per
-// knot is what matters (about 420 against 730): the powers of f come from one
+// knot is what matters (about 330 an m and 85 a mode, against 730 a mode): the powers of f come from one
 // exponential of the log-spaced step (f^(1/6) and its powers, no cube root or square root),
-// one division serves v, the amplitude and the three arms, and the response is in orbital
-// harmonics (response.cuh).  6144 systems of 1024 knots: 8.4 -> 5.4 ms with the
-// source kernel.  One block of 128 threads per system left all but a few SMs idle in small
+// one division serves v, the amplitude and the three arms, the response is in orbital
+// harmonics, and the modes of equal m share all of it but their polarisation weights
+// (response.cuh).  1024 walkers, six modes of 1024 knots: 8.4 -> 4.1 ms with the source kernel
+// (5.4 with one mode per thread).  One block of 128 threads per system left all but a few SMs idle in small
 // calls (6 systems of 1024 knots: 246 us), hence one knot per thread.
 template <bool kSplit>
 __global__ void __launch_bounds__(128) knot_kernel(StageDims d, StageBufs b) {
-    const size_t wm = blockIdx.x;
+    const int w = blockIdx.x / d.L, first = blockIdx.x % d.L;
+    if (d.same[first]) return;  // done with the first mode of its m
+    const size_t wm = (size_t)w * d.L + d.ord[first];
     if (!b.band[wm * 3]) return;  // inactive modes (and invalid walkers) have no knots
     __shared__ WalkerConst wc;
     __shared__ ModeConst mc;
     {
-        const double *src = reinterpret_cast<const double *>(b.wconst + wm / d.L);
+        const double *src = reinterpret_cast<const double *>(b.wconst + w);
         double *dst = reinterpret_cast<double *>(&wc);
         if (threadIdx.x < sizeof(WalkerConst) / 8) dst[threadIdx.x] = src[threadIdx.x];
         const double *msrc = reinterpret_cast<const double *>(b.mconst + wm);
@@ -282,31 +285,36 @@ __global__ void __launch_bounds__(128) knot_kernel(StageDims d, StageBufs b) {
     const double flo = b.fedge[wm * 2], fhi = b.fedge[wm * 2 + 1];
     const double e6 = exp(mc.s6 * (double)k), e3 = e6 * e6;
     const double f = (k == K - 1) ? fhi : flo * (e3 * e3 * e3);
-    b.fk[wm * K + k] = f;
     // first dense bin at or above this knot: a guess, then exact by the bin frequencies
     // themselves
     const double g = ceil((f - d.f0) / d.df);
     int j = g <= 0.0 ? 0 : (g >= (double)d.N ? d.N : (int)g);
     while (j > 0 && bin_freq(d.f0, d.df, j - 1) >= f) j--;
     while (j < d.N && bin_freq(d.f0, d.df, j) < f) j++;
-    b.kb[wm * K + k] = j;
-    double amp, ph;
-    cplx T[3];
-    mode_response(wc, mc, f, mc.v0 * e3, mc.x160 * e6, amp, ph, T);
-    double *vm = b.vals + wm * kNSeries * (size_t)K;
-    vm[1 * K + k] = ph;
-    if (kSplit) {
-        float *v32 = split_vals32(b.vals, wm, K);
-        v32[k] = (float)(amp * kAmpScale64);
-        for (int c = 0; c < 3; c++) {
-            v32[(1 + 2 * c) * K + k] = (float)T[c].re;
-            v32[(2 + 2 * c) * K + k] = (float)T[c].im;
-        }
-    } else {
-        vm[0 * K + k] = amp;
-        for (int c = 0; c < 3; c++) {
-            vm[(2 + 2 * c) * K + k] = T[c].re;
-            vm[(3 + 2 * c) * K + k] = T[c].im;
+    ModeBase base;
+    mode_base(wc, mc, f, mc.v0 * e3, mc.x160 * e6, base);
+    for (int i = first; i < d.L && (i == first || d.same[i]); i++) {
+        const size_t m = (size_t)w * d.L + d.ord[i];
+        double amp;
+        cplx T[3];
+        mode_channels(base, i == first ? mc : b.mconst[m], amp, T);
+        b.fk[m * K + k] = f;
+        b.kb[m * K + k] = j;
+        double *vm = b.vals + m * kNSeries * (size_t)K;
+        vm[1 * K + k] = base.phase;
+        if (kSplit) {
+            float *v32 = split_vals32(b.vals, m, K);
+            v32[k] = (float)(amp * kAmpScale64);
+            for (int c = 0; c < 3; c++) {
+                v32[(1 + 2 * c) * K + k] = (float)T[c].re;
+                v32[(2 + 2 * c) * K + k] = (float)T[c].im;
+            }
+        } else {
+            vm[0 * K + k] = amp;
+            for (int c = 0; c < 3; c++) {
+                vm[(2 + 2 * c) * K + k] = T[c].re;
+                vm[(3 + 2 * c) * K + k] = T[c].im;
+            }
         }
     }
 }
