@@ -345,7 +345,7 @@ lisa_status enqueue(lisa_like_t *h, const double *dparams, int B, double *lnL, d
     LCK(split ? launch_spline_split(d, b, s) : launch_spline(d, b, s), "spline kernel launch");
     LCK(mark(2), "cudaEventRecord");
     if (split)
-        LCK(launch_segprep(d, b, h->segs, s), "segment kernel launch");
+        LCK(launch_segprep(d, b, h->segs, h->tune.per_thread, s), "segment kernel launch");
     else
         LCK(launch_phaseprep(d, b, h->phases, s), "segment kernel launch");
     LCK(mark(3), "cudaEventRecord");
