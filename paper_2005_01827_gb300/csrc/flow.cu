@@ -2,16 +2,25 @@
 // directions, training (forward, back-propagation, Adam) and the independence
 // Metropolis-Hastings step of the sampler (Eq. (13)).
 //
-// Every network layer is a GEMM on the tensor cores: bfloat16 operands staged in shared
-// memory, FP32 accumulation, mma.sync.m16n8k16.  A block holds 64 samples; each of its
-// four warps owns 16 of them for every per-sample GEMM (so a layer needs only warp
-// synchronisation), and the weight-gradient GEMMs, which contract over the block's 64
-// samples, run after a block barrier and add into FP32 gradients in global memory.  The
-// back-propagation recomputes each layer's activations from the layer input stored in
-// the forward pass (64 x 11 values per coupling) instead of keeping them.
+// Every network layer is a GEMM on the tensor cores: bfloat16 operands, FP32 accumulation,
+// mma.sync.m16n8k16.  The networks are small (128 x 128) and the batches few hundred to a few
+// thousand samples, so what bounds a pass is the latency of its 24 layers one after another,
+// not arithmetic.  Hence the smallest unit the instruction has: a block holds 16 samples, its
+// eight warps share a layer's outputs (16 columns each), and as each weight is then used by
+// one warp only, it goes from L2 to that warp's registers in the order of the instruction's
+// fragments (packed so by the optimiser), fetched for the next coupling as soon as this one's are
+// used; no staging of weights in shared memory, four block barriers a coupling.  256 samples in
+// both directions, two calls: 156 -> 37 us (64 samples a block, weights staged between barriers).
+//
+// Training keeps a coupling's activations in shared memory for the backward pass and writes
+// the operands of the weight gradients, contractions over the samples, to global memory in
+// fragment order; a second kernel reduces them without atomics, 16 x 128 weights a block, and
+// goes on to the Adam step and the packed copies of the weights it owns.  One iteration, 1024
+// samples: 840 -> 53 us.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -28,18 +37,19 @@ using bf16 = __nv_bfloat16;
 namespace {
 
 constexpr int FD = 11, FH = 128, FC = 8, FO = 22;
-constexpr int K1 = 16;   // layer-1 reduction length (11 padded)
 constexpr int N3 = 24;   // layer-3 outputs (22 padded)
-constexpr int R3 = 32;   // W3 rows kept (22 padded to two k-steps of the backward GEMM)
 // master FP32 layout of one coupling
 constexpr int OW1 = 0, OB1 = OW1 + FH * FD, OW2 = OB1 + FH, OB2 = OW2 + FH * FH, OW3 = OB2 + FH,
               OB3 = OW3 + FO * FH, PC = OB3 + FO;
 static_assert(PC == LISA_FLOW_PARAMS_PER_COUPLING, "weight layout");
 constexpr int NP = FC * PC;
-// bfloat16 copies of one coupling: W1 [128][16], W2 [128][128], W3 [32][128]
-constexpr int BW1 = 0, BW2 = BW1 + FH * K1, BW3 = BW2 + FH * FH, BC = BW3 + R3 * FH;
-constexpr int TS = 64;    // samples per block
-constexpr int NTH = 128;  // four warps of 16 samples
+constexpr int TS = 16;     // samples per block
+constexpr int NTH = 256;   // eight warps of 16 columns
+constexpr int kBatchUnit = 64;  // minibatches are multiples of it
+// bfloat16 copies of one coupling in the order of the mma's B fragments (pair_at, single_at):
+// the forward layers and the backward ones (transposed)
+constexpr int BF1 = 0, BF2 = BF1 + 8 * 256, BF3 = BF2 + 64 * 256, BG3 = BF3 + 12 * 256,
+              BG2 = BG3 + 16 * 256, BG1 = BG2 + 64 * 256, BC = BG1 + 8 * 256;
 // shared-memory leading dimensions (bf16 elements), padded against bank conflicts
 constexpr int LW1 = 24, LH = 136, LGO = 40, LU = 12;
 constexpr float kS = 2.0f;  // s = kS tanh(o_s / kS)
@@ -54,533 +64,629 @@ __host__ __device__ inline bool keep(int c, int d) {
     }
 }
 
-// ------------------------------------------------------------------ shared memory
-struct alignas(16) SmemNet {
-    bf16 w1[FH * LW1];
-    bf16 w2[FH * LH];
-    bf16 w3[R3 * LH];
-    float b1[FH], b2[FH], b3[N3];
-    bf16 a0[TS * LW1];
-    bf16 a1[TS * LH];
-    bf16 a2[TS * LH];
-    float o[TS * N3];
-    float u[TS * LU];
-};
-
-struct alignas(16) SmemTrain {
-    SmemNet n;
-    bf16 go[TS * LGO];
-    bf16 gz2[TS * LH];
-    bf16 gz1[TS * LH];
-    float ust[FC * TS * LU];  // layer inputs of the forward pass
-    float gv[TS * LU];        // dL/dv of the current layer's output
-    float db1[FH], db2[FH], db3[N3];
-    double lsum[4];
-};
-
-// ------------------------------------------------------------------ warp GEMMs
-__device__ __forceinline__ uint32_t ld2(const bf16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
-__device__ __forceinline__ uint32_t pk(bf16 lo, bf16 hi) {
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+// Position of B[k][n] of a K = 16 KS operand: lane (n % 8) 4 + (k % 8) / 2 of the fragment
+// (n / 8, k / 16), 16 bytes a lane, which hold two neighbouring n tiles (pair) or k steps (single)
+__host__ __device__ inline int pair_at(int k, int n, int KS) {
+    const int lane = (n & 7) * 4 + ((k & 7) >> 1);
+    return (((n >> 4) * KS + (k >> 4)) * 32 + lane) * 8 + ((n >> 3) & 1) * 4 + ((k >> 3) & 1) * 2 + (k & 1);
+}
+__host__ __device__ inline int single_at(int k, int n, int KS) {
+    const int lane = (n & 7) * 4 + ((k & 7) >> 1);
+    return (((n >> 3) * (KS / 2) + (k >> 5)) * 32 + lane) * 8 + ((k >> 4) & 1) * 4 + ((k >> 3) & 1) * 2 + (k & 1);
 }
 
-__device__ __forceinline__ void mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
-                                    uint32_t a3, uint32_t b0, uint32_t b1) {
+// master weight i of a coupling (not a bias) into both packed copies
+__device__ __forceinline__ void pack_weight(bf16 *wb, int i, float v) {
+    const bf16 h = __float2bfloat16_rn(v);
+    if (i < OB1) {
+        const int r = i / FD, k = i % FD;
+        wb[BF1 + pair_at(k, r, 1)] = h;
+        wb[BG1 + single_at(r, k, 8)] = h;
+    } else if (i >= OW2 && i < OB2) {
+        const int r = (i - OW2) / FH, k = (i - OW2) % FH;
+        wb[BF2 + pair_at(k, r, 8)] = h;
+        wb[BG2 + pair_at(r, k, 8)] = h;
+    } else if (i >= OW3 && i < OB3) {
+        const int r = (i - OW3) / FH, k = (i - OW3) % FH;
+        wb[BF3 + single_at(k, r, 8)] = h;
+        wb[BG3 + pair_at(r, k, 2)] = h;
+    }
+}
+
+// ------------------------------------------------------------------ warp GEMMs
+__device__ __forceinline__ uint32_t pk(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+__device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
         "{%8,%9}, {%0,%1,%2,%3};\n"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// C[16][8 NT] += A[16][16 KS] B with A row-major (lda) and B[k][n] = Bt[n][k] (ldb)
-template <int NT, int KS>
-__device__ __forceinline__ void mma_nt(const bf16 *A, int lda, const bf16 *Bt, int ldb,
-                                       float (&c)[NT][4], int lane) {
-    const int g = lane >> 2, t = lane & 3;
+// A fragment of A[16][16] at p (row-major, leading dimension ld, 16-byte aligned rows)
+__device__ __forceinline__ void load_a(uint32_t (&a)[4], const bf16 *p, int ld, int lane) {
+    const uint32_t s = (uint32_t)__cvta_generic_to_shared(p + (lane & 15) * ld + (lane >> 4) * 8);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+                 : "r"(s));
+}
+
+// S[16][16] at p transposed: as the A fragment of S^T (16 m of 16 k), or as the B fragments
+// of two neighbouring n tiles (S = B[k][n])
+__device__ __forceinline__ uint4 load_t(const bf16 *p, int ld, int lane, bool as_a) {
+    const int q = lane >> 3, r = lane & 7;
+    const int kh = as_a ? q >> 1 : q & 1, mh = as_a ? q & 1 : q >> 1;
+    const uint32_t s = (uint32_t)__cvta_generic_to_shared(p + (r + 8 * kh) * ld + 8 * mh);
+    uint4 v;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(s));
+    return v;
+}
+
+__device__ __forceinline__ uint4 frag(const bf16 *wb, int at, int lane) {
+    return __ldg(reinterpret_cast<const uint4 *>(wb + at) + lane);
+}
+
+// c[2] (16 columns) += A[16][16 KS] B, A in shared memory
+template <int KS>
+__device__ __forceinline__ void gemm_pair(const bf16 *A, int lda, const uint4 (&b)[KS], float (&c)[2][4],
+                                          int lane) {
 #pragma unroll
     for (int ks = 0; ks < KS; ks++) {
-        const int k0 = 16 * ks + 2 * t;
-        const uint32_t a0 = ld2(A + g * lda + k0), a1 = ld2(A + (g + 8) * lda + k0);
-        const uint32_t a2 = ld2(A + g * lda + k0 + 8), a3 = ld2(A + (g + 8) * lda + k0 + 8);
-#pragma unroll
-        for (int nt = 0; nt < NT; nt++) {
-            const bf16 *bp = Bt + (nt * 8 + g) * ldb + k0;
-            mma(c[nt], a0, a1, a2, a3, ld2(bp), ld2(bp + 8));
-        }
+        uint32_t a[4];
+        load_a(a, A + 16 * ks, lda, lane);
+        mma(c[0], a, b[ks].x, b[ks].y);
+        mma(c[1], a, b[ks].z, b[ks].w);
     }
 }
 
-// C[16][8 NT] += A[16][16 KS] B with A row-major (lda) and B[k][n] = Bk[k][n] (ldb)
-template <int NT, int KS>
-__device__ __forceinline__ void mma_nn(const bf16 *A, int lda, const bf16 *Bk, int ldb,
-                                       float (&c)[NT][4], int lane) {
-    const int g = lane >> 2, t = lane & 3;
+// c (8 columns) += A[16][128] B
+__device__ __forceinline__ void gemm_single(const bf16 *A, int lda, const uint4 (&b)[4], float (&c)[4],
+                                            int lane) {
 #pragma unroll
-    for (int ks = 0; ks < KS; ks++) {
-        const int k0 = 16 * ks + 2 * t;
-        const uint32_t a0 = ld2(A + g * lda + k0), a1 = ld2(A + (g + 8) * lda + k0);
-        const uint32_t a2 = ld2(A + g * lda + k0 + 8), a3 = ld2(A + (g + 8) * lda + k0 + 8);
-#pragma unroll
-        for (int nt = 0; nt < NT; nt++) {
-            const int n = nt * 8 + g;
-            const uint32_t b0 = pk(Bk[k0 * ldb + n], Bk[(k0 + 1) * ldb + n]);
-            const uint32_t b1 = pk(Bk[(k0 + 8) * ldb + n], Bk[(k0 + 9) * ldb + n]);
-            mma(c[nt], a0, a1, a2, a3, b0, b1);
-        }
+    for (int k2 = 0; k2 < 4; k2++) {
+        uint32_t a[4];
+        load_a(a, A + 32 * k2, lda, lane);
+        mma(c, a, b[k2].x, b[k2].y);
+        load_a(a, A + 32 * k2 + 16, lda, lane);
+        mma(c, a, b[k2].z, b[k2].w);
     }
 }
 
-// C[16][8 NT] += At^T B over the 64 samples: A[m][k] = At[k][m0 + m] (lda),
-// B[k][n] = Bk[k][n0 + n] (ldb)
-template <int NT>
-__device__ __forceinline__ void mma_tn(const bf16 *At, int lda, int m0, const bf16 *Bk, int ldb,
-                                       int n0, float (&c)[NT][4], int lane) {
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int ks = 0; ks < TS / 16; ks++) {
-        const int k0 = 16 * ks + 2 * t;
-        const int m = m0 + g;
-        const uint32_t a0 = pk(At[k0 * lda + m], At[(k0 + 1) * lda + m]);
-        const uint32_t a1 = pk(At[k0 * lda + m + 8], At[(k0 + 1) * lda + m + 8]);
-        const uint32_t a2 = pk(At[(k0 + 8) * lda + m], At[(k0 + 9) * lda + m]);
-        const uint32_t a3 = pk(At[(k0 + 8) * lda + m + 8], At[(k0 + 9) * lda + m + 8]);
-#pragma unroll
-        for (int nt = 0; nt < NT; nt++) {
-            const int n = n0 + nt * 8 + g;
-            const uint32_t b0 = pk(Bk[k0 * ldb + n], Bk[(k0 + 1) * ldb + n]);
-            const uint32_t b1 = pk(Bk[(k0 + 8) * ldb + n], Bk[(k0 + 9) * ldb + n]);
-            mma(c[nt], a0, a1, a2, a3, b0, b1);
-        }
-    }
-}
-
-template <int NT>
-__device__ __forceinline__ void zero(float (&c)[NT][4]) {
-#pragma unroll
-    for (int i = 0; i < NT; i++) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.0f;
-}
-
-// ------------------------------------------------------------------ network pieces
-__device__ void load_coupling(SmemNet &sm, const bf16 *wb, const float *w, int c) {
-    const bf16 *src = wb + (size_t)c * BC;
-    const float *ws = w + (size_t)c * PC;
-    for (int i = threadIdx.x; i < FH * 2; i += NTH) {
-        const int r = i >> 1, q = i & 1;
-        *reinterpret_cast<uint4 *>(sm.w1 + r * LW1 + q * 8) =
-            *reinterpret_cast<const uint4 *>(src + BW1 + r * K1 + q * 8);
-    }
-    for (int i = threadIdx.x; i < FH * 16; i += NTH) {
-        const int r = i >> 4, q = i & 15;
-        *reinterpret_cast<uint4 *>(sm.w2 + r * LH + q * 8) =
-            *reinterpret_cast<const uint4 *>(src + BW2 + r * FH + q * 8);
-    }
-    for (int i = threadIdx.x; i < R3 * 16; i += NTH) {
-        const int r = i >> 4, q = i & 15;
-        *reinterpret_cast<uint4 *>(sm.w3 + r * LH + q * 8) =
-            *reinterpret_cast<const uint4 *>(src + BW3 + r * FH + q * 8);
-    }
-    for (int i = threadIdx.x; i < FH; i += NTH) {
-        sm.b1[i] = ws[OB1 + i];
-        sm.b2[i] = ws[OB2 + i];
-        if (i < N3) sm.b3[i] = i < FO ? ws[OB3 + i] : 0.0f;
-    }
-}
-
-// The coupling network of layer c on the warp's 16 rows r0.. of `uin` (row stride LU):
-// a0 = bf16(m u), a1 = bf16(relu(W1 a0 + b1)), a2 = bf16(relu(W2 a1 + b2)), o = W3 a2 + b3.
-__device__ void net_forward(SmemNet &sm, const float *uin, int c, int r0, int lane) {
-    for (int i = lane; i < 16 * K1; i += 32) {
-        const int r = i >> 4, k = i & 15;
-        const float v = (k < FD && keep(c, k)) ? uin[(r0 + r) * LU + k] : 0.0f;
-        sm.a0[(r0 + r) * LW1 + k] = __float2bfloat16_rn(v);
-    }
-    __syncwarp();
-    const int g = lane >> 2, t = lane & 3;
-    {
-        float acc[16][4];
-        zero(acc);
-        mma_nt<16, 1>(sm.a0 + r0 * LW1, LW1, sm.w1, LW1, acc, lane);
-#pragma unroll
-        for (int nt = 0; nt < 16; nt++) {
-            const int col = nt * 8 + 2 * t;
-            const float bl = sm.b1[col], bh = sm.b1[col + 1];
-            *reinterpret_cast<uint32_t *>(sm.a1 + (r0 + g) * LH + col) =
-                pk(__float2bfloat16_rn(fmaxf(acc[nt][0] + bl, 0.0f)),
-                   __float2bfloat16_rn(fmaxf(acc[nt][1] + bh, 0.0f)));
-            *reinterpret_cast<uint32_t *>(sm.a1 + (r0 + g + 8) * LH + col) =
-                pk(__float2bfloat16_rn(fmaxf(acc[nt][2] + bl, 0.0f)),
-                   __float2bfloat16_rn(fmaxf(acc[nt][3] + bh, 0.0f)));
-        }
-    }
-    __syncwarp();
-    {
-        float acc[16][4];
-        zero(acc);
-        mma_nt<16, 8>(sm.a1 + r0 * LH, LH, sm.w2, LH, acc, lane);
-#pragma unroll
-        for (int nt = 0; nt < 16; nt++) {
-            const int col = nt * 8 + 2 * t;
-            const float bl = sm.b2[col], bh = sm.b2[col + 1];
-            *reinterpret_cast<uint32_t *>(sm.a2 + (r0 + g) * LH + col) =
-                pk(__float2bfloat16_rn(fmaxf(acc[nt][0] + bl, 0.0f)),
-                   __float2bfloat16_rn(fmaxf(acc[nt][1] + bh, 0.0f)));
-            *reinterpret_cast<uint32_t *>(sm.a2 + (r0 + g + 8) * LH + col) =
-                pk(__float2bfloat16_rn(fmaxf(acc[nt][2] + bl, 0.0f)),
-                   __float2bfloat16_rn(fmaxf(acc[nt][3] + bh, 0.0f)));
-        }
-    }
-    __syncwarp();
-    {
-        float acc[3][4];
-        zero(acc);
-        mma_nt<3, 8>(sm.a2 + r0 * LH, LH, sm.w3, LH, acc, lane);
-#pragma unroll
-        for (int nt = 0; nt < 3; nt++) {
-            const int col = nt * 8 + 2 * t;
-            sm.o[(r0 + g) * N3 + col] = acc[nt][0] + sm.b3[col];
-            sm.o[(r0 + g) * N3 + col + 1] = acc[nt][1] + sm.b3[col + 1];
-            sm.o[(r0 + g + 8) * N3 + col] = acc[nt][2] + sm.b3[col];
-            sm.o[(r0 + g + 8) * N3 + col + 1] = acc[nt][3] + sm.b3[col + 1];
-        }
-    }
-    __syncwarp();
-}
-
-// the coupling update of one row: normalizing (x -> z) or generating (z -> x); returns
-// the row's sum of s
-__device__ float couple_row(SmemNet &sm, int c, int row, bool gen) {
-    float ssum = 0.0f;
-    for (int d = 0; d < FD; d++) {
-        if (keep(c, d)) continue;
-        const float s = kS * tanhf(sm.o[row * N3 + d] / kS);
-        const float tt = sm.o[row * N3 + FD + d];
-        float &u = sm.u[row * LU + d];
-        u = gen ? u * expf(s) + tt : (u - tt) * expf(-s);
-        ssum += s;
-    }
-    return ssum;
-}
-
-// ------------------------------------------------------------------ evaluation
+// ------------------------------------------------------------------ network
 struct FlowView {
     const float *w;
     const bf16 *wb;
     const double *mu, *L;  // mean [11], lower-triangular whitening factor [11][11]
 };
 
-// u = L^{-1} (x - mu) by forward substitution (FP64), written as FP32
-__device__ inline void whiten_row(const double *x, const double *mu, const double *L, float *u) {
+// the weights of a coupling that a warp needs in the forward pass
+struct Forward {
+    uint4 f1[1], f2[8], f3[4];
+    float b1[4], b2[4], b3[2];
+
+    __device__ __forceinline__ void load1(const FlowView &f, int c, int warp, int lane) {
+        f1[0] = frag(f.wb + (size_t)c * BC, BF1 + warp * 256, lane);
+        bias(b1, f.w + (size_t)c * PC + OB1, warp, lane);
+    }
+    __device__ __forceinline__ void load2(const FlowView &f, int c, int warp, int lane) {
+#pragma unroll
+        for (int ks = 0; ks < 8; ks++) f2[ks] = frag(f.wb + (size_t)c * BC, BF2 + (warp * 8 + ks) * 256, lane);
+        bias(b2, f.w + (size_t)c * PC + OB2, warp, lane);
+    }
+    __device__ __forceinline__ void load3(const FlowView &f, int c, int warp, int lane) {
+        if (warp >= 3) return;
+#pragma unroll
+        for (int k2 = 0; k2 < 4; k2++) f3[k2] = frag(f.wb + (size_t)c * BC, BF3 + (warp * 4 + k2) * 256, lane);
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+            const int col = warp * 8 + 2 * (lane & 3) + j;
+            b3[j] = col < FO ? __ldg(f.w + (size_t)c * PC + OB3 + col) : 0.0f;
+        }
+    }
+    static __device__ __forceinline__ void bias(float (&b)[4], const float *src, int warp, int lane) {
+#pragma unroll
+        for (int j = 0; j < 4; j++) b[j] = __ldg(src + warp * 16 + (j >> 1) * 8 + 2 * (lane & 3) + (j & 1));
+    }
+};
+
+// relu(c + b) of a warp's 16 columns to bf16 rows
+__device__ __forceinline__ void put_relu(bf16 *out, const float (&c)[2][4], const float (&b)[4], int warp,
+                                         int lane) {
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+        const int col = warp * 16 + i * 8 + 2 * t;
+        *reinterpret_cast<uint32_t *>(out + g * LH + col) =
+            pk(fmaxf(c[i][0] + b[2 * i], 0.0f), fmaxf(c[i][1] + b[2 * i + 1], 0.0f));
+        *reinterpret_cast<uint32_t *>(out + (g + 8) * LH + col) =
+            pk(fmaxf(c[i][2] + b[2 * i], 0.0f), fmaxf(c[i][3] + b[2 * i + 1], 0.0f));
+    }
+}
+
+// The coupling network on the block's 16 rows: a1 = bf16(relu(W1 a0 + b1)), a2 =
+// bf16(relu(W2 a1 + b2)), o = W3 a2 + b3; the weights of coupling cn (if >= 0) are fetched as
+// those of this one have been used.  Ends with a block barrier.
+__device__ __forceinline__ void net_forward(const FlowView &f, Forward &w, int cn, const bf16 *a0, bf16 *a1,
+                                            bf16 *a2, float *o, int warp, int lane) {
+    {
+        float acc[2][4] = {};
+        gemm_pair<1>(a0, LW1, w.f1, acc, lane);
+        put_relu(a1, acc, w.b1, warp, lane);
+        if (cn >= 0) w.load1(f, cn, warp, lane);
+    }
+    __syncthreads();
+    {
+        float acc[2][4] = {};
+        gemm_pair<8>(a1, LH, w.f2, acc, lane);
+        put_relu(a2, acc, w.b2, warp, lane);
+        if (cn >= 0) w.load2(f, cn, warp, lane);
+    }
+    __syncthreads();
+    if (warp < 3) {
+        float acc[4] = {};
+        gemm_single(a2, LH, w.f3, acc, lane);
+        const int g = lane >> 2, col = warp * 8 + 2 * (lane & 3);
+        o[g * N3 + col] = acc[0] + w.b3[0];
+        o[g * N3 + col + 1] = acc[1] + w.b3[1];
+        o[(g + 8) * N3 + col] = acc[2] + w.b3[0];
+        o[(g + 8) * N3 + col + 1] = acc[3] + w.b3[1];
+        if (cn >= 0) w.load3(f, cn, warp, lane);
+    }
+    __syncthreads();
+}
+
+// thread (row, d): coordinate d of row after coupling c, normalizing (x -> z) or generating
+// (z -> x); s is what it was scaled by (kept coordinates: 0)
+__device__ __forceinline__ float couple(const float *o, int c, int row, int d, bool gen, float u, float &s) {
+    s = 0.0f;
+    if (d >= FD || keep(c, d)) return u;
+    s = kS * tanhf(o[row * N3 + d] / kS);
+    const float tt = o[row * N3 + FD + d];
+    return gen ? u * expf(s) + tt : (u - tt) * expf(-s);
+}
+
+// thread (row, d): the network's input of coupling c
+__device__ __forceinline__ void put_a0(bf16 *a0, int c, int row, int d, float u) {
+    a0[row * LW1 + d] = __float2bfloat16_rn(d < FD && keep(c, d) ? u : 0.0f);
+}
+
+// a row's sum of s in coupling c, in the order of the coordinates
+__device__ __forceinline__ float s_sum(const float *s, int c) {
+    float t = 0.0f;
+    for (int d = 0; d < FD; d++)
+        if (!keep(c, d)) t += s[d];
+    return t;
+}
+
+// u = L^{-1} (x - mu) by forward substitution (FP64), written as FP32: one thread per row, the
+// rows of a block in one warp (an FP64 instruction takes a warp's time, 16 clocks of the SM's
+// pipe, however few lanes take part: dealt to 16 threads a row, this took 12 us)
+__device__ __forceinline__ void whiten_row(const FlowView &f, const double *x, float *u) {
     double v[FD];
+#pragma unroll
     for (int d = 0; d < FD; d++) {
-        double acc = x[d] - mu[d];
-        for (int j = 0; j < d; j++) acc -= L[d * FD + j] * v[j];
-        v[d] = acc / L[d * FD + d];
+        double acc = x[d] - f.mu[d];
+#pragma unroll
+        for (int j = 0; j < d; j++) acc -= f.L[d * FD + j] * v[j];
+        v[d] = acc / f.L[d * FD + d];
         u[d] = (float)v[d];
     }
 }
 
-__device__ inline double log_det_factor(const double *L) {
+// sum of the logarithms of the factor's diagonal, in order: a whole warp, result on all lanes
+__device__ __forceinline__ double log_det_factor(const double *L, int lane) {
+    const double l = log(L[min(lane, FD - 1) * (FD + 1)]);
     double s = 0.0;
-    for (int d = 0; d < FD; d++) s += log(L[d * FD + d]);
+    for (int d = 0; d < FD; d++) s += __shfl_sync(0xffffffffu, l, d);
     return s;
 }
 
-// Both directions for up to 64 rows per block.  Normalizing: in = x, out = z;
+struct SmemNet {
+    alignas(16) bf16 a0[TS * LW1];
+    alignas(16) bf16 a1[TS * LH];
+    alignas(16) bf16 a2[TS * LH];
+    float o[TS * N3];
+    float u[TS * LU];
+    float s[FC][TS][LU];
+    double lsig;
+};
+
+// all couplings on the block's rows; u: this thread's coordinate (row threadIdx.x / 16, d =
+// threadIdx.x % 16), also left in sm.u.  `w` holds the first coupling's weights, and the
+// second pass's first one's (cn2, or -1) on return.
+__device__ __forceinline__ float run_couplings(SmemNet &sm, const FlowView &f, Forward &w, float u, bool gen,
+                                               int cn2) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, row = threadIdx.x >> 4, d = threadIdx.x & 15;
+    put_a0(sm.a0, gen ? FC - 1 : 0, row, d, u);
+    __syncthreads();
+    for (int k = 0; k < FC; k++) {
+        const int c = gen ? FC - 1 - k : k, cn = k + 1 < FC ? (gen ? c - 1 : c + 1) : -1;
+        net_forward(f, w, cn >= 0 ? cn : cn2, sm.a0, sm.a1, sm.a2, sm.o, warp, lane);
+        float s;
+        u = couple(sm.o, c, row, d, gen, u, s);
+        if (d < LU) sm.s[c][row][d] = s;
+        if (cn >= 0)
+            put_a0(sm.a0, cn, row, d, u);
+        else if (d < LU)
+            sm.u[row * LU + d] = u;
+        __syncthreads();
+    }
+    return u;
+}
+
+__device__ __forceinline__ void first_weights(const FlowView &f, Forward &w, int c) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    w.load1(f, c, warp, lane);
+    w.load2(f, c, warp, lane);
+    w.load3(f, c, warp, lane);
+}
+
+// ------------------------------------------------------------------ evaluation
+// Both directions for up to 16 rows per block.  Normalizing: in = x, out = z;
 // generating: in = z, out = x.  logq = log q(x) in both cases.
 __global__ void __launch_bounds__(NTH) flow_eval_kernel(FlowView f, const double *in, int n,
                                                         int gen, double *out, double *logq) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    SmemNet &sm = *reinterpret_cast<SmemNet *>(smraw);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r0 = warp * 16;
-    const int row0 = blockIdx.x * TS;
-    double lq = 0.0;  // lanes 0..15: the row r0 + lane
+    __shared__ SmemNet sm;
+    Forward w;
+    first_weights(f, w, gen ? FC - 1 : 0);
+    const int r = threadIdx.x >> 4, d = threadIdx.x & 15, row = blockIdx.x * TS + r;
+    const int own = blockIdx.x * TS + threadIdx.x;  // threads 0 .. 15: one row each
     if (threadIdx.x < TS) {
-        const int r = threadIdx.x, row = row0 + r;
-        float *u = sm.u + r * LU;
-        for (int d = 0; d < LU; d++) u[d] = 0.0f;
-        if (row < n) {
+        float *u = sm.u + threadIdx.x * LU;
+        for (int j = 0; j < LU; j++) u[j] = 0.0f;
+        if (own < n) {
             if (gen)
-                for (int d = 0; d < FD; d++) u[d] = (float)in[(size_t)row * FD + d];
+                for (int j = 0; j < FD; j++) u[j] = (float)in[(size_t)own * FD + j];
             else
-                whiten_row(in + (size_t)row * FD, f.mu, f.L, u);
+                whiten_row(f, in + (size_t)own * FD, u);
         }
     }
+    if (threadIdx.x >= NTH - 32) {
+        const double l = log_det_factor(f.L, threadIdx.x & 31);
+        if (threadIdx.x == NTH - 1) sm.lsig = l;
+    }
     __syncthreads();
-    if (gen && lane < 16) {
-        const int row = row0 + r0 + lane;
-        if (row < n) {
-            double zz = 0.0;
-            for (int d = 0; d < FD; d++) {
-                const double zv = in[(size_t)row * FD + d];
+    const float u = run_couplings(sm, f, w, d < LU ? sm.u[r * LU + d] : 0.0f, gen != 0, -1);
+    if (row < n && d < FD) {
+        if (gen) {
+            double xv = f.mu[d];  // x = mu + L v
+            for (int j = 0; j <= d; j++) xv += f.L[d * FD + j] * (double)sm.u[r * LU + j];
+            out[(size_t)row * FD + d] = xv;
+        } else if (out) {
+            out[(size_t)row * FD + d] = u;
+        }
+    }
+    if (threadIdx.x < TS && own < n) {
+        double zz = 0.0, lq = 0.0;
+        if (gen) {
+            for (int j = 0; j < FD; j++) {
+                const double zv = in[(size_t)own * FD + j];
                 zz += zv * zv;
             }
             lq = -0.5 * zz - 0.5 * FD * kLog2Pi;
         }
-    }
-    for (int k = 0; k < FC; k++) {
-        const int c = gen ? FC - 1 - k : k;
-        load_coupling(sm, f.wb, f.w, c);
-        __syncthreads();
-        net_forward(sm, sm.u, c, r0, lane);
-        if (lane < 16) lq -= (double)couple_row(sm, c, r0 + lane, gen != 0);
-        __syncwarp();
-        __syncthreads();
-    }
-    if (lane < 16) {
-        const int rr = r0 + lane, row = row0 + rr;
-        if (row < n) {
-            const double lsig = log_det_factor(f.L);
-            double zz = 0.0;
-            for (int d = 0; d < FD; d++) {
-                const double v = sm.u[rr * LU + d];
-                if (gen) {
-                    double xv = f.mu[d];  // x = mu + L v
-                    for (int j = 0; j <= d; j++) xv += f.L[d * FD + j] * (double)sm.u[rr * LU + j];
-                    out[(size_t)row * FD + d] = xv;
-                } else {
-                    zz += v * v;
-                    if (out) out[(size_t)row * FD + d] = v;
-                }
-            }
-            logq[row] = gen ? lq - lsig : -0.5 * zz - 0.5 * FD * kLog2Pi + lq - lsig;
+        for (int k = 0; k < FC; k++) {
+            const int c = gen ? FC - 1 - k : k;
+            lq -= (double)s_sum(sm.s[c][threadIdx.x], c);
         }
+        if (!gen)
+            for (int j = 0; j < FD; j++) {
+                const double v = sm.u[threadIdx.x * LU + j];
+                zz += v * v;
+            }
+        logq[own] = gen ? lq - sm.lsig : -0.5 * zz - 0.5 * FD * kLog2Pi + lq - sm.lsig;
     }
 }
 
 // ------------------------------------------------------------------ training
+// Operands of the weight gradients of one coupling and 16 samples (a k step of the
+// contraction), as 512-byte fragments: dL/d(pre-activations) of layers 2 and 3 and the inputs
+// of layer 1 as A, the inputs of layers 2 and 3 and dL/d(pre-activations) of layer 1 as B.
+constexpr int UGZ2 = 0, UGO = 8, UA0 = 10, UA1 = 11, UA2 = 19, UGZ1 = 27, kUnits = 35;
+constexpr int kChunkSteps = 128;  // k steps held at a time: 2048 samples, 18 MB
+constexpr int kBias = 2 * FH + N3;
+
 struct TrainArgs {
-    const float *w;
-    const bf16 *wb;
-    float *grad;            // [8][PC], accumulated
-    const double *mu, *L;
+    FlowView f;
     const double *data;     // [n][11]
     long long n;
     int batch;              // rows of this minibatch (multiple of 64)
+    int row0;               // first of them in this chunk
     uint32_t k0, k1, round, iter;
     int random_rows;        // 1: Philox minibatch rows; 0: rows 0..batch-1 in order
-    double *loss;           // accumulated mean loss of the minibatch
+    uint4 *act;             // [FC][steps][kUnits][32]
+    float *bias;            // [steps][FC][kBias]: sums over the step's samples
+    double *lossp;          // [steps]
 };
 
+struct SmemTrain {
+    alignas(16) bf16 a0[FC][TS * LW1];
+    alignas(16) bf16 a1[FC][TS * LH];
+    alignas(16) bf16 a2[FC][TS * LH];
+    alignas(16) bf16 go[TS * LGO];
+    alignas(16) bf16 gz2[TS * LH];
+    alignas(16) bf16 gz1[TS * LH];
+    float o[FC][TS * N3];
+    float s[FC][TS][LU];
+    float z[TS * LU], gv[TS * LU];  // gv: dL/dv of the current layer's output
+    float g3[TS * N3];
+    double lrow[TS];
+};
+
+// sums over the 16 rows of a warp's 16 columns
+__device__ __forceinline__ void column_sums(float *out, float (&v)[2][4], int warp, int lane) {
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+            float s = v[i][j] + v[i][j + 2];
+            for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane < 4) out[warp * 16 + i * 8 + 2 * lane + j] = s;
+        }
+}
+
+// masked by the relu's output a (> 0), to bf16 rows
+__device__ __forceinline__ void put_masked(bf16 *out, float (&v)[2][4], const bf16 *a, int warp, int lane) {
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int at = (g + 8 * h) * LH + warp * 16 + i * 8 + 2 * t;
+            float &v0 = v[i][2 * h], &v1 = v[i][2 * h + 1];
+            if (!(__bfloat162float(a[at]) > 0.0f)) v0 = 0.0f;
+            if (!(__bfloat162float(a[at + 1]) > 0.0f)) v1 = 0.0f;
+            *reinterpret_cast<uint32_t *>(out + at) = pk(v0, v1);
+        }
+}
+
+// Forward and backward pass of 16 samples: one k step of the weight gradients.
 __global__ void __launch_bounds__(NTH) flow_train_kernel(TrainArgs a) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    SmemTrain &st = *reinterpret_cast<SmemTrain *>(smraw);
-    SmemNet &sm = st.n;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r0 = warp * 16;
-    const int g = lane >> 2, t = lane & 3;
+    SmemTrain &sm = *reinterpret_cast<SmemTrain *>(smraw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int row = threadIdx.x >> 4, d = threadIdx.x & 15, step = blockIdx.x, steps = gridDim.x;
     const float inv_n = 1.0f / (float)a.batch;
+    const FlowView f = a.f;
+    Forward w;
+    first_weights(f, w, 0);
     // minibatch rows, whitened
+    float u, us[FC];  // coordinate d of every coupling's input
     if (threadIdx.x < TS) {
-        const int r = threadIdx.x, j = blockIdx.x * TS + r;
+        const int j = a.row0 + step * TS + threadIdx.x;
         long long idx = j;
         if (a.random_rows) {
             const lisa_smp::U4 q = lisa_smp::philox(a.round, 5u, a.iter, (uint32_t)(j >> 2), a.k0, a.k1);
             idx = (long long)(lisa_smp::unit(q.v[j & 3]) * (double)a.n);
             if (idx > a.n - 1) idx = a.n - 1;
         }
-        sm.u[r * LU + FD] = 0.0f;
-        whiten_row(a.data + idx * FD, a.mu, a.L, sm.u + r * LU);
+        sm.z[threadIdx.x * LU + FD] = 0.0f;
+        whiten_row(f, a.data + idx * FD, sm.z + threadIdx.x * LU);
     }
     __syncthreads();
-    float ssum = 0.0f;  // lanes 0..15: the row's sum of s
+    u = d < LU ? sm.z[row * LU + d] : 0.0f;
+    put_a0(sm.a0[0], 0, row, d, u);
+    __syncthreads();
+#pragma unroll
     for (int c = 0; c < FC; c++) {
-        load_coupling(sm, a.wb, a.w, c);
-        for (int i = lane; i < 16 * LU; i += 32) st.ust[(c * TS + r0) * LU + i] = sm.u[r0 * LU + i];
-        __syncthreads();
-        net_forward(sm, sm.u, c, r0, lane);
-        if (lane < 16) ssum += couple_row(sm, c, r0 + lane, false);
-        __syncwarp();
+        us[c] = u;
+        net_forward(f, w, c + 1 < FC ? c + 1 : -1, sm.a0[c], sm.a1[c], sm.a2[c], sm.o[c], warp, lane);
+        float s;
+        u = couple(sm.o[c], c, row, d, false, u, s);
+        if (d < LU) sm.s[c][row][d] = s;
+        if (c + 1 < FC) put_a0(sm.a0[c + 1], c + 1, row, d, u);
+        uint4 *act = a.act + ((size_t)c * steps + step) * kUnits * 32 + lane;
+        if (warp == 0) act[UA0 * 32] = load_t(sm.a0[c], LW1, lane, true);
+        act[(UA1 + warp) * 32] = load_t(sm.a1[c] + 16 * warp, LH, lane, false);
+        act[(UA2 + warp) * 32] = load_t(sm.a2[c] + 16 * warp, LH, lane, false);
         __syncthreads();
     }
     // loss and dL/dz = z / batch
-    double lrow = 0.0;
-    if (lane < 16) {
-        const int rr = r0 + lane;
-        float zz = 0.0f;
-        for (int d = 0; d < FD; d++) {
-            const float z = sm.u[rr * LU + d];
-            zz += z * z;
-            st.gv[rr * LU + d] = z * inv_n;
-        }
-        lrow = 0.5 * (double)zz + (double)ssum;
-    }
-    for (int o = 16; o > 0; o >>= 1) lrow += __shfl_xor_sync(0xffffffffu, lrow, o);
-    if (lane == 0) st.lsum[warp] = lrow;
+    if (d < LU) sm.z[row * LU + d] = u;
+    float gv = u * inv_n;  // dL/dv of coordinate d
+    uint4 g3[2], g2[8], g1[4];
+    auto load3 = [&](int c) {
+#pragma unroll
+        for (int ks = 0; ks < 2; ks++) g3[ks] = frag(f.wb + (size_t)c * BC, BG3 + (warp * 2 + ks) * 256, lane);
+    };
+    auto load2 = [&](int c) {
+#pragma unroll
+        for (int ks = 0; ks < 8; ks++) g2[ks] = frag(f.wb + (size_t)c * BC, BG2 + (warp * 8 + ks) * 256, lane);
+    };
+    auto load1 = [&](int c) {
+        if (warp >= 2) return;
+#pragma unroll
+        for (int k2 = 0; k2 < 4; k2++) g1[k2] = frag(f.wb + (size_t)c * BC, BG1 + (warp * 4 + k2) * 256, lane);
+    };
+    load3(FC - 1);
+    load2(FC - 1);
+    load1(FC - 1);
     __syncthreads();
-    if (threadIdx.x == 0)
-        atomicAdd(a.loss, (st.lsum[0] + st.lsum[1] + st.lsum[2] + st.lsum[3]) / (double)a.batch);
+    if (threadIdx.x < TS) {
+        const int r = threadIdx.x;
+        float zz = 0.0f, ssum = 0.0f;
+        for (int j = 0; j < FD; j++) zz += sm.z[r * LU + j] * sm.z[r * LU + j];
+        for (int c = 0; c < FC; c++) ssum += s_sum(sm.s[c][r], c);
+        sm.lrow[r] = 0.5 * (double)zz + (double)ssum;
+    }
+#pragma unroll
     for (int c = FC - 1; c >= 0; c--) {
-        load_coupling(sm, a.wb, a.w, c);
-        for (int i = threadIdx.x; i < FH; i += NTH) {
-            st.db1[i] = 0.0f;
-            st.db2[i] = 0.0f;
-            if (i < N3) st.db3[i] = 0.0f;
-        }
-        for (int i = lane; i < 16 * LU; i += 32) sm.u[r0 * LU + i] = st.ust[(c * TS + r0) * LU + i];
-        __syncthreads();
-        net_forward(sm, sm.u, c, r0, lane);
+        float *bias = a.bias + ((size_t)step * FC + c) * kBias;
         // dL/ds, dL/dt of the coupling, and dL/du through the affine map
-        if (lane < 16) {
-            const int rr = r0 + lane;
-            for (int k = 0; k < LGO; k++) st.go[rr * LGO + k] = __float2bfloat16_rn(0.0f);
-            for (int d = 0; d < FD; d++) {
-                if (keep(c, d)) continue;
-                const float th = tanhf(sm.o[rr * N3 + d] / kS);
+        {
+            float gs = 0.0f, gt = 0.0f;
+            if (d < FD && !keep(c, d)) {
+                const float th = tanhf(sm.o[c][row * N3 + d] / kS);
                 const float s = kS * th;
                 const float e = expf(-s);
-                const float v = (sm.u[rr * LU + d] - sm.o[rr * N3 + FD + d]) * e;
-                const float gvd = st.gv[rr * LU + d];
-                const float gs = (-gvd * v + inv_n) * (1.0f - th * th);
-                const float gt = -gvd * e;
-                st.go[rr * LGO + d] = __float2bfloat16_rn(gs);
-                st.go[rr * LGO + FD + d] = __float2bfloat16_rn(gt);
-                atomicAdd(&st.db3[d], gs);
-                atomicAdd(&st.db3[FD + d], gt);
-                st.gv[rr * LU + d] = gvd * e;
+                const float v = (us[c] - sm.o[c][row * N3 + FD + d]) * e;
+                gs = (-gv * v + inv_n) * (1.0f - th * th);
+                gt = -gv * e;
+                gv = gv * e;
+            }
+            if (d < FD) {
+                sm.go[row * LGO + d] = __float2bfloat16_rn(gs);
+                sm.go[row * LGO + FD + d] = __float2bfloat16_rn(gt);
+                sm.g3[row * N3 + d] = gs;
+                sm.g3[row * N3 + FD + d] = gt;
+                sm.gv[row * LU + d] = gv;
+            } else {
+                *reinterpret_cast<uint32_t *>(sm.go + row * LGO + FO + 2 * (d - FD)) = 0u;
             }
         }
-        __syncwarp();
+        __syncthreads();
+        uint4 *act = a.act + ((size_t)c * steps + step) * kUnits * 32 + lane;
         {  // dL/da2 = go W3, through the relu
-            float acc[16][4];
-            zero(acc);
-            mma_nn<16, 2>(st.go + r0 * LGO, LGO, sm.w3, LH, acc, lane);
-#pragma unroll
-            for (int nt = 0; nt < 16; nt++) {
-                const int col = nt * 8 + 2 * t;
-#pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    const int rr = r0 + g + 8 * h;
-                    const float v0 = __bfloat162float(sm.a2[rr * LH + col]) > 0.0f ? acc[nt][2 * h] : 0.0f;
-                    const float v1 = __bfloat162float(sm.a2[rr * LH + col + 1]) > 0.0f ? acc[nt][2 * h + 1] : 0.0f;
-                    atomicAdd(&st.db2[col], v0);
-                    atomicAdd(&st.db2[col + 1], v1);
-                    *reinterpret_cast<uint32_t *>(st.gz2 + rr * LH + col) =
-                        pk(__float2bfloat16_rn(v0), __float2bfloat16_rn(v1));
-                }
+            float acc[2][4] = {};
+            gemm_pair<2>(sm.go, LGO, g3, acc, lane);
+            if (c > 0) load3(c - 1);
+            put_masked(sm.gz2, acc, sm.a2[c], warp, lane);
+            column_sums(bias + FH, acc, warp, lane);
+            if (warp < 2) act[(UGO + warp) * 32] = load_t(sm.go + 16 * warp, LGO, lane, true);
+            if (warp == 7 && lane < FO) {
+                float t = 0.0f;
+                for (int r = 0; r < TS; r++) t += sm.g3[r * N3 + lane];
+                bias[2 * FH + lane] = t;
             }
         }
-        __syncwarp();
+        __syncthreads();
         {  // dL/da1 = gz2 W2, through the relu
-            float acc[16][4];
-            zero(acc);
-            mma_nn<16, 8>(st.gz2 + r0 * LH, LH, sm.w2, LH, acc, lane);
-#pragma unroll
-            for (int nt = 0; nt < 16; nt++) {
-                const int col = nt * 8 + 2 * t;
-#pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    const int rr = r0 + g + 8 * h;
-                    const float v0 = __bfloat162float(sm.a1[rr * LH + col]) > 0.0f ? acc[nt][2 * h] : 0.0f;
-                    const float v1 = __bfloat162float(sm.a1[rr * LH + col + 1]) > 0.0f ? acc[nt][2 * h + 1] : 0.0f;
-                    atomicAdd(&st.db1[col], v0);
-                    atomicAdd(&st.db1[col + 1], v1);
-                    *reinterpret_cast<uint32_t *>(st.gz1 + rr * LH + col) =
-                        pk(__float2bfloat16_rn(v0), __float2bfloat16_rn(v1));
-                }
-            }
+            float acc[2][4] = {};
+            gemm_pair<8>(sm.gz2, LH, g2, acc, lane);
+            if (c > 0) load2(c - 1);
+            put_masked(sm.gz1, acc, sm.a1[c], warp, lane);
+            column_sums(bias, acc, warp, lane);
+            act[(UGZ2 + warp) * 32] = load_t(sm.gz2 + 16 * warp, LH, lane, true);
         }
-        __syncwarp();
-        {  // dL/da0 = gz1 W1: reaches the kept coordinates of u
-            float acc[2][4];
-            zero(acc);
-            mma_nn<2, 8>(st.gz1 + r0 * LH, LH, sm.w1, LW1, acc, lane);
+        __syncthreads();
+        act[(UGZ1 + warp) * 32] = load_t(sm.gz1 + 16 * warp, LH, lane, false);
+        if (warp < 2) {  // dL/da0 = gz1 W1: reaches the kept coordinates of u
+            float acc[4] = {};
+            gemm_single(sm.gz1, LH, g1, acc, lane);
+            if (c > 0) load1(c - 1);
 #pragma unroll
-            for (int nt = 0; nt < 2; nt++) {
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const int col = nt * 8 + 2 * t + (j & 1), rr = r0 + g + 8 * (j >> 1);
-                    if (col < FD && keep(c, col)) st.gv[rr * LU + col] += acc[nt][j];
-                }
+            for (int j = 0; j < 4; j++) {
+                const int col = warp * 8 + 2 * (lane & 3) + (j & 1), rr = (lane >> 2) + 8 * (j >> 1);
+                if (col < FD && keep(c, col)) sm.gv[rr * LU + col] += acc[j];
             }
         }
         __syncthreads();
-        // weight gradients: contractions over the block's 64 samples
-        float *gw = a.grad + (size_t)c * PC;
-        {  // dW3 [22][128] = go^T a2: warp w takes columns 32w..32w+31
-            for (int mt = 0; mt < 2; mt++) {
-                float acc[4][4];
-                zero(acc);
-                mma_tn<4>(st.go, LGO, 16 * mt, sm.a2, LH, 32 * warp, acc, lane);
-#pragma unroll
-                for (int nt = 0; nt < 4; nt++)
-#pragma unroll
-                    for (int j = 0; j < 4; j++) {
-                        const int m = 16 * mt + g + 8 * (j >> 1);
-                        const int n = 32 * warp + nt * 8 + 2 * t + (j & 1);
-                        if (m < FO) atomicAdd(gw + OW3 + m * FH + n, acc[nt][j]);
-                    }
-            }
-        }
-        {  // dW2 [128][128] = gz2^T a1: warp w takes rows 32w..32w+31
-            for (int mt = 0; mt < 2; mt++)
-                for (int nc = 0; nc < 2; nc++) {
-                    float acc[8][4];
-                    zero(acc);
-                    mma_tn<8>(st.gz2, LH, 32 * warp + 16 * mt, sm.a1, LH, 64 * nc, acc, lane);
-#pragma unroll
-                    for (int nt = 0; nt < 8; nt++)
-#pragma unroll
-                        for (int j = 0; j < 4; j++) {
-                            const int m = 32 * warp + 16 * mt + g + 8 * (j >> 1);
-                            const int n = 64 * nc + nt * 8 + 2 * t + (j & 1);
-                            atomicAdd(gw + OW2 + m * FH + n, acc[nt][j]);
-                        }
-                }
-        }
-        {  // dW1 [128][11] = gz1^T a0
-            for (int mt = 0; mt < 2; mt++) {
-                float acc[2][4];
-                zero(acc);
-                mma_tn<2>(st.gz1, LH, 32 * warp + 16 * mt, sm.a0, LW1, 0, acc, lane);
-#pragma unroll
-                for (int nt = 0; nt < 2; nt++)
-#pragma unroll
-                    for (int j = 0; j < 4; j++) {
-                        const int m = 32 * warp + 16 * mt + g + 8 * (j >> 1);
-                        const int n = nt * 8 + 2 * t + (j & 1);
-                        if (n < FD) atomicAdd(gw + OW1 + m * FD + n, acc[nt][j]);
-                    }
-            }
-        }
-        for (int i = threadIdx.x; i < FH; i += NTH) {
-            atomicAdd(gw + OB1 + i, st.db1[i]);
-            atomicAdd(gw + OB2 + i, st.db2[i]);
-            if (i < FO) atomicAdd(gw + OB3 + i, st.db3[i]);
-        }
-        __syncthreads();
+        if (d < FD) gv = sm.gv[row * LU + d];
+    }
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int r = 0; r < TS; r++) t += sm.lrow[r];
+        a.lossp[step] = t / (double)a.batch;
     }
 }
 
+struct UpdateArgs {
+    const uint4 *act;
+    const float *bias;
+    const double *lossp;
+    int steps;
+    float *w, *g, *m, *v;
+    bf16 *wb;
+    double *loss;
+    int first, adam;   // first chunk of the minibatch; Adam step (or the gradient to g)
+    float lr, c1, c2;
+};
+
 // Adam on the FP32 master weights (Kingma & Ba 2015), then the bf16 copies
-__global__ void adam_kernel(float *w, const float *g, float *m, float *v, int n, float lr,
-                            float c1, float c2) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float gi = g[i];
+__device__ __forceinline__ void update(const UpdateArgs &a, int c, int i, float gi) {
+    const size_t at = (size_t)c * PC + i;
+    if (!a.first) gi += a.g[at];
+    if (!a.adam) {
+        a.g[at] = gi;
+        return;
+    }
     if (!isfinite(gi)) gi = 0.0f;
-    const float mi = 0.9f * m[i] + 0.1f * gi;
-    const float vi = 0.999f * v[i] + 0.001f * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+    const float mi = 0.9f * a.m[at] + 0.1f * gi;
+    const float vi = 0.999f * a.v[at] + 0.001f * gi * gi;
+    a.m[at] = mi;
+    a.v[at] = vi;
+    const float wi = a.w[at] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + 1e-8f);
+    a.w[at] = wi;
+    pack_weight(a.wb + (size_t)c * BC, i, wi);
+}
+
+// Weight gradients: jobs 0..7 of a coupling are 16 rows of W2 each, 8 and 9 of W3, 10 is W1
+// (transposed), 11 the biases of the hidden layers, 12 those of the outputs and the loss.  The warps take every eighth group of 64 samples
+// (four k steps in the accumulator, a minibatch's unit) and add up.
+constexpr int kJobs = 13;
+__global__ void __launch_bounds__(NTH) flow_update_kernel(UpdateArgs a) {
+    extern __shared__ __align__(16) float part[];  // [8][16][128]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, job = blockIdx.x, c = blockIdx.y;
+    if (job >= 11) {
+        const int i = job == 11 ? threadIdx.x : 2 * FH + threadIdx.x;
+        if (i < 2 * FH + FO) {
+            float s = 0.0f;
+#pragma unroll 16
+            for (int k = 0; k < a.steps; k++) s += __ldg(a.bias + ((size_t)k * FC + c) * kBias + i);
+            update(a, c, i < FH ? OB1 + i : i < 2 * FH ? OB2 + i - FH : OB3 + i - 2 * FH, s);
+        } else if (c == 0 && threadIdx.x == NTH - 1) {
+            double t = a.first ? 0.0 : *a.loss;
+#pragma unroll 16
+            for (int k = 0; k < a.steps; k++) t += __ldg(a.lossp + k);
+            *a.loss = t;
+        }
+        return;
+    }
+    const int ua = job < 8 ? UGZ2 + job : job < 10 ? UGO + job - 8 : UA0;
+    const int ub = job < 8 ? UA1 : job < 10 ? UA2 : UGZ1;
+    float sum[16][4] = {};
+    for (int k0 = 4 * warp; k0 < a.steps; k0 += 32) {
+        float acc[16][4] = {};
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const uint4 *p = a.act + ((size_t)c * a.steps + k0 + k) * kUnits * 32 + lane;
+            const uint4 fa = p[ua * 32];
+            uint4 fb[8];
+#pragma unroll
+            for (int i = 0; i < 8; i++) fb[i] = p[(ub + i) * 32];
+            const uint32_t av[4] = {fa.x, fa.y, fa.z, fa.w};
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                mma(acc[2 * i], av, fb[i].x, fb[i].y);
+                mma(acc[2 * i + 1], av, fb[i].z, fb[i].w);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 16; i++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) sum[i][j] += acc[i][j];
+    }
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        float *o = part + warp * 16 * FH + i * 8 + 2 * t;
+        *reinterpret_cast<float2 *>(o + g * FH) = make_float2(sum[i][0], sum[i][1]);
+        *reinterpret_cast<float2 *>(o + (g + 8) * FH) = make_float2(sum[i][2], sum[i][3]);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 16 * FH; e += NTH) {
+        float s = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; k++) s += part[k * 16 * FH + e];
+        const int r = e / FH, n = e % FH;
+        if (job < 8)
+            update(a, c, OW2 + (16 * job + r) * FH + n, s);
+        else if (job < 10) {
+            if (16 * (job - 8) + r < FO) update(a, c, OW3 + (16 * (job - 8) + r) * FH + n, s);
+        } else if (r < FD)
+            update(a, c, OW1 + n * FD + r, s);
+    }
 }
 
 __global__ void pack_kernel(const float *w, bf16 *wb) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= FC * BC) return;
-    const int c = i / BC, e = i % BC;
-    const float *ws = w + (size_t)c * PC;
-    float v = 0.0f;
-    if (e < BW2) {
-        const int r = e / K1, k = e % K1;
-        v = k < FD ? ws[OW1 + r * FD + k] : 0.0f;
-    } else if (e < BW3) {
-        v = ws[OW2 + (e - BW2)];
-    } else {
-        const int r = (e - BW3) / FH, k = (e - BW3) % FH;
-        v = r < FO ? ws[OW3 + r * FH + k] : 0.0f;
-    }
-    wb[i] = __float2bfloat16_rn(v);
+    if (i < NP) pack_weight(wb + (size_t)(i / PC) * BC, i % PC, w[i]);
 }
 
 // mean of each coordinate (one block per coordinate, FP64)
@@ -622,124 +728,105 @@ __global__ void cov_kernel(const double *x, long long n, const double *mu, doubl
     }
 }
 
-// Cholesky factor of the covariance, each pivot floored at 1e-12 of its diagonal entry
+// Cholesky factor of the covariance, each pivot floored at 1e-12 of its diagonal entry: one
+// warp, lane i holds row i (one thread alone: 41 us, a square root or division after another)
 __global__ void cholesky_kernel(const double *cov, double *L) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    for (int i = 0; i < FD * FD; i++) L[i] = 0.0;
-    for (int i = 0; i < FD; i++)
-        for (int j = 0; j <= i; j++) {
-            double acc = cov[i * FD + j];
-            for (int k = 0; k < j; k++) acc -= L[i * FD + k] * L[j * FD + k];
-            if (i == j) {
-                const double cii = cov[i * FD + i];
-                const double floor = cii > 0.0 ? 1e-12 * cii : 1e-300;
-                L[i * FD + i] = sqrt(fmax(acc, floor));
-            } else {
-                L[i * FD + j] = acc / L[j * FD + j];
-            }
-        }
+    const int i = threadIdx.x;
+    double l[FD], row[FD];
+#pragma unroll
+    for (int j = 0; j < FD; j++) {
+        l[j] = 0.0;
+        row[j] = i < FD ? cov[i * FD + j] : 0.0;
+    }
+#pragma unroll
+    for (int j = 0; j < FD; j++) {
+        double acc = row[j];
+#pragma unroll
+        for (int k = 0; k < j; k++) acc -= l[k] * __shfl_sync(0xffffffffu, l[k], j);
+        const double cjj = __shfl_sync(0xffffffffu, row[j], j);
+        const double piv = sqrt(fmax(__shfl_sync(0xffffffffu, acc, j), cjj > 0.0 ? 1e-12 * cjj : 1e-300));
+        if (i == j) l[j] = piv;
+        if (i > j) l[j] = acc / piv;
+    }
+    if (i < FD)
+#pragma unroll
+        for (int j = 0; j < FD; j++) L[i * FD + j] = l[j];
 }
 
 // ------------------------------------------------------------------ sampler step
 // Independence proposals for the coldest temperature: y = flow(z) with z from Philox
 // counters (step, 3, blk, w) by Box-Muller, and log q(x) - log q(y).
 __global__ void __launch_bounds__(NTH) flow_propose_kernel(FlowView f, lisa_flowint::FStep a) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    SmemNet &sm = *reinterpret_cast<SmemNet *>(smraw);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r0 = warp * 16;
-    const int w0 = blockIdx.x * TS;
+    __shared__ SmemNet sm;
+    __shared__ double zlat[TS * FD], qy[TS], px[TS * FD];
+    Forward wt;
+    first_weights(f, wt, FC - 1);
+    const int r = threadIdx.x >> 4, d = threadIdx.x & 15, w = blockIdx.x * TS + r;
     const unsigned step = *a.step;
-    __shared__ double zlat[TS * FD];
-    __shared__ double qy[TS];
-    // latent draws
+    // latent draws: threads 0 .. 47, four (three) normals each
+    if (threadIdx.x < 3 * TS) {
+        const int rr = threadIdx.x % TS, blk = threadIdx.x / TS;
+        const lisa_smp::U4 q = lisa_smp::philox(step, 3u, (uint32_t)blk, (uint32_t)(blockIdx.x * TS + rr), a.k0, a.k1);
+        for (int p = 0; p < 2; p++) {
+            const double u1 = lisa_smp::unit(q.v[2 * p]), u2 = lisa_smp::unit(q.v[2 * p + 1]);
+            const double rad = sqrt(-2.0 * log(u1));
+            double sn, cs;
+            sincos(2.0 * lisa_smp::kPi * u2, &sn, &cs);
+            const int at = 4 * blk + 2 * p;
+            zlat[rr * FD + at] = rad * cs;
+            if (at + 1 < FD) zlat[rr * FD + at + 1] = rad * sn;
+        }
+    }
+    if (threadIdx.x >= NTH - 32) {
+        const double l = log_det_factor(f.L, threadIdx.x & 31);
+        if (threadIdx.x == NTH - 1) sm.lsig = l;
+    }
+    __syncthreads();
+    float u = run_couplings(sm, f, wt, d < FD ? (float)zlat[r * FD + d] : 0.0f, true, 0);  // generate
+    const double lsig = sm.lsig;
+    const int own = blockIdx.x * TS + threadIdx.x;  // threads 0 .. 15: one row each
+    if (d < FD) {
+        double xv = f.mu[d];  // y = mu + L v
+        for (int j = 0; j <= d; j++) xv += f.L[d * FD + j] * (double)sm.u[r * LU + j];
+        if (w < a.W) a.fy[(size_t)w * FD + d] = xv;
+        px[r * FD + d] = xv;
+    }
     if (threadIdx.x < TS) {
-        const int w = w0 + threadIdx.x;
-        double nrm[12];
-        for (int blk = 0; blk < 3; blk++) {
-            const lisa_smp::U4 q = lisa_smp::philox(step, 3u, (uint32_t)blk, (uint32_t)w, a.k0, a.k1);
-            for (int p = 0; p < 2; p++) {
-                const double u1 = lisa_smp::unit(q.v[2 * p]), u2 = lisa_smp::unit(q.v[2 * p + 1]);
-                const double r = sqrt(-2.0 * log(u1));
-                double sn, cs;
-                sincos(2.0 * lisa_smp::kPi * u2, &sn, &cs);
-                nrm[4 * blk + 2 * p] = r * cs;
-                nrm[4 * blk + 2 * p + 1] = r * sn;
-            }
-        }
-        double zz = 0.0;
-        for (int d = 0; d < FD; d++) {
-            zlat[threadIdx.x * FD + d] = nrm[d];
-            zz += nrm[d] * nrm[d];
-        }
+        double zz = 0.0, lq = 0.0;
+        for (int j = 0; j < FD; j++) zz += zlat[threadIdx.x * FD + j] * zlat[threadIdx.x * FD + j];
+        for (int c = FC - 1; c >= 0; c--) lq -= (double)s_sum(sm.s[c][threadIdx.x], c);
         qy[threadIdx.x] = -0.5 * zz - 0.5 * FD * kLog2Pi;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < TS * LU; i += NTH) {
-        const int r = i / LU, d = i % LU;
-        sm.u[i] = d < FD ? (float)zlat[r * FD + d] : 0.0f;
-    }
-    __syncthreads();
-    double lq = 0.0;
-    for (int k = 0; k < FC; k++) {  // generate
-        const int c = FC - 1 - k;
-        load_coupling(sm, f.wb, f.w, c);
-        __syncthreads();
-        net_forward(sm, sm.u, c, r0, lane);
-        if (lane < 16) lq -= (double)couple_row(sm, c, r0 + lane, true);
-        __syncwarp();
-        __syncthreads();
-    }
-    const double lsig = log_det_factor(f.L);
-    if (lane < 16) {
-        const int rr = r0 + lane, w = w0 + rr;
-        if (w < a.W) {
-            for (int d = 0; d < FD; d++) {
-                double xv = f.mu[d];  // y = mu + L v
-                for (int j = 0; j <= d; j++) xv += f.L[d * FD + j] * (double)sm.u[rr * LU + j];
-                a.fy[(size_t)w * FD + d] = xv;
-            }
-            qy[rr] += lq - lsig;
-        }
+        qy[threadIdx.x] += lq - lsig;
     }
     __syncthreads();
     // log q of the current walkers
     if (threadIdx.x < TS) {
-        const int r = threadIdx.x, w = w0 + r;
-        float *u = sm.u + r * LU;
-        for (int d = 0; d < LU; d++) u[d] = 0.0f;
-        if (w < a.W) whiten_row(a.x + (size_t)w * FD, f.mu, f.L, u);
+        float *v = sm.u + threadIdx.x * LU;
+        for (int j = 0; j < LU; j++) v[j] = 0.0f;
+        if (own < a.W) whiten_row(f, a.x + (size_t)own * FD, v);
     }
     __syncthreads();
-    lq = 0.0;
-    for (int c = 0; c < FC; c++) {
-        load_coupling(sm, f.wb, f.w, c);
-        __syncthreads();
-        net_forward(sm, sm.u, c, r0, lane);
-        if (lane < 16) lq -= (double)couple_row(sm, c, r0 + lane, false);
-        __syncwarp();
-        __syncthreads();
-    }
-    if (lane < 16) {
-        const int rr = r0 + lane, w = w0 + rr;
-        if (w < a.W) {
-            double zz = 0.0;
-            for (int d = 0; d < FD; d++) {
-                const double v = sm.u[rr * LU + d];
-                zz += v * v;
-            }
-            const double qx = -0.5 * zz - 0.5 * FD * kLog2Pi + lq - lsig;
-            a.fq[w] = qx - qy[rr];
-            double y[FD];
-            for (int d = 0; d < FD; d++) y[d] = a.fy[(size_t)w * FD + d];
-            const double py = lisa_smp::ln_prior(y, a.lo, a.hi);
-            a.fpy[w] = py;
-            if (a.target == LISA_TARGET_GAUSSIAN)
-                a.fly[w] = lisa_smp::gauss_lnl(y, a.mean, a.sig);
-            else if (isfinite(py))
-                lisa_smp::to_physical(y, a.lisa_frame, a.t0, a.fpth + (size_t)w * FD);
-            else
-                lisa_smp::invalid_params(a.fpth + (size_t)w * FD);
+    u = d < LU ? sm.u[r * LU + d] : 0.0f;
+    run_couplings(sm, f, wt, u, false, -1);
+    if (threadIdx.x < TS && own < a.W) {
+        double zz = 0.0, lq = 0.0;
+        for (int c = 0; c < FC; c++) lq -= (double)s_sum(sm.s[c][threadIdx.x], c);
+        for (int j = 0; j < FD; j++) {
+            const double v = sm.u[threadIdx.x * LU + j];
+            zz += v * v;
         }
+        const double qx = -0.5 * zz - 0.5 * FD * kLog2Pi + lq - lsig;
+        a.fq[own] = qx - qy[threadIdx.x];
+        double y[FD];
+        for (int j = 0; j < FD; j++) y[j] = px[threadIdx.x * FD + j];
+        const double py = lisa_smp::ln_prior(y, a.lo, a.hi);
+        a.fpy[own] = py;
+        if (a.target == LISA_TARGET_GAUSSIAN)
+            a.fly[own] = lisa_smp::gauss_lnl(y, a.mean, a.sig);
+        else if (isfinite(py))
+            lisa_smp::to_physical(y, a.lisa_frame, a.t0, a.fpth + (size_t)own * FD);
+        else
+            lisa_smp::invalid_params(a.fpth + (size_t)own * FD);
     }
 }
 
@@ -794,8 +881,8 @@ __global__ void flow_accept_kernel(lisa_flowint::FStep a) {
     }
 }
 
-int eval_smem() { return (int)sizeof(SmemNet); }
 int train_smem() { return (int)sizeof(SmemTrain); }
+int update_smem() { return (int)(sizeof(float) * 8 * 16 * FH); }
 
 }  // namespace
 
@@ -805,6 +892,9 @@ struct lisa_flow {
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     bf16 *wb = nullptr;
     double *mu = nullptr, *L = nullptr, *cov = nullptr, *loss = nullptr;
+    uint4 *act = nullptr;      // weight-gradient operands, bias sums and losses of a chunk's k steps
+    float *bias = nullptr;
+    double *lossp = nullptr;
     int loss_cap = 0, last_iters = 0;
     float *h_grad = nullptr;
     std::string err;
@@ -832,16 +922,14 @@ lisa_status fcuda(lisa_flow_t *f, cudaError_t e, const char *what) {
 FlowView view(const lisa_flow_t *f) { return {f->w, f->wb, f->mu, f->L}; }
 
 cudaError_t set_smem_limits() {
-    cudaError_t e = cudaFuncSetAttribute(flow_eval_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, eval_smem());
+    cudaError_t e = cudaFuncSetAttribute(flow_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, train_smem());
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(flow_propose_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, eval_smem());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(flow_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, train_smem());
+        e = cudaFuncSetAttribute(flow_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, update_smem());
     return e;
 }
 
 lisa_status pack(lisa_flow_t *f, cudaStream_t s) {
-    pack_kernel<<<(FC * BC + 255) / 256, 256, 0, s>>>(f->w, f->wb);
+    pack_kernel<<<(NP + 255) / 256, 256, 0, s>>>(f->w, f->wb);
     FCK(cudaGetLastError(), "pack kernel launch");
     return LISA_OK;
 }
@@ -859,36 +947,44 @@ lisa_status train_iters(lisa_flow_t *f, const double *d_data, int64_t n, int ite
                         double lr, uint64_t seed, uint32_t round, cudaStream_t s, int random_rows) {
     lisa_status st = ensure_loss(f, iters);
     if (st != LISA_OK) return st;
-    FCK(cudaMemsetAsync(f->loss, 0, sizeof(double) * iters, s), "cudaMemsetAsync");
-    for (int it = 0; it < iters; it++) {
-        FCK(cudaMemsetAsync(f->g, 0, sizeof(float) * NP, s), "cudaMemsetAsync");
-        TrainArgs a;
-        a.w = f->w;
-        a.wb = f->wb;
-        a.grad = f->g;
-        a.mu = f->mu;
-        a.L = f->L;
-        a.data = d_data;
-        a.n = n;
-        a.batch = batch;
-        a.k0 = (uint32_t)seed;
-        a.k1 = (uint32_t)(seed >> 32);
-        a.round = round;
-        a.iter = (uint32_t)it;
-        a.random_rows = random_rows;
-        a.loss = f->loss + it;
-        flow_train_kernel<<<batch / TS, NTH, train_smem(), s>>>(a);
-        FCK(cudaGetLastError(), "flow training kernel launch");
-        if (lr > 0.0) {
-            const int t = it + 1;
-            adam_kernel<<<(NP + 255) / 256, 256, 0, s>>>(f->w, f->g, f->m, f->v, NP, (float)lr,
-                                                         (float)(1.0 - std::pow(0.9, t)),
-                                                         (float)(1.0 - std::pow(0.999, t)));
-            FCK(cudaGetLastError(), "Adam kernel launch");
-            st = pack(f, s);
-            if (st != LISA_OK) return st;
+    for (int it = 0; it < iters; it++)
+        for (int row0 = 0; row0 < batch; row0 += kChunkSteps * TS) {
+            const int steps = std::min(kChunkSteps, (batch - row0) / TS), t = it + 1;
+            TrainArgs a;
+            a.f = view(f);
+            a.data = d_data;
+            a.n = n;
+            a.batch = batch;
+            a.row0 = row0;
+            a.k0 = (uint32_t)seed;
+            a.k1 = (uint32_t)(seed >> 32);
+            a.round = round;
+            a.iter = (uint32_t)it;
+            a.random_rows = random_rows;
+            a.act = f->act;
+            a.bias = f->bias;
+            a.lossp = f->lossp;
+            flow_train_kernel<<<steps, NTH, train_smem(), s>>>(a);
+            FCK(cudaGetLastError(), "flow training kernel launch");
+            UpdateArgs u;
+            u.act = f->act;
+            u.bias = f->bias;
+            u.lossp = f->lossp;
+            u.steps = steps;
+            u.w = f->w;
+            u.g = f->g;
+            u.m = f->m;
+            u.v = f->v;
+            u.wb = f->wb;
+            u.loss = f->loss + it;
+            u.first = row0 == 0;
+            u.adam = lr > 0.0 && row0 + steps * TS == batch;
+            u.lr = (float)lr;
+            u.c1 = (float)(1.0 - std::pow(0.9, t));
+            u.c2 = (float)(1.0 - std::pow(0.999, t));
+            flow_update_kernel<<<dim3(kJobs, FC), NTH, update_smem(), s>>>(u);
+            FCK(cudaGetLastError(), "flow update kernel launch");
         }
-    }
     f->last_iters = iters;
     return LISA_OK;
 }
@@ -898,7 +994,7 @@ lisa_status train_iters(lisa_flow_t *f, const double *d_data, int64_t n, int ite
 namespace lisa_flowint {
 
 cudaError_t launch_flow_propose(lisa_flow_t *f, const FStep &a, cudaStream_t s) {
-    flow_propose_kernel<<<(a.W + TS - 1) / TS, NTH, eval_smem(), s>>>(view(f), a);
+    flow_propose_kernel<<<(a.W + TS - 1) / TS, NTH, 0, s>>>(view(f), a);
     return cudaGetLastError();
 }
 
@@ -952,6 +1048,10 @@ lisa_status lisa_flow_create(uint64_t seed, lisa_flow_t **out) {
         if (e == cudaSuccess) e = cudaMalloc(&f->m, sizeof(float) * NP);
         if (e == cudaSuccess) e = cudaMalloc(&f->v, sizeof(float) * NP);
         if (e == cudaSuccess) e = cudaMalloc(&f->wb, sizeof(bf16) * FC * BC);
+        if (e == cudaSuccess) e = cudaMemset(f->wb, 0, sizeof(bf16) * FC * BC);  // the padding
+        if (e == cudaSuccess) e = cudaMalloc(&f->act, sizeof(uint4) * 32 * kUnits * FC * kChunkSteps);
+        if (e == cudaSuccess) e = cudaMalloc(&f->bias, sizeof(float) * kBias * FC * kChunkSteps);
+        if (e == cudaSuccess) e = cudaMalloc(&f->lossp, sizeof(double) * kChunkSteps);
         if (e == cudaSuccess) e = cudaMalloc(&f->mu, sizeof(double) * FD);
         if (e == cudaSuccess) e = cudaMalloc(&f->L, sizeof(double) * FD * FD);
         if (e == cudaSuccess) e = cudaMalloc(&f->cov, sizeof(double) * FD * FD);
@@ -995,7 +1095,8 @@ void lisa_flow_destroy(lisa_flow_t *f) {
     cudaSetDevice(f->device);
     cudaDeviceSynchronize();
     for (void *p : {(void *)f->w, (void *)f->g, (void *)f->m, (void *)f->v, (void *)f->wb,
-                    (void *)f->mu, (void *)f->L, (void *)f->cov, (void *)f->loss})
+                    (void *)f->mu, (void *)f->L, (void *)f->cov, (void *)f->loss, (void *)f->act,
+                    (void *)f->bias, (void *)f->lossp})
         if (p) cudaFree(p);
     if (f->h_grad) cudaFreeHost(f->h_grad);
     delete f;
@@ -1057,7 +1158,7 @@ static lisa_status eval(lisa_flow_t *f, const double *in, int n, int gen, double
     if (!in || !logq || n < 0 || (gen && !out)) return ffail(f, LISA_ERR_ARG, "NULL pointer or n < 0");
     if (n == 0) return LISA_OK;
     FCK(cudaSetDevice(f->device), "cudaSetDevice");
-    flow_eval_kernel<<<(n + TS - 1) / TS, NTH, eval_smem(), (cudaStream_t)stream>>>(view(f), in, n, gen, out, logq);
+    flow_eval_kernel<<<(n + TS - 1) / TS, NTH, 0, (cudaStream_t)stream>>>(view(f), in, n, gen, out, logq);
     FCK(cudaGetLastError(), "flow kernel launch");
     return LISA_OK;
 }
@@ -1075,7 +1176,7 @@ lisa_status lisa_flow_generate(lisa_flow_t *f, const double *d_z, int n, double 
 lisa_status lisa_flow_gradients(lisa_flow_t *f, const double *d_x, int n, float *grad,
                                 double *loss, void *stream) {
     if (!f) return LISA_ERR_ARG;
-    if (!d_x || n < TS || n % TS) return ffail(f, LISA_ERR_ARG, "n must be a positive multiple of 64");
+    if (!d_x || n < kBatchUnit || n % kBatchUnit) return ffail(f, LISA_ERR_ARG, "n must be a positive multiple of 64");
     FCK(cudaSetDevice(f->device), "cudaSetDevice");
     cudaStream_t s = (cudaStream_t)stream;
     lisa_status st = train_iters(f, d_x, n, 1, n, 0.0, 0, 0, s, 0);
@@ -1093,7 +1194,7 @@ lisa_status lisa_flow_train(lisa_flow_t *f, const double *d_data, int64_t n, int
                             int batch, double lr, uint64_t seed, uint32_t round, double *loss,
                             void *stream) {
     if (!f) return LISA_ERR_ARG;
-    if (!d_data || n < 2 || iters < 1 || batch < TS || batch % TS || !(lr > 0.0))
+    if (!d_data || n < 2 || iters < 1 || batch < kBatchUnit || batch % kBatchUnit || !(lr > 0.0))
         return ffail(f, LISA_ERR_ARG, "need data (n >= 2), iters >= 1, batch a multiple of 64, lr > 0");
     FCK(cudaSetDevice(f->device), "cudaSetDevice");
     cudaStream_t s = (cudaStream_t)stream;
