@@ -129,7 +129,7 @@ __device__ inline bool make_source_core(const double *th, double t0, Source &s) 
     const double eta = s.eta;
     s.k128 = 1.0 / (128.0 * eta);
     s.m2pi = s.M / kTwoPi;
-    s.amp0 = sqrt(2.0 * eta / 3.0) * pow(kPi, -1.0 / 6.0) * s.M * s.M / s.dist;
+    s.amp0 = sqrt(2.0 * eta / 3.0) * 0.82630748711075811083 * s.M * s.M / s.dist;
     s.al2 = -323.0 / 224.0 + 451.0 / 168.0 * eta;
     s.al3 = (27.0 / 8.0 - 11.0 / 6.0 * eta) * s.chis + 27.0 / 8.0 * s.dlt * s.chia;
     s.ps2 = 3715.0 / 756.0 + 55.0 / 9.0 * eta;
@@ -139,7 +139,7 @@ __device__ inline bool make_source_core(const double *th, double t0, Source &s) 
                 0.3 * s.chieff;
     af = fmin(0.99, fmax(-0.99, af));
     const double mf = 1.0 - 0.0572 * eta - 0.498 * eta * eta;
-    s.xrd = (1.0 - 0.63 * pow(1.0 - af, 0.3)) / (2.0 * kPi * mf);
+    s.xrd = (1.0 - 0.63 * exp(0.3 * log(1.0 - af))) / (2.0 * kPi * mf);
     // merger-ringdown continuation with matching value, slope and curvature
     const PhaseSet j = inspiral_phase(s, kXJoin);
     s.phj = j.p;
@@ -276,9 +276,9 @@ __device__ inline void mode_all(const Source &s, const Mode &md, double f, doubl
     amp = amp_ratio(s, md, v) * a22;
 }
 
-// -2Y_lm(iota, phi) for l = 2..4 in closed form; (l, m) with |m| from the mode table
-__device__ inline cplx ylm_m2(int l, int m, double th, double ph) {
-    const double c = cos(0.5 * th), s = sin(0.5 * th), ct = cos(th);
+// |-2Y_lm| with sign for l = 2..4 in closed form, (l, m) with |m| from the mode table, from
+// c = cos(iota / 2), s = sin(iota / 2), ct = cos(iota)
+__device__ inline double ylm_value(int l, int m, double c, double s, double ct) {
     const double c2 = c * c, s2 = s * s;
     double v = 0.0;
     if (l == 2) {
@@ -297,20 +297,27 @@ __device__ inline cplx ylm_m2(int l, int m, double th, double ph) {
         if (m == 3) v = -3.0 * sqrt(7.0 / (2.0 * kPi)) * c2 * c2 * c * s * (2.0 * ct - 1.0);
         if (m == -3) v = 3.0 * sqrt(7.0 / (2.0 * kPi)) * s2 * s2 * s * c * (2.0 * ct + 1.0);
     }
-    return {v * cos(m * ph), v * sin(m * ph)};
+    return v;
 }
 
 // Polarisation weights of the positive-frequency content of mode (l, m):
 // h+ = Kp h_lm and hx = Kc h_lm, from h = h+ - i hx = sum h_lm Y_lm and the
 // aligned-spin symmetry h_{l,-m}(f) = (-1)^l h*_lm(-f).
-__device__ inline void pol_weights(const Source &s, const Mode &md, cplx &kp, cplx &kc) {
-    const cplx yp = ylm_m2(md.l, md.m, s.iota, s.phiref);
-    const cplx ym = ylm_m2(md.l, -md.m, s.iota, s.phiref);
+// (c, s, ct as in ylm_value; cm, sm: cos and sin of m phi_ref)
+__device__ inline void pol_weights(const Mode &md, double c, double s, double ct, double cm, double sm,
+                                   cplx &kp, cplx &kc) {
+    const double vp = ylm_value(md.l, md.m, c, s, ct), vm = ylm_value(md.l, -md.m, c, s, ct);
+    const cplx yp = {vp * cm, vp * sm}, ym = {vm * cm, -vm * sm};
     const double sg = (md.l & 1) ? -1.0 : 1.0;
     const cplx ypc = {sg * yp.re, -sg * yp.im};  // (-1)^l conj(Y_lm)
     kp = {0.5 * (ym.re + ypc.re), 0.5 * (ym.im + ypc.im)};
     const cplx d = {ym.re - ypc.re, ym.im - ypc.im};
     kc = {-0.5 * d.im, 0.5 * d.re};  // (i/2) d
+}
+
+__device__ inline void pol_weights(const Source &src, const Mode &md, cplx &kp, cplx &kc) {
+    pol_weights(md, cos(0.5 * src.iota), sin(0.5 * src.iota), cos(src.iota), cos(md.m * src.phiref),
+                sin(md.m * src.phiref), kp, kc);
 }
 
 // ---------------------------------------------------------------- orbit and response

@@ -3,13 +3,16 @@
 // (the cut where t_lm(f) < 0 and the ringdown cut) with its integer dense-bin range, and
 // the coefficients of the response in the constellation's orbital harmonics.
 //
-// One warp per walker.  Both roots (the peak, and the frequency where the signal starts,
-// which is one mapped frequency x = 2 M f / m for all modes) are bracketed by two rounds
-// of 31 points, one per lane (five bisections a round), and finished by Newton steps.
-// What bounds it is the latency of one evaluation after another (about 2 us each: cube
-// root, divisions), so their number is what counts: about 16 against 94 of two bisections
-// to 1e-14 in one thread.  Source and knots together, one walker, one mode, 256 knots: 281 ->
-// 98 us.
+// One warp per walker.  What bounds it is the latency of FP64 operations one after another (about
+// 40 clocks each), so the chain is kept short:
+//  * both roots (the peak, and the frequency where the signal starts, which is one mapped
+//    frequency x = 2 M f / m for all modes) are bracketed in FP32, 31 points a round, one per
+//    lane, and finished by Newton steps in FP64 inside the whole range (quadratic: the step
+//    that moves x by less than 1e-8 leaves 1e-16);
+//  * what is needed at several places or angles is evaluated in one pass, a lane for each: the
+//    ends of the peak's range, phase and slope at the band's ends and the peak, sines and cosines.
+// One walker, one mode: 80 -> @@ us (two rounds of 31 points and up to six Newton steps in FP64, all
+// else one after another).
 #include "fixed.cuh"
 #include "kernels.h"
 #include "model.cuh"
@@ -34,22 +37,37 @@ __device__ __forceinline__ int bisect32(unsigned above) {
     return pos;
 }
 
+// the interval among 31 interior points of [lo, hi], equally spaced in the logarithm, that holds
+// the root of f (above(x): the root lies above x), `rounds` times
+template <class F>
+__device__ __forceinline__ float bracket32(float lo, float hi, int rounds, int lane, F above) {
+    float l0 = log2f(lo), st = log2f(hi) - l0;
+    for (int r = 0; r < rounds; r++) {
+        st *= 1.0f / 32.0f;
+        const int p = bisect32(__ballot_sync(0xffffffffu, above(exp2f(fmaf(st, (float)lane, l0)))));
+        l0 = fmaf(st, (float)p, l0);
+    }
+    return exp2f(l0 + 0.5f * st);
+}
+
 // peak of f^2 A_22 (t_coal is reached there, Sec. II): the zero of its log-derivative over
 // [x_RD / 4, 2 x_RD], or the end of that range that it lies beyond
 __device__ double find_peak_warp(const Source &s, int lane) {
     double lo = 0.25 * s.xrd, hi = 2.0 * s.xrd;
-    if (peak_equation(s, lo) <= 0.0) return lo;
-    if (peak_equation(s, hi) >= 0.0) return hi;
-    for (int round = 0; round < 2; round++) {
-        const double st = (hi - lo) * (1.0 / 32.0);
-        const unsigned up = __ballot_sync(0xffffffffu, peak_equation(s, lo + st * lane) > 0.0);
-        const int p = bisect32(up);
-        hi = (p == 31) ? hi : lo + st * (p + 1);
-        lo = lo + st * p;
-    }
-    double x = 0.5 * (lo + hi);
-    for (int it = 0; it < 6; it++) {
-        const double v = cbrt(kPi * x), r = x / s.xrd, r2 = r * r, r6 = r2 * r2 * r2;
+    const double ge = peak_equation(s, lane == 0 ? lo : hi);
+    const double gl = __shfl_sync(0xffffffffu, ge, 0), gh = __shfl_sync(0xffffffffu, ge, 1);
+    if (gl <= 0.0) return lo;
+    if (gh >= 0.0) return hi;
+    const float al2 = (float)s.al2, al3 = (float)s.al3;
+    // in units of x_RD
+    const float v3 = (float)(kPi * s.xrd);
+    double x = s.xrd * (double)bracket32(0.25f, 2.0f, 3, lane, [&](float r) {
+        const float v = cbrtf(v3 * r), r2 = r * r, r6 = r2 * r2 * r2;
+        return 5.0f / 6.0f + v * v * fmaf(al3, v, (2.0f / 3.0f) * al2) > 6.0f * r6 / (1.0f + r6);
+    });
+    const double ixrd = 1.0 / s.xrd;
+    for (int it = 0; it < 100; it++) {
+        const double v = cbrt(kPi * x), r = x * ixrd, r2 = r * r, r6 = r2 * r2 * r2;
         const double q2 = s.al2 * v * v, q3 = s.al3 * v * v * v, den = 1.0 / (1.0 + r6);
         const double g = 5.0 / 6.0 + (2.0 / 3.0) * q2 + q3 - 6.0 * r6 * den;
         const double gx = (4.0 / 9.0) * q2 + q3 - 36.0 * r6 * den * den;  // x dg/dx
@@ -61,40 +79,51 @@ __device__ double find_peak_warp(const Source &s, int lane) {
         if (!(nx >= lo && nx <= hi)) nx = 0.5 * (lo + hi);
         const double dx = fabs(nx - x);
         x = nx;
-        if (dx <= 1e-15 * x) break;
+        if (dx <= 1e-8 * x) break;
     }
     return x;
 }
 
-// t_22 at the mapped frequency x
-__device__ __forceinline__ double time_at(const Source &s, double x) {
-    return s.tc - s.M / kTwoPi * (raw_slope(s, x) - s.dphpk);
+// phase and slope of the (2,2) mode before its alignment, and the slope's derivative
+__device__ __forceinline__ PhaseSet raw_set(const Source &s, double x) {
+    PhaseSet r;
+    if (x <= kXJoin) {
+        r = inspiral_phase(s, x);
+    } else {
+        const double ix = 1.0 / x;
+        r.p = s.phj + s.c1 * (x - kXJoin) - s.c2 * (ix - 1.0 / kXJoin);
+        r.dp = s.c1 + s.c2 * (ix * ix);
+        r.d2p = -2.0 * s.c2 * (ix * ix * ix);
+    }
+    return r;
 }
 
 // mapped frequency where t_22 = 0, inside [xa, xb] with t(xa) < 0 <= t(xb): t rises with x
 __device__ double find_start_warp(const Source &s, double xa, double xb, int lane) {
     double lo = xa, hi = xb;
-    for (int round = 0; round < 2; round++) {
-        const double st = log(hi / lo) * (1.0 / 32.0);
-        const double x = lo * exp(st * lane);
-        const int p = bisect32(__ballot_sync(0xffffffffu, time_at(s, x) < 0.0));
-        const double l2 = __shfl_sync(0xffffffffu, x, p), h2 = __shfl_sync(0xffffffffu, x, (p + 1) & 31);
-        lo = p == 0 ? lo : l2;
-        hi = p == 31 ? hi : h2;
-    }
-    double x = 0.5 * (lo + hi);
-    for (int it = 0; it < 8; it++) {
-        const double t = time_at(s, x);
-        const double d2 = x <= kXJoin ? inspiral_phase(s, x).d2p : -2.0 * s.c2 / (x * x * x);
+    const double target = s.tc * (kTwoPi / s.M) + s.dphpk;  // the slope where t = 0
+    const float want = (float)target, k = (float)s.k128, ps2 = (float)s.ps2, ps3 = (float)s.ps3;
+    const float c1 = (float)s.c1, c2 = (float)s.c2;
+    double x = (double)bracket32((float)xa, (float)xb, 4, lane, [&](float y) {
+        const float iv = 1.0f / cbrtf((float)kPi * y), iv2 = iv * iv;
+        const float dp = y <= (float)kXJoin
+                             ? k / y * iv2 * fmaf(iv, fmaf(5.0f, iv2, 3.0f * ps2), 2.0f * ps3)
+                             : c1 + c2 / (y * y);
+        return dp > want;
+    });
+    x = fmin(hi, fmax(lo, x));
+    for (int it = 0; it < 100; it++) {
+        const PhaseSet r = raw_set(s, x);
+        const double t = target - r.dp;  // 2 pi t / M
         if (t < 0.0)
             lo = fmax(lo, x);
         else
             hi = fmin(hi, x);
-        double nx = x + t / (s.M / kTwoPi * d2);
+        double nx = x + t / r.d2p;
         if (!(nx >= lo && nx <= hi)) nx = 0.5 * (lo + hi);
         const double dx = fabs(nx - x);
         x = nx;
-        if (dx <= 1e-15 * x) break;
+        if (dx <= 1e-8 * x) break;
     }
     return x;
 }
@@ -127,24 +156,32 @@ __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
     Source src;
     const bool ok = make_source_core(b.params + (size_t)w * kNPar, d.t0, src);
     const double fmn = d.f0, fmx = bin_freq(d.f0, d.df, d.N - 1);
-    if (ok) set_peak(src, find_peak_warp(src, lane));
     // lanes 0 .. L-1: one mode each
     const bool mode = lane < d.L;
-    Mode md = {2, 2};
+    Mode md = {2, 2};  // of lane % 8
 #pragma unroll
     for (int i = 0; i < kMaxModes; i++)
-        if (i == lane && i < d.L) md = {d.ml[i], d.mm[i]};
+        if (i == (lane & 7) && i < d.L) md = {d.ml[i], d.mm[i]};
     bool act = false, whole = false;
     double lo = 0.0, hi = 0.0;
-    if (ok && mode) {
+    if (ok) {
+        const double xpk = find_peak_warp(src, lane);
         const double fcut = 0.5 * md.m * kXCut / src.M;
         hi = fmx < fcut ? fmx : fcut;
-        act = hi > fmn * (1.0 + 1e-12);
+        // phase and slope at the first bin (lanes 0 .. 7), at the modes' ends and at the peak
+        const PhaseSet at =
+            raw_set(src, lane < 8 ? mapped_x(src, md, fmn) : lane < 16 ? mapped_x(src, md, hi) : xpk);
+        src.xpk = xpk;
+        src.phpk = __shfl_sync(0xffffffffu, at.p, 16);
+        src.dphpk = __shfl_sync(0xffffffffu, at.dp, 16);
+        const double t = src.tc - src.M / kTwoPi * (at.dp - src.dphpk);  // mode_time
+        const double tend = __shfl_sync(0xffffffffu, t, (lane & 7) + 8);
+        act = mode && hi > fmn * (1.0 + 1e-12);
         if (act) {
-            whole = mode_time(src, md, fmn) >= 0.0;
+            whole = t >= 0.0;
             if (whole)
                 lo = fmn;
-            else if (mode_time(src, md, hi) < 0.0)
+            else if (tend < 0.0)
                 act = false;  // the mode ends before the observation starts
         }
     }
@@ -183,12 +220,26 @@ __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
         b.xpk[w] = ok ? src.xpk : 0.0;
     }
     if (!ok) return;
+    // sines and cosines: lanes 0 .. 8 one angle each, lanes 2 .. 5 are m = 1 .. 4
+    double sn, cs;
+    {
+        double angle = src.phiref * (double)(lane - 1);
+        if (lane == 0) angle = 0.5 * src.iota;
+        if (lane == 1) angle = src.iota;
+        if (lane == 6) angle = 2.0 * src.psi;
+        if (lane == 7) angle = src.lam;
+        if (lane >= 8) angle = src.beta;
+        sincos(angle, &sn, &cs);
+    }
+    auto sine = [&](int i) { return __shfl_sync(0xffffffffu, sn, i); };
+    auto cosine = [&](int i) { return __shfl_sync(0xffffffffu, cs, i); };
+    const double shi = sine(0), chi = cosine(0), ci = cosine(1), s2 = sine(6), c2 = cosine(6);
+    const double sl = sine(7), cl = cosine(7), sb = sine(8), cb = cosine(8);
+    const double sm = sine(md.m + 1), cm = cosine(md.m + 1);
     if (act) {  // this lane's mode
         ModeConst c;
         cplx kp, kc;
-        pol_weights(src, md, kp, kc);
-        double s2, c2;
-        sincos(2.0 * src.psi, &s2, &c2);
+        pol_weights(md, chi, shi, ci, cm, sm, kp, kc);
         c.are = kp.re * c2 - kc.re * s2;
         c.aim = kp.im * c2 - kc.im * s2;
         c.bre = 2.0 * (kp.re * s2 + kc.re * c2);
@@ -218,9 +269,6 @@ __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
         c.al2 = src.al2;
         c.al3 = src.al3;
         c.ixrd = 1.0 / src.xrd;
-        double sl, cl, sb, cb;
-        sincos(src.lam, &sl, &cl);
-        sincos(src.beta, &sb, &cb);
         const double u[3] = {sl, -cl, 0.0}, p[3] = {-sb * cl, -sb * sl, cb};
         const double k[3] = {-cb * cl, -cb * sl, -sb};
         const double h = 0.8660254037844386467637;  // cos, sin of 0, 2 pi / 3, 4 pi / 3
