@@ -52,13 +52,23 @@ __device__ __forceinline__ void turns_fixed(double x, unsigned long long &hi,
     double r = fma(-k, kTwoPiHi, x);
     r = fma(-k, kTwoPiMid, r);
     r = fma(-k, kTwoPiLo, r);
-    double fr = r * kInvTwoPi;  // in about [-0.5, 0.5]
-    if (fr >= 0.5) fr -= 1.0;
-    if (fr < -0.5) fr += 1.0;
-    const double t = ldexp(fr, 64);  // exact scaling
-    const double ft = floor(t);      // exact
-    hi = (unsigned long long)(long long)ft;
-    lo = (unsigned long long)ldexp(t - ft, 64);  // t - ft in [0, 1), exact
+    const i64 b = double_bits(r * kInvTwoPi);  // in about [-0.5, 0.5]: m 2^sh units of 2^-64
+    const int e = (int)((b >> 52) & 0x7ff), sh = e - 1075 + 64;
+    const unsigned long long m = (b & 0xfffffffffffffLL) | 0x10000000000000LL;
+    unsigned long long h = 0, l = 0;
+    if (sh >= 0) {
+        h = m << sh;
+    } else if (sh > -117 && e != 0) {
+        const int k = -sh;
+        h = k < 64 ? m >> k : 0;
+        l = k < 64 ? m << (64 - k) : m >> (k - 64);
+    }
+    if (b < 0) {  // two's complement of both words
+        l = 0ull - l;
+        h = ~h + (l == 0);
+    }
+    hi = h;
+    lo = l;
 }
 
 __device__ __forceinline__ double bin_freq_s(double f0, double df, int j) {
