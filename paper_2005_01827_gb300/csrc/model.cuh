@@ -76,11 +76,11 @@ __device__ inline PhaseSet inspiral_phase(const Source &s, double x) {
     const double v = cbrt(kPi * x);
     const double iv = 1.0 / v;
     const double iv2 = iv * iv, iv3 = iv2 * iv, iv5 = iv3 * iv2;
-    const double k = 1.0 / (128.0 * s.eta);
+    const double k = s.k128, kx = k * (kPi * iv3), kxx = kx * (kPi * iv3);  // k / x, k / x^2
     PhaseSet r;
     r.p = -3.0 * k * (iv5 + s.ps2 * iv3 + s.ps3 * iv2);
-    r.dp = k / x * (5.0 * iv5 + 3.0 * s.ps2 * iv3 + 2.0 * s.ps3 * iv2);
-    r.d2p = -k / (x * x) * ((40.0 / 3.0) * iv5 + 6.0 * s.ps2 * iv3 + (10.0 / 3.0) * s.ps3 * iv2);
+    r.dp = kx * (5.0 * iv5 + 3.0 * s.ps2 * iv3 + 2.0 * s.ps3 * iv2);
+    r.d2p = -kxx * ((40.0 / 3.0) * iv5 + 6.0 * s.ps2 * iv3 + (10.0 / 3.0) * s.ps3 * iv2);
     return r;
 }
 
@@ -112,14 +112,15 @@ __device__ inline bool make_source_core(const double *th, double t0, Source &s) 
     if (!(mt > 0.0) || !(q > 0.0) || !(q <= 1.0) || !(fabs(a1) <= 0.99) ||
         !(fabs(a2) <= 0.99) || !(dl > 0.0) || !isfinite(t0))
         return false;
-    const double opq = 1.0 + q;
+    // few divisions: each is a chain of a dozen operations, and so is one walker's time
+    const double opq = 1.0 + q, iopq = 1.0 / opq;
     s.M = mt * kMsunS;
-    s.eta = q / (opq * opq);
-    s.dlt = (1.0 - q) / opq;
+    s.eta = q * iopq * iopq;
+    s.dlt = (1.0 - q) * iopq;
     s.chis = 0.5 * (a1 + a2);
     s.chia = 0.5 * (a1 - a2);
-    s.chieff = (a1 + q * a2) / opq;
-    s.dist = dl * kGpcM / kClight;
+    s.chieff = (a1 + q * a2) * iopq;
+    s.dist = dl * (kGpcM / kClight);
     s.phiref = th[5];
     s.iota = th[6];
     s.lam = th[7];
@@ -127,8 +128,8 @@ __device__ inline bool make_source_core(const double *th, double t0, Source &s) 
     s.psi = th[9];
     s.tc = th[10] + t0;
     const double eta = s.eta;
-    s.k128 = 1.0 / (128.0 * eta);
-    s.m2pi = s.M / kTwoPi;
+    s.k128 = opq * opq / (128.0 * q);
+    s.m2pi = s.M * (1.0 / kTwoPi);
     s.amp0 = sqrt(2.0 * eta / 3.0) * 0.82630748711075811083 * s.M * s.M / s.dist;
     s.al2 = -323.0 / 224.0 + 451.0 / 168.0 * eta;
     s.al3 = (27.0 / 8.0 - 11.0 / 6.0 * eta) * s.chis + 27.0 / 8.0 * s.dlt * s.chia;
@@ -278,26 +279,25 @@ __device__ inline void mode_all(const Source &s, const Mode &md, double f, doubl
 
 // |-2Y_lm| with sign for l = 2..4 in closed form, (l, m) with |m| from the mode table, from
 // c = cos(iota / 2), s = sin(iota / 2), ct = cos(iota)
+// (one formula for all modes, so that the lanes of a warp can have one each: with (A, B) =
+// (c, s), or (s, c) for m < 0, N A^2 times A^2, A^3 B, A^4 B^2 or A B and a linear function of ct)
 __device__ inline double ylm_value(int l, int m, double c, double s, double ct) {
-    const double c2 = c * c, s2 = s * s;
-    double v = 0.0;
-    if (l == 2) {
-        if (m == 2) v = sqrt(5.0 / (4.0 * kPi)) * c2 * c2;
-        if (m == -2) v = sqrt(5.0 / (4.0 * kPi)) * s2 * s2;
-        if (m == 1) v = sqrt(5.0 / kPi) * c2 * c * s;
-        if (m == -1) v = sqrt(5.0 / kPi) * s2 * s * c;
-    } else if (l == 3) {
-        if (m == 3) v = -sqrt(21.0 / (2.0 * kPi)) * c2 * c2 * c * s;
-        if (m == -3) v = sqrt(21.0 / (2.0 * kPi)) * s2 * s2 * s * c;
-        if (m == 2) v = 0.5 * sqrt(7.0 / kPi) * c2 * c2 * (3.0 * ct - 2.0);
-        if (m == -2) v = 0.5 * sqrt(7.0 / kPi) * s2 * s2 * (3.0 * ct + 2.0);
-    } else if (l == 4) {
-        if (m == 4) v = 3.0 * sqrt(7.0 / kPi) * c2 * c2 * c2 * s2;
-        if (m == -4) v = 3.0 * sqrt(7.0 / kPi) * s2 * s2 * s2 * c2;
-        if (m == 3) v = -3.0 * sqrt(7.0 / (2.0 * kPi)) * c2 * c2 * c * s * (2.0 * ct - 1.0);
-        if (m == -3) v = 3.0 * sqrt(7.0 / (2.0 * kPi)) * s2 * s2 * s * c * (2.0 * ct + 1.0);
-    }
-    return v;
+    const int id = mode_index(l, m < 0 ? -m : m);
+    const double A = m < 0 ? s : c, B = m < 0 ? c : s, sg = m < 0 ? 1.0 : -1.0;
+    const double A2 = A * A, AB = A * B;
+    double n = 0.0, f = 1.0, g = A2;  // N, the linear factor, and the power of A beyond A^2 with B
+    if (id == 0) n = sqrt(5.0 / (4.0 * kPi));
+    if (id == 1) n = sg * sqrt(21.0 / (2.0 * kPi));
+    if (id == 2) n = 3.0 * sqrt(7.0 / kPi);
+    if (id == 3) n = sqrt(5.0 / kPi);
+    if (id == 4) n = 0.5 * sqrt(7.0 / kPi);
+    if (id == 5) n = sg * 3.0 * sqrt(7.0 / (2.0 * kPi));
+    if (id == 4) f = fma(3.0, ct, 2.0 * sg);
+    if (id == 5) f = fma(2.0, ct, sg);
+    if (id == 1 || id == 5) g = A2 * AB;
+    if (id == 2) g = A2 * (AB * AB);
+    if (id == 3) g = AB;
+    return n * A2 * g * f;
 }
 
 // Polarisation weights of the positive-frequency content of mode (l, m):

@@ -11,7 +11,7 @@
 //    that moves x by less than 1e-8 leaves 1e-16);
 //  * what is needed at several places or angles is evaluated in one pass, a lane for each: the
 //    ends of the peak's range, phase and slope at the band's ends and the peak, sines and cosines.
-// One walker, one mode: 80 -> @@ us (two rounds of 31 points and up to six Newton steps in FP64, all
+// One walker, one mode: 80 -> 29 us (98 -> 38 with cold caches; two rounds of 31 points and up to six Newton steps in FP64, all
 // else one after another).
 #include "fixed.cuh"
 #include "kernels.h"
@@ -52,20 +52,23 @@ __device__ __forceinline__ float bracket32(float lo, float hi, int rounds, int l
 
 // peak of f^2 A_22 (t_coal is reached there, Sec. II): the zero of its log-derivative over
 // [x_RD / 4, 2 x_RD], or the end of that range that it lies beyond
-__device__ double find_peak_warp(const Source &s, int lane) {
+__device__ double find_peak_warp(const Source &s, double ixrd, int lane) {
     double lo = 0.25 * s.xrd, hi = 2.0 * s.xrd;
-    const double ge = peak_equation(s, lane == 0 ? lo : hi);
-    const double gl = __shfl_sync(0xffffffffu, ge, 0), gh = __shfl_sync(0xffffffffu, ge, 1);
-    if (gl <= 0.0) return lo;
-    if (gh >= 0.0) return hi;
     const float al2 = (float)s.al2, al3 = (float)s.al3;
     // in units of x_RD
     const float v3 = (float)(kPi * s.xrd);
-    double x = s.xrd * (double)bracket32(0.25f, 2.0f, 3, lane, [&](float r) {
+    auto equation = [&](float r) {
         const float v = cbrtf(v3 * r), r2 = r * r, r6 = r2 * r2 * r2;
-        return 5.0f / 6.0f + v * v * fmaf(al3, v, (2.0f / 3.0f) * al2) > 6.0f * r6 / (1.0f + r6);
-    });
-    const double ixrd = 1.0 / s.xrd;
+        return 5.0f / 6.0f + v * v * fmaf(al3, v, (2.0f / 3.0f) * al2) - 6.0f * r6 / (1.0f + r6);
+    };
+    // the ends in FP32, and in FP64 where those could have the wrong sign
+    if (!(equation(0.25f) > 1e-3f && equation(2.0f) < -1e-3f)) {
+        const double ge = peak_equation(s, lane == 0 ? lo : hi);
+        const double gl = __shfl_sync(0xffffffffu, ge, 0), gh = __shfl_sync(0xffffffffu, ge, 1);
+        if (gl <= 0.0) return lo;
+        if (gh >= 0.0) return hi;
+    }
+    double x = s.xrd * (double)bracket32(0.25f, 2.0f, 4, lane, [&](float r) { return equation(r) > 0.0f; });
     for (int it = 0; it < 100; it++) {
         const double v = cbrt(kPi * x), r = x * ixrd, r2 = r * r, r6 = r2 * r2 * r2;
         const double q2 = s.al2 * v * v, q3 = s.al3 * v * v * v, den = 1.0 / (1.0 + r6);
@@ -75,7 +78,7 @@ __device__ double find_peak_warp(const Source &s, int lane) {
             lo = fmax(lo, x);
         else
             hi = fmin(hi, x);
-        double nx = x - x * g / gx;
+        double nx = fma(-x, g / gx, x);
         if (!(nx >= lo && nx <= hi)) nx = 0.5 * (lo + hi);
         const double dx = fabs(nx - x);
         x = nx;
@@ -99,9 +102,9 @@ __device__ __forceinline__ PhaseSet raw_set(const Source &s, double x) {
 }
 
 // mapped frequency where t_22 = 0, inside [xa, xb] with t(xa) < 0 <= t(xb): t rises with x
-__device__ double find_start_warp(const Source &s, double xa, double xb, int lane) {
+__device__ double find_start_warp(const Source &s, double iM, double xa, double xb, int lane) {
     double lo = xa, hi = xb;
-    const double target = s.tc * (kTwoPi / s.M) + s.dphpk;  // the slope where t = 0
+    const double target = s.tc * (kTwoPi * iM) + s.dphpk;  // the slope where t = 0
     const float want = (float)target, k = (float)s.k128, ps2 = (float)s.ps2, ps3 = (float)s.ps3;
     const float c1 = (float)s.c1, c2 = (float)s.c2;
     double x = (double)bracket32((float)xa, (float)xb, 4, lane, [&](float y) {
@@ -132,12 +135,17 @@ __device__ double find_start_warp(const Source &s, double xa, double xb, int lan
 // v . sum_i g_i q_i / L as {1, cos 2a, sin 2a, cos a, sin a} coefficients, with
 // cb = sum g_i cos b_i and sb = sum g_i sin b_i (b_i = 2 pi i / 3), a the orbital angle
 __device__ __forceinline__ void harmonics(const double v[3], double cb, double sb, double o[5]) {
-    const double p = 1.0 / (4.0 * sqrt(3.0));
+    constexpr double p = 0.14433756729740644113;  // 1 / (4 sqrt 3)
     o[0] = -3.0 * p * (v[0] * cb + v[1] * sb);
     o[1] = p * (v[0] * cb - v[1] * sb);
     o[2] = p * (v[0] * sb + v[1] * cb);
     o[3] = -0.5 * v[2] * cb;
     o[4] = -0.5 * v[2] * sb;
+}
+
+// x / (M f) of a mode's mapped frequency
+__device__ __forceinline__ double md_scale(const Mode &md) {
+    return md.m == 1 ? 2.0 : md.m == 2 ? 1.0 : md.m == 3 ? 2.0 / 3.0 : 0.5;
 }
 
 // One block more than the walkers need writes the phasor table of the FP64 dense kernel.
@@ -163,18 +171,21 @@ __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
     for (int i = 0; i < kMaxModes; i++)
         if (i == (lane & 7) && i < d.L) md = {d.ml[i], d.mm[i]};
     bool act = false, whole = false;
-    double lo = 0.0, hi = 0.0;
+    double lo = 0.0, hi = 0.0, ixrd = 0.0, iM = 0.0, xf = 0.0;  // xf: x / f, this lane's mode
     if (ok) {
-        const double xpk = find_peak_warp(src, lane);
-        const double fcut = 0.5 * md.m * kXCut / src.M;
+        ixrd = 1.0 / src.xrd;
+        iM = 1.0 / src.M;
+        xf = src.M * md_scale(md);
+        const double xpk = find_peak_warp(src, ixrd, lane);
+        const double fcut = 0.5 * md.m * kXCut * iM;
         hi = fmx < fcut ? fmx : fcut;
         // phase and slope at the first bin (lanes 0 .. 7), at the modes' ends and at the peak
         const PhaseSet at =
-            raw_set(src, lane < 8 ? mapped_x(src, md, fmn) : lane < 16 ? mapped_x(src, md, hi) : xpk);
+            raw_set(src, lane < 8 ? xf * fmn : lane < 16 ? xf * hi : xpk);
         src.xpk = xpk;
         src.phpk = __shfl_sync(0xffffffffu, at.p, 16);
         src.dphpk = __shfl_sync(0xffffffffu, at.dp, 16);
-        const double t = src.tc - src.M / kTwoPi * (at.dp - src.dphpk);  // mode_time
+        const double t = src.tc - src.m2pi * (at.dp - src.dphpk);  // mode_time
         const double tend = __shfl_sync(0xffffffffu, t, (lane & 7) + 8);
         act = mode && hi > fmn * (1.0 + 1e-12);
         if (act) {
@@ -188,13 +199,13 @@ __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
     // the modes that start inside the observation share one mapped starting frequency
     const bool inside = act && !whole;
     if (__any_sync(0xffffffffu, inside)) {
-        double xa = inside ? mapped_x(src, md, fmn) : INFINITY, xb = inside ? mapped_x(src, md, hi) : 0.0;
+        double xa = inside ? xf * fmn : INFINITY, xb = inside ? xf * hi : 0.0;
         for (int o = 16; o > 0; o >>= 1) {
             xa = fmin(xa, __shfl_xor_sync(0xffffffffu, xa, o));
             xb = fmax(xb, __shfl_xor_sync(0xffffffffu, xb, o));
         }
-        const double x0 = find_start_warp(src, xa, xb, lane);
-        if (inside) lo = fmin(hi, fmax(fmn, 0.5 * md.m * x0 / src.M));
+        const double x0 = find_start_warp(src, iM, xa, xb, lane);
+        if (inside) lo = fmin(hi, fmax(fmn, 0.5 * md.m * x0 * iM));
     }
     int jl = 0, jh = -1;
     if (act && !(hi > lo * (1.0 + 1e-12))) act = false;
@@ -244,7 +255,7 @@ __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
         c.aim = kp.im * c2 - kc.im * s2;
         c.bre = 2.0 * (kp.re * s2 + kc.re * c2);
         c.bim = 2.0 * (kp.im * s2 + kc.im * c2);
-        c.xf = 2.0 * src.M / md.m;
+        c.xf = xf;
         c.v0 = cbrt(kPi * (c.xf * lo));
         c.x160 = sqrt(c.v0 * kInvCbrtPi);
         c.s6 = log(hi / lo) / (6.0 * (double)(d.K - 1));
@@ -255,39 +266,39 @@ __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
         c.pad = 0;
         b.mconst[(size_t)w * d.L + lane] = c;
     }
+    WalkerConst *c = b.wconst + w;
     if (lane == 0) {
-        WalkerConst c;
-        c.k128 = src.k128;
-        c.ps2 = src.ps2;
-        c.ps3 = src.ps3;
-        c.phj = src.phj - src.c1 * kXJoin + src.c2 / kXJoin;
-        c.c1 = src.c1;
-        c.c2 = src.c2;
-        c.dphpk = src.dphpk;
-        c.tc = src.tc;
-        c.m2pi = src.m2pi;
-        c.al2 = src.al2;
-        c.al3 = src.al3;
-        c.ixrd = 1.0 / src.xrd;
-        const double u[3] = {sl, -cl, 0.0}, p[3] = {-sb * cl, -sb * sl, cb};
-        const double k[3] = {-cb * cl, -cb * sl, -sb};
-        const double h = 0.8660254037844386467637;  // cos, sin of 0, 2 pi / 3, 4 pi / 3
-        // arms 0 -> 1 and 1 -> 2 (differences) and their sums
-        harmonics(k, -1.5, h, c.kn[0]);
-        harmonics(k, 0.0, -2.0 * h, c.kn[1]);
-        harmonics(k, 0.5, h, c.kq[0]);
-        harmonics(k, -1.0, 0.0, c.kq[1]);
-        harmonics(p, -1.5, h, c.wn[0]);
-        harmonics(p, 0.0, -2.0 * h, c.wn[1]);
-        double o[5];
-        harmonics(u, -1.5, h, o);
-        for (int i = 0; i < 3; i++) c.un[0][i] = o[i];
-        harmonics(u, 0.0, -2.0 * h, o);
-        for (int i = 0; i < 3; i++) c.un[1][i] = o[i];
+        c->k128 = src.k128;
+        c->ps2 = src.ps2;
+        c->ps3 = src.ps3;
+        c->phj = src.phj - src.c1 * kXJoin + src.c2 * (1.0 / kXJoin);
+        c->c1 = src.c1;
+        c->c2 = src.c2;
+        c->dphpk = src.dphpk;
+        c->tc = src.tc;
+        c->m2pi = src.m2pi;
+        c->al2 = src.al2;
+        c->al3 = src.al3;
+        c->ixrd = ixrd;
         const double R = kAuM / kClight;
-        c.dx = -kTwoPi * R * k[0];
-        c.dy = -kTwoPi * R * k[1];
-        b.wconst[w] = c;
+        c->dx = kTwoPi * R * (cb * cl);
+        c->dy = kTwoPi * R * (cb * sl);
+    }
+    if (lane < 8) {
+        // lanes 0 .. 7: kn, kq, wn, un, each for arms 0 -> 1 and 1 -> 2 (differences, or sums for kq)
+        const int what = lane >> 1;
+        const bool second = lane & 1;
+        const double h = 0.8660254037844386467637;  // cos, sin of 0, 2 pi / 3, 4 pi / 3
+        double v[3] = {-cb * cl, -cb * sl, -sb};  // k
+        if (what == 2) v[0] = -sb * cl, v[1] = -sb * sl, v[2] = cb;
+        if (what == 3) v[0] = sl, v[1] = -cl, v[2] = 0.0;
+        const double gc = what == 1 ? (second ? -1.0 : 0.5) : (second ? 0.0 : -1.5);
+        const double gs = what == 1 ? (second ? 0.0 : h) : (second ? -2.0 * h : h);
+        double o[5];
+        harmonics(v, gc, gs, o);
+        double *dst = what == 0 ? c->kn[second] : what == 1 ? c->kq[second] : what == 2 ? c->wn[second] : c->un[second];
+        const int n = what == 3 ? 3 : 5;
+        for (int i = 0; i < n; i++) dst[i] = o[i];
     }
 }
 
