@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(128, 4) dense_split_kernel(StageDims d, StageB
     float *sbin = reinterpret_cast<float *>(smem);  // [tile_bins][9]
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + sizeof(float) * kBinFloats * tile_bins);
     __shared__ float2 tab[256];
-    __shared__ int s_item, s_walker[G], s_lo[G][kMaxModes], s_hi[G][kMaxModes];
+    __shared__ int s_item, s_walker[G], s_here[G], s_lo[G][kMaxModes], s_hi[G][kMaxModes];
     __shared__ float s_flo[G][kMaxModes], s_scl[G][kMaxModes];
     __shared__ float4 red[G == 8 ? 1 : G][4];  // per slot, per warp: (ri, ri comp, hh, hh comp)
     // the first mode of each m (in the order of d.ord), their number; per walker and m the index
@@ -595,7 +595,6 @@ __global__ void __launch_bounds__(128, 4) dense_split_kernel(StageDims d, StageB
     // groups of 8 walkers: the (ri, ri comp, hh, hh comp) per slot of two threads together,
     // reduced once per item below instead of by warp shuffles per walker
     float4 *part_s = reinterpret_cast<float4 *>(bar + 2);  // [G][64], G = 8
-    __shared__ int s_skip[G];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int k = tid; k < 256; k += blockDim.x) {
         double sn, cs;
@@ -638,8 +637,10 @@ __global__ void __launch_bounds__(128, 4) dense_split_kernel(StageDims d, StageB
         if (tid < tail * kBinFloats)
             sbin[full * kBinFloats + tid] = bins[((size_t)J0 + full) * kBinFloats + tid];
         if (tid < G) {
-            const int i = g * G + tid;
-            s_walker[tid] = i < d.B ? b.order[i] : -1;
+            const int i = g * G + tid, w = i < d.B ? b.order[i] : -1;
+            s_walker[tid] = w;
+            // not an empty slot, and a band that reaches into the tile
+            s_here[tid] = w >= 0 && b.wrange[2 * w + 1] >= J0 && b.wrange[2 * w] < Jend;
         }
         if (tid < G * kMaxModes) {
             const int k = tid / kMaxModes, mi = tid % kMaxModes;
@@ -702,11 +703,7 @@ __global__ void __launch_bounds__(128, 4) dense_split_kernel(StageDims d, StageB
 
         for (int k = 0; k < G; k++) {
             const int w = s_walker[k];
-            if (w < 0 || b.wrange[2 * w + 1] < J0 || b.wrange[2 * w] >= Jend) {
-                if (tid == 0) s_skip[k] = 1;  // empty slot or band outside the tile
-                continue;
-            }
-            if (tid == 0) s_skip[k] = 0;
+            if (!s_here[k]) continue;
             const int j0 = J0 + tid * C;
             float hr[C][3], hm[C][3];
 #pragma unroll
@@ -868,7 +865,7 @@ __global__ void __launch_bounds__(128, 4) dense_split_kernel(StageDims d, StageB
             // thread, then the 8 threads' pairs by shuffles
             const int grp = tid >> 3, j = tid & 7, k = grp >> 1, q = grp & 1;
             float ps = 0.0f, pe = 0.0f;
-            if (s_walker[k] >= 0 && !s_skip[k]) {
+            if (s_here[k]) {
                 for (int i = 0; i < 8; i++) {
                     const float4 v = part_s[k * 64 + i * 8 + j];
                     float t, r;
@@ -890,7 +887,7 @@ __global__ void __launch_bounds__(128, 4) dense_split_kernel(StageDims d, StageB
         } else if (tid < G && s_walker[tid] >= 0) {
             const size_t slot = (size_t)item * G + tid;
             double a = 0.0, c = 0.0;
-            if (!s_skip[tid]) {
+            if (s_here[tid]) {
                 float4 v = red[tid][0];
                 float as = v.x, ae = v.y, cs = v.z, ce = v.w;
                 for (int q = 1; q < (int)(blockDim.x >> 5); q++) {
