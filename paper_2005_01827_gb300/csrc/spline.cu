@@ -15,11 +15,13 @@
 //
 // What bounds it: with few systems the latency of the sweep steps, so the series are dealt
 // to several blocks; with many systems the FP64 pipe (2 lanes per clock per SM): slopes and
-// right-hand sides are independent and use full warps, a sweep step is two or three FP64
-// operations.  Measured on GB300 (solve and coefficient kernel) against one
-// system per lane of one warp with every row in series: 1 system of 256 knots 367 -> 39 us,
-// 148 systems of 509 knots 938 -> 82 us, 6144 systems of 1024 knots 3.66 -> 3.11 ms in FP64
-// and 2.29 -> 1.55 ms in split precision.
+// right-hand sides and the divisions by the pivots are independent and use full warps, a sweep
+// step is one FP64 operation (the quotients are formed first, and pivots come as ratios of
+// minors, so that no division is in a chain: with divisions in the chain 39 us, 82 us, 3.11 and
+// 1.57 ms for the cases below).  Measured on GB300 (solve and coefficient kernel) against one
+// system per lane of one warp with every row in series: 1 system of 256 knots 367 -> 31 us,
+// 148 systems of 509 knots 938 -> 58 us, 6144 systems of 1024 knots 3.66 -> 2.71 ms in FP64
+// and 2.29 -> 1.45 ms in split precision.
 #include "kernels.h"
 #include "model.cuh"
 
@@ -49,23 +51,20 @@ __host__ __device__ inline Rows rows_of(int K, int tps) {
     return r;
 }
 
-// sweeping threads per series of a block that owns nq series
-__host__ __device__ inline int sweep_threads(int nq) {
-    return nq > 4 ? 32 : nq > 2 ? 64 : nq > 1 ? 128 : 256;
-}
+// Sweeping threads per series of a block that owns nq series.  A step has a latency of about
+// 50 clocks and takes 32 of the pipe per warp, so few warps with longer chunks (less run-in) are
+// best: the solve of one system of 256 (1024) knots, one series a block, 256 threads 25.6 (46.4)
+// us, 128 24.4 (44.3), 64 24.6 (44.8), 32 24.8 (46.7).
+__host__ __device__ inline int sweep_threads(int nq) { return nq > 1 ? 32 : 64; }
 
-// Forward sweep of one chunk: rp_i = (rhs_i - sub_i rp_{i-1}) / pivot_i in place.  `run`
-// selects the run-in (nothing stored) or the chunk itself.
+// Forward sweep of one chunk: rp_i = rhs_i / pivot_i - (sub_i / pivot_i) rp_{i-1} in place, the
+// quotients in y and sd.  `store` selects the chunk itself (the run-in stores nothing).
 template <typename T>
-__device__ __forceinline__ T sweep_forward(T *y, const T *h, const T *ih, const T *inv, const Rows R,
-                                           int from, int to, int n, T prev, bool store) {
+__device__ __forceinline__ T sweep_forward(T *y, const T *sd, const Rows R, int from, int to, T prev,
+                                           bool store) {
     for (int i = from; i < to; i++) {
         const int o = R.at(i);
-        const T hi = h[o];
-        T sb = h[R.at(i - 1)];
-        if (i == n - 2) sb -= hi * hi * ih[R.at(i - 1)];
-        const T rhs = y[o], dv = inv[o];
-        prev = (i == 1) ? rhs * dv : (rhs - sb * prev) * dv;
+        prev = y[o] - sd[o] * prev;
         if (store) y[o] = prev;
     }
     return prev;
@@ -88,7 +87,7 @@ __device__ __forceinline__ T sweep_backward(T *y, const T *c, const Rows R, int 
 // entries that the neighbours' chunks overwrite, hence stages of their own.
 template <typename T>
 __device__ __forceinline__ void solve_stage(int stage, T &v, T *y, const T *h, const T *ih,
-                                            const T *inv, const T *c, const Rows R, int t, int n) {
+                                            const T *sd, const T *c, const Rows R, int t, int n) {
     const int C = R.mask + 1;
     const int i0 = 1 + t * C, i1 = min(i0 + C, n - 1);
     if (stage == 4) {  // M_0 and M_{K-1} from their neighbours
@@ -99,8 +98,8 @@ __device__ __forceinline__ void solve_stage(int stage, T &v, T *y, const T *h, c
         return;
     }
     if (i0 >= n - 1) return;
-    if (stage == 0) v = sweep_forward(y, h, ih, inv, R, max(1, i0 - kHalo), i0, n, T(0), false);
-    if (stage == 1) sweep_forward(y, h, ih, inv, R, i0, i1, n, v, true);
+    if (stage == 0) v = sweep_forward(y, sd, R, max(1, i0 - kHalo), i0, T(0), false);
+    if (stage == 1) sweep_forward(y, sd, R, i0, i1, v, true);
     if (stage == 2) v = sweep_backward(y, c, R, i1, min(n - 1, i1 + kHalo), n, T(0), false);
     if (stage == 3) sweep_backward(y, c, R, i0, i1, n, v, true);
 }
@@ -119,12 +118,12 @@ __global__ void __launch_bounds__(kThreads) spline_kernel(StageDims d, StageBufs
     const int tps = sweep_threads(per);
     const Rows R = rows_of(K, tps);
     const int NP = R.at(K - 1) + 1;
-    double *h = reinterpret_cast<double *>(spl_sm), *ih = h + NP, *inv = ih + NP, *c = inv + NP;
+    double *h = reinterpret_cast<double *>(spl_sm), *ih = h + NP, *sd = ih + NP, *c = sd + NP;
     // FP64 series, then (split) the FP32 copies of the matrix and the FP32 series; a block of
     // one series holds only the kind it owns
     double *ys = c + NP;  // [1 or per][NP]
     float *h32 = reinterpret_cast<float *>(ys + (!kSplit ? per : per == 1 && q0 != 1 ? 0 : 1) * NP);
-    float *ih32 = h32 + NP, *inv32 = ih32 + NP, *c32 = inv32 + NP;
+    float *ih32 = h32 + NP, *sd32 = ih32 + NP, *c32 = sd32 + NP;
     float *ys32 = c32 + NP;  // split: [per][NP] (phase slot unused)
     const bool own32 = kSplit && !(per == 1 && q0 == 1);
     const double *x = b.fk + wm * K;
@@ -142,32 +141,34 @@ __global__ void __launch_bounds__(kThreads) spline_kernel(StageDims d, StageBufs
         }
     }
     __syncthreads();
-    // warp 0: pivots and super-diagonal of its chunk of rows; the others: right-hand sides
-    // 6 (slope_i - slope_{i-1}) of the block's series
+    // Warp 0: pivots of its chunk of rows, as ratios p_i / p_{i-1} of the leading minors p_i =
+    // dia_i p_{i-1} - sub_i sup_{i-1} p_{i-2} (in units of the chunk's first step), which have no
+    // division in the chain; left as p_i in c and p_{i-1} in sd.  The other warps: right-hand
+    // sides 6 (slope_i - slope_{i-1}) of the block's series
     if (tid < 32) {
         const int F = (n - 2 + 31) / 32, i0 = 1 + tid * F, i1 = min(i0 + F, n - 1);
-        double cp = 0.0;
-        for (int i = max(1, i0 - kPivotHalo); i < i1; i++) {
+        const int is = max(1, i0 - kPivotHalo);
+        const double unit = is < n - 1 ? ih[R.at(is)] : 0.0;
+        double pm = 0.0, p = 1.0, sup = 0.0;  // p_{i-2}, p_{i-1}, sup_{i-1}
+        for (int i = is; i < i1; i++) {
             const int o = R.at(i), om = R.at(i - 1);
             const double hp = h[om], hc = h[o];
-            double dia = 2.0 * (hp + hc), sup = hc, sb = hp;
+            double dia = 2.0 * (hp + hc), sb = hp, su = hc;
             if (i == 1) {
                 dia += hp * (hp + hc) * ih[o];
-                sup -= hp * hp * ih[o];
+                su -= hp * hp * ih[o];
             }
             if (i == n - 2) {
                 dia += hc * (hp + hc) * ih[om];
                 sb -= hc * hc * ih[om];
             }
-            const double v = 1.0 / ((i == 1) ? dia : dia - sb * cp);
-            cp = sup * v;
+            const double w = (sb * unit) * (sup * unit) * pm;
+            pm = p;
+            p = fma(dia * unit, p, -w);
+            sup = su;
             if (i >= i0) {
-                inv[o] = v;
-                c[o] = cp;
-                if (own32) {
-                    inv32[o] = (float)v;
-                    c32[o] = (float)cp;
-                }
+                sd[o] = pm * unit;
+                c[o] = p;
             }
         }
     } else {
@@ -192,6 +193,26 @@ __global__ void __launch_bounds__(kThreads) spline_kernel(StageDims d, StageBufs
         }
     }
     __syncthreads();
+    // divide by the pivots: sub- and super-diagonal, right-hand sides
+    for (int i = 1 + tid; i < n - 1; i += kThreads) {
+        const int o = R.at(i), om = R.at(i - 1);
+        const double hp = h[om], hc = h[o], v = sd[o] / c[o];
+        const double s = (i == 1) ? 0.0 : (i == n - 2) ? hp - hc * hc * ih[om] : hp;
+        const double u = (i == 1) ? hc - hp * hp * ih[o] : hc;
+        sd[o] = s * v;
+        c[o] = u * v;
+        if (own32) {
+            sd32[o] = (float)(s * v);
+            c32[o] = (float)(u * v);
+        }
+        for (int q = q0; q < q0 + per; q++) {
+            if (kSplit && q != 1)
+                ys32[(size_t)(q - q0) * NP + o] *= (float)v;
+            else
+                ys[(size_t)(kSplit ? 0 : q - q0) * NP + o] *= v;
+        }
+    }
+    __syncthreads();
     // a series' threads lie in whole warps, so the FP64 / FP32 choice is uniform per warp
     const int ql = tid / tps, t = tid % tps;
     double v64 = 0.0;
@@ -199,9 +220,9 @@ __global__ void __launch_bounds__(kThreads) spline_kernel(StageDims d, StageBufs
     for (int stage = 0; stage < 5; stage++) {
         if (ql < per) {
             if (kSplit && q0 + ql != 1)
-                solve_stage<float>(stage, v32, ys32 + (size_t)ql * NP, h32, ih32, inv32, c32, R, t, n);
+                solve_stage<float>(stage, v32, ys32 + (size_t)ql * NP, h32, ih32, sd32, c32, R, t, n);
             else
-                solve_stage<double>(stage, v64, ys + (size_t)(kSplit ? 0 : ql) * NP, h, ih, inv, c, R, t, n);
+                solve_stage<double>(stage, v64, ys + (size_t)(kSplit ? 0 : ql) * NP, h, ih, sd, c, R, t, n);
         }
         __syncthreads();
     }
@@ -269,13 +290,14 @@ size_t spline_smem(int K, int per) {
     return per == 1 ? NP * (8 * 4 + 4 * 5) : NP * (8 * 5 + 4 * (4 + per));
 }
 
-// Blocks per system: one while the systems fill the chip, more (each with fewer series,
-// the pivots repeated) while they do not or while a block's rows would not fit in shared
-// memory (K above about 2300).
+// Blocks per system: one while the systems fill the chip's 152 SMs, more (each with fewer
+// series, the pivots repeated) while they do not or while a block's rows would not fit in
+// shared memory (K above about 2300).  Solve and coefficients with 1, 2, 4, 8 blocks a system: one
+// system of 256 knots 35, 33, 31, 31 us, 148 systems of 509 knots 58, 62, 70, 105 us.
 template <bool kSplit>
 int spline_blocks(int nsys, int K) {
     int y = 1;
-    while (y < kNSeries && nsys * y * 2 <= 152 * 2) y *= 2;
+    while (y < kNSeries && nsys * y * 2 <= 152) y *= 2;
     while (y < kNSeries && spline_smem<kSplit>(K, kNSeries / y) > kMaxSmem) y *= 2;
     return y;
 }
