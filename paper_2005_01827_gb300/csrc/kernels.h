@@ -76,7 +76,7 @@ struct StageBufs {
     int *grange;           // [groups][2] union range of each group (start a multiple of 4)
     int *item_start;       // [groups+1] exclusive prefix of the dense work items
     int *counter;          // dense work-queue counter
-    const FxTab *fxtab;    // phasor table of the FP64 dense kernel, written by the source kernel
+    const FxTab *fxtab;    // phasor table of the fixed-point kernels, written by the source kernel
     int *err;              // set by a device wait that gave up
     double *part;          // [items][G][2] per-item, per-slot partial sums
     // Test only (0 in normal operation): when > 0 the dense kernels arm the barrier of each

@@ -49,7 +49,7 @@ struct lisa_like {
     int N = 0;
     double *bins = nullptr;   // [N][9] FP64 staged data
     float4 *rows = nullptr;   // the same in the FP64 dense kernel's form (FP64 precision)
-    FxTab *fxtab = nullptr;   // its phasor table
+    FxTab *fxtab = nullptr;   // phasor table of the knots and the FP64 dense kernel
     float *bins32 = nullptr;  // [N][kBinFloats] FP32 whitened data (split precision)
     SegRec *segs = nullptr;   // [max_batch][L][K-1] split-precision segment records
     unsigned long long *phases = nullptr;  // [max_batch][L][K-1][8] FP64-path phase records
@@ -162,10 +162,9 @@ lisa_status alloc_batch(lisa_like_t *h) {
     LCK(dalloc(&h->out, 3 * B), "device allocation (outputs)");
     if (h->precision == LISA_PREC_SPLIT)
         LCK(dalloc(&h->segs, B * L * (K - 1)), "device allocation (split segments)");
-    else {
+    else
         LCK(dalloc(&h->phases, B * L * (K - 1) * kPhaseWords), "device allocation (phase anchors)");
-        LCK(dalloc((unsigned char **)&h->fxtab, kFxTabBytes), "device allocation (phasor table)");
-    }
+    LCK(dalloc((unsigned char **)&h->fxtab, kFxTabBytes), "device allocation (phasor table)");
     LCK(cudaMallocHost(&h->h_params, sizeof(double) * B * kNPar), "pinned allocation");
     LCK(cudaMallocHost(&h->h_out, sizeof(double) * 3 * B), "pinned allocation");
     LCK(cudaMallocHost(&h->h_err, sizeof(int)), "pinned allocation");

@@ -22,6 +22,13 @@ namespace lisa {
 
 constexpr double kPi = 3.141592653589793238462643383279502884;
 constexpr double kTwoPi = 6.283185307179586476925286766559005768;
+// Cody-Waite three-part split of 2 pi for the exact reduction of a knot phase to a
+// fraction of a turn: a head with few significant bits (so k x head is exact for the
+// multiples k that occur), then the FP64 middle and tail of the remainder.
+constexpr double kTwoPiHi = 6.2831854820251465;        // FP32-exact leading part of 2 pi
+constexpr double kTwoPiMid = -1.748455600074497e-07;   // 2 pi - hi
+constexpr double kTwoPiLo = -1.0687562935444062e-23;   // 2 pi - hi - mid
+constexpr double kInvTwoPi = 0.15915494309189535;
 constexpr double kMsunS = 4.925490947641267e-06;  // G M_sun / c^3 [s]
 constexpr double kClight = 299792458.0;
 constexpr double kGpcM = 3.0856775814913673e25;

@@ -229,7 +229,7 @@ __device__ inline double block_sum(double v, double *red) {
 // the response but for their polarisation weights (response.cuh), powers of the edge frequencies
 // are tabulated, divisions by the fiducial and by the bin widths are in the stored
 // data, each ratio is formed once, and the pairs of a mode are summed before its ratio
-// multiplies them (12 operations a pair).  1024 walkers, 128 bins, six modes: 3.67 -> 1.7 ms.
+// multiplies them (12 operations a pair).  1024 walkers, 128 bins, six modes: 3.67 -> 1.5 ms.
 __global__ void __launch_bounds__(kRbThreads, 2) rb_walker_kernel(RbDev r, StageDims d, StageBufs b,
                                                                   double *lnL, double *dh,
                                                                   double *hh) {
@@ -277,8 +277,8 @@ __global__ void __launch_bounds__(kRbThreads, 2) rb_walker_kernel(RbDev r, Stage
         ModeBase base;
         double sn = 0.0, cs = 0.0;
         if (in) {
-            mode_base(wc, mc[a0], f, mc[a0].v0 * r.fe[ne + e], mc[a0].x160 * r.fe[2 * ne + e], base);
-            sincos(base.phase - 2.0 * kPi * f * wc.tc, &sn, &cs);
+            mode_base(wc, mc[a0], b.fxtab, f, mc[a0].v0 * r.fe[ne + e], mc[a0].x160 * r.fe[2 * ne + e], base);
+            phasor_radians(base.phase - 2.0 * kPi * f * wc.tc, b.fxtab, sn, cs);
         }
         for (int q = i0; q < L && (q == i0 || d.same[q]); q++) {
             const int a = d.ord[q];

@@ -12,6 +12,7 @@
 // y_ca + D y_ac = e^{-ix} E ((s1 + s2) cos x + i (s2 - s1) sin x), and 1 - D^2 =
 // 2i sin 2x e^{-2ix}.
 #pragma once
+#include "fixed.cuh"
 #include "model.cuh"
 
 namespace lisa {
@@ -52,6 +53,49 @@ static __device__ __noinline__ double near_arm_link(double x, double g) {
     return g == 0.0 ? x : sin(x * g) / g;
 }
 
+// cos and sin of 2 pi turns on the integer units (fixed.cuh; |turns| < 2^20), with an absolute error of
+// about 2e-16, like the rounding of a cosine near 1: for unit phasors and angles, not where a small
+// sine counts.  tab: the phasor table of kFxTab entries
+__device__ __forceinline__ void phasor_turns(double turns, const FxTab *__restrict__ tab, double &sn, double &cs) {
+    const double fr = turns - rint(turns);
+    const i64 v = to_fixed(fr, 62);  // |fr| <= 1/2
+    const unsigned long long ph = (unsigned long long)v << 2;
+    const int4 e = __ldg(reinterpret_cast<const int4 *>(tab + fx_cell(ph)));
+    i64 zr, zi;
+    fx_rotate(ph, FxTab{Bal{e.x, e.y}, Bal{e.z, e.w}}, zr, zi);
+    cs = (double)zr * 0x1p-60;
+    sn = (double)zi * 0x1p-60;
+}
+
+// cos and sin of x radians, |x| < 1e9, likewise: x is reduced by the split of 2 pi, without the
+// slow path that sincos() takes beyond 1e5
+__device__ __forceinline__ void phasor_radians(double x, const FxTab *__restrict__ tab, double &sn, double &cs) {
+    const double k = rint(x * kInvTwoPi);
+    double r = fma(-k, kTwoPiHi, x);
+    r = fma(-k, kTwoPiMid, r);
+    r = fma(-k, kTwoPiLo, r);
+    phasor_turns(r * kInvTwoPi, tab, sn, cs);
+}
+
+// sin and cos of |x| <= 0.35 by their Taylor series (the next terms are below 2e-17 of them): 15
+// operations against about 25 of sincos()
+__device__ __forceinline__ void sincos_small(double x, double &sn, double &cs) {
+    const double y = x * x;
+    double a = fma(y, 1.0 / 6227020800.0, -1.0 / 39916800.0);
+    a = fma(y, a, 1.0 / 362880.0);
+    a = fma(y, a, -1.0 / 5040.0);
+    a = fma(y, a, 1.0 / 120.0);
+    a = fma(y, a, -1.0 / 6.0);
+    sn = fma(x * y, a, x);
+    double b = fma(y, -1.0 / 87178291200.0, 1.0 / 479001600.0);
+    b = fma(y, b, -1.0 / 3628800.0);
+    b = fma(y, b, 1.0 / 40320.0);
+    b = fma(y, b, -1.0 / 720.0);
+    b = fma(y, b, 1.0 / 24.0);
+    b = fma(y, b, -0.5);
+    cs = fma(y, b, 1.0);
+}
+
 // What the modes of equal m share at one frequency: (m / 2) phi_22(2 f / m) with the
 // constellation-centre delay, the amplitude up to the mode's factor, and the response up to
 // the mode's polarisation weights.  Their modes add about 85 operations each to about 340.
@@ -63,8 +107,9 @@ struct ModeBase {
 };
 
 // v = (pi x)^(1/3) and x16 = x^(1/6) of the mapped frequency x = xf f; m: any mode of this m
-__device__ __forceinline__ void mode_base(const WalkerConst &w, const ModeConst &m, double f,
-                                          double v, double x16, ModeBase &o) {
+__device__ __forceinline__ void mode_base(const WalkerConst &w, const ModeConst &m,
+                                          const FxTab *__restrict__ tab, double f, double v, double x16,
+                                          ModeBase &o) {
     const double x = m.xf * f;
     const double r = x * w.ixrd, r2 = r * r;
     const double v2 = v * v;
@@ -83,7 +128,7 @@ __device__ __forceinline__ void mode_base(const WalkerConst &w, const ModeConst 
     }
     const double t = fma(-w.m2pi, dp - w.dphpk, w.tc);
     double sa, ca;
-    sincos((kTwoPi / kYearS) * t, &sa, &ca);
+    phasor_turns((1.0 / kYearS) * t, tab, sa, ca);
     const double s2a = 2.0 * sa * ca, c2a = fma(-2.0 * sa, sa, 1.0);
     o.phase = fma(m.half_m, fma(-w.dphpk, x, p), m.off) + f * fma(w.dx, ca, w.dy * sa);
     auto harm5 = [&](const double *o) {
@@ -103,21 +148,30 @@ __device__ __forceinline__ void mode_base(const WalkerConst &w, const ModeConst 
     const double kq0 = harm5(w.kq[0]), kq2 = harm5(w.kq[1]);
 
     const double xl = (kPi * (kArmM / kClight)) * f;  // pi f L
+    // |k.n| <= 1, so every angle below but the propagation phases is at most x
+    const bool small = xl <= 0.35;  // f < 13 mHz
+    auto sine = [&](double a, double &sn, double &cs) {
+        if (small)
+            sincos_small(a, sn, cs);
+        else
+            sincos(a, &sn, &cs);
+    };
     double sx, cx;
-    sincos(xl, &sx, &cx);
+    sine(xl, sx, cx);
     // e^{-i x k.(q_a + q_c) / L}; the middle arm's is the conjugate product of the others
     cplx g[3];
     {
         double s0, c0, s2, c2;
-        sincos(xl * kq0, &s0, &c0);
-        sincos(xl * kq2, &s2, &c2);
+        const double xt = xl * (1.0 / kTwoPi);
+        phasor_turns(xt * kq0, tab, s0, c0);
+        phasor_turns(xt * kq2, tab, s2, c2);
         g[0] = {c0, -s0};
         g[2] = {c2, -s2};
         g[1] = {c0 * c2 - s0 * s2, c0 * s2 + s0 * c2};
     }
     double sn[3], cn[3];
-    sincos(xl * kn[0], &sn[0], &cn[0]);
-    sincos(xl * kn[2], &sn[2], &cn[2]);
+    sine(xl * kn[0], sn[0], cn[0]);
+    sine(xl * kn[2], sn[2], cn[2]);
     sn[1] = sn[0] * cn[2] + cn[0] * sn[2];
     cn[1] = cn[0] * cn[2] - sn[0] * sn[2];
 

@@ -148,7 +148,7 @@ __device__ __forceinline__ double md_scale(const Mode &md) {
     return md.m == 1 ? 2.0 : md.m == 2 ? 1.0 : md.m == 3 ? 2.0 / 3.0 : 0.5;
 }
 
-// One block more than the walkers need writes the phasor table of the FP64 dense kernel.
+// One block more than the walkers need writes the phasor table of the fixed-point kernels.
 __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
     if (blockIdx.x == gridDim.x - 1) {
         FxTab *tab = const_cast<FxTab *>(b.fxtab);
@@ -314,15 +314,16 @@ cudaError_t launch_source(const StageDims &d, const StageBufs &b, cudaStream_t s
 // split-precision layout).
 //
 // Bound by the FP64 pipe (2 lanes per clock per SM), so the count of FP64 operations per
-// knot is what matters (about 330 an m and 85 a mode, against 730 a mode): the powers of f come from one
+// knot is what matters (about 270 an m and 85 a mode, against 730 a mode): the powers of f come from one
 // exponential of the log-spaced step (f^(1/6) and its powers, no cube root or square root),
 // one division serves v, the amplitude and the three arms, the response is in orbital
 // harmonics, and the modes of equal m share all of it but their polarisation weights
-// (response.cuh).  1024 walkers, six modes of 1024 knots: 8.4 -> 4.1 ms with the source kernel
-// (5.4 with one mode per thread).  One block of 128 threads per system left all but a few SMs idle in small
+// (response.cuh), whose unit phasors and orbital angle are evaluated on the integer units and the
+// sines of small angles by series.  1024 walkers, six modes of 1024 knots: 8.4 -> 3.3 ms with the
+// source kernel (5.4 with one mode per thread, 4.0 with sincos() throughout).  One block of 128 threads per system left all but a few SMs idle in small
 // calls (6 systems of 1024 knots: 246 us), hence one knot per thread.
 template <bool kSplit>
-__global__ void __launch_bounds__(128) knot_kernel(StageDims d, StageBufs b) {
+__global__ void __launch_bounds__(128) knot_kernel(StageDims d, StageBufs b, double idf, double near) {
     const int w = blockIdx.x / d.L, first = blockIdx.x % d.L;
     if (d.same[first]) return;  // done with the first mode of its m
     const size_t wm = (size_t)w * d.L + d.ord[first];
@@ -346,12 +347,14 @@ __global__ void __launch_bounds__(128) knot_kernel(StageDims d, StageBufs b) {
     const double f = (k == K - 1) ? fhi : flo * (e3 * e3 * e3);
     // first dense bin at or above this knot: a guess, then exact by the bin frequencies
     // themselves
-    const double g = ceil((f - d.f0) / d.df);
-    int j = g <= 0.0 ? 0 : (g >= (double)d.N ? d.N : (int)g);
-    while (j > 0 && bin_freq(d.f0, d.df, j - 1) >= f) j--;
-    while (j < d.N && bin_freq(d.f0, d.df, j) < f) j++;
+    const double g = (f - d.f0) * idf, gc = ceil(g);
+    int j = gc <= 0.0 ? 0 : (gc >= (double)d.N ? d.N : (int)gc);
+    if (fabs(g - rint(g)) < near) {
+        while (j > 0 && bin_freq(d.f0, d.df, j - 1) >= f) j--;
+        while (j < d.N && bin_freq(d.f0, d.df, j) < f) j++;
+    }
     ModeBase base;
-    mode_base(wc, mc, f, mc.v0 * e3, mc.x160 * e6, base);
+    mode_base(wc, mc, b.fxtab, f, mc.v0 * e3, mc.x160 * e6, base);
     for (int i = first; i < d.L && (i == first || d.same[i]); i++) {
         const size_t m = (size_t)w * d.L + d.ord[i];
         double amp;
@@ -382,7 +385,9 @@ template <bool kSplit>
 static cudaError_t launch_knots_t(const StageDims &d, const StageBufs &b, cudaStream_t s) {
     cudaError_t e = launch_source(d, b, s);
     if (e != cudaSuccess) return e;
-    knot_kernel<kSplit><<<dim3(d.B * d.L, (d.K + 127) / 128), 128, 0, s>>>(d, b);
+    // how near to a whole number a knot's bin number may be wrong: numbers below 1e11 are right to 1e-4
+    const double near = d.f0 / d.df + d.N < 1e11 ? 1e-3 : 1.0;
+    knot_kernel<kSplit><<<dim3(d.B * d.L, (d.K + 127) / 128), 128, 0, s>>>(d, b, 1.0 / d.df, near);
     return cudaGetLastError();
 }
 

@@ -34,16 +34,6 @@
 
 namespace lisa {
 
-namespace {
-// Cody-Waite three-part split of 2 pi for the exact reduction of a knot phase to a
-// fraction of a turn: a head with few significant bits (so k x head is exact for the
-// multiples k that occur), then the FP64 middle and tail of the remainder.
-constexpr double kTwoPiHi = 6.2831854820251465;        // FP32-exact leading part of 2 pi
-constexpr double kTwoPiMid = -1.748455600074497e-07;   // 2 pi - hi
-constexpr double kTwoPiLo = -1.0687562935444062e-23;   // 2 pi - hi - mid
-constexpr double kInvTwoPi = 0.15915494309189535;
-}  // namespace
-
 // fraction of a turn of x radians as a 128-bit two's-complement fixed-point number:
 // hi holds the turns scaled by 2^64 (modulo 2^64), lo the next 64 fractional bits
 __device__ __forceinline__ void turns_fixed(double x, unsigned long long &hi,
