@@ -156,28 +156,31 @@ cudaError_t launch_plan(const StageDims &d, const StageBufs &b, int tile_bins, i
 }
 
 // ---------------------------------------------------------------------------- finish
-// Per walker, the sums of its slot over its group's items: one warp per walker, each lane a
-// stride of the items, then a fixed tree, so the result does not depend on which block ran
-// which item.  FP64: ln L = <d|h> - <h|h>/2 - <d|d>/2 (Eq. (2)).  Split: the parts hold sum
+// Per walker, the sums of its slot over its group's items: `warps` warps per walker (a block
+// holds kFinishWarps), each lane a stride of the items, then a fixed tree, so the result does not
+// depend on which block ran which item.  FP64: ln L = <d|h> - <h|h>/2 - <d|d>/2 (Eq. (2)).  Split: the parts hold sum
 // (|h|^2 - 2 Re(d h*)) and <h|h>, and ln L = -sum/2 - <d|d>/2.  A device wait that gave up
 // poisons every output with NaN.
 //
 // A walker of the 1-yr grid has up to 3082 items; one thread summing them in series was
 // bound by the latency of dependent loads (620 us for five walkers, 778 us for 1024);
-// a warp per walker takes 6 us for one walker and 29 us for
-// 1024.
-__global__ void __launch_bounds__(128) finish_kernel(StageDims d, StageBufs b, int G, int split,
-                                                     double dd, double *lnL, double *dh, double *hh) {
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (w >= d.B) return;
-    const bool ok = b.valid[w] != 0;
+// a warp per walker takes 25 us for five walkers and 29 us for 1024, eight warps 10 and 24; eight are
+// used while the walkers' blocks fit the chip at once.
+constexpr int kFinishWarps = 8;
+__global__ void __launch_bounds__(32 * kFinishWarps) finish_kernel(StageDims d, StageBufs b, int G, int split,
+                                                                  int warps, double dd, double *lnL,
+                                                                  double *dh, double *hh) {
+    __shared__ double2 s_part[kFinishWarps];
+    const int warp = threadIdx.x >> 5, sub = warp % warps;
+    const int w = (blockIdx.x * kFinishWarps + warp) / warps, lane = threadIdx.x & 31;
+    const bool ok = w < d.B && b.valid[w] != 0;
     double a = 0.0, c = 0.0;
     if (ok) {
         const int i = b.slot_of[w], g = i / G, k = i % G;
         const int end = b.item_start[g + 1];
         const double2 *part = reinterpret_cast<const double2 *>(b.part);
 #pragma unroll 4
-        for (int it = b.item_start[g] + lane; it < end; it += 32) {
+        for (int it = b.item_start[g] + sub * 32 + lane; it < end; it += 32 * warps) {
             const double2 v = part[(size_t)it * G + k];
             a += v.x;
             c += v.y;
@@ -187,7 +190,13 @@ __global__ void __launch_bounds__(128) finish_kernel(StageDims d, StageBufs b, i
         a += __shfl_down_sync(0xffffffffu, a, o);
         c += __shfl_down_sync(0xffffffffu, c, o);
     }
-    if (lane) return;
+    if (lane == 0) s_part[warp] = make_double2(a, c);
+    __syncthreads();
+    if (lane || sub || w >= d.B) return;
+    for (int i = 1; i < warps; i++) {
+        a += s_part[warp + i].x;
+        c += s_part[warp + i].y;
+    }
     double out = !ok ? -INFINITY : split ? -0.5 * a - 0.5 * dd : a - 0.5 * c - 0.5 * dd;
     double dhv = split ? 0.5 * (c - a) : a;
     if (*b.err) {
@@ -202,7 +211,9 @@ __global__ void __launch_bounds__(128) finish_kernel(StageDims d, StageBufs b, i
 
 cudaError_t launch_finish(const StageDims &d, const StageBufs &b, int group, int split, double dd,
                           double *lnL, double *dh, double *hh, cudaStream_t s) {
-    finish_kernel<<<(d.B + 3) / 4, 128, 0, s>>>(d, b, group, split, dd, lnL, dh, hh);
+    const int warps = d.B <= 8 * 152 ? kFinishWarps : 1;
+    finish_kernel<<<(d.B * warps + kFinishWarps - 1) / kFinishWarps, 32 * kFinishWarps, 0, s>>>(
+        d, b, group, split, warps, dd, lnL, dh, hh);
     return cudaGetLastError();
 }
 
