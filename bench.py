@@ -46,23 +46,26 @@ WORKLOAD_C3 = ("8192 walkers with M_T log-uniform in [1e3, 1e9] Msun, 6 modes, K
 # integrand Re(d h*) w and |h|^2 w with its partial-sum add, about 25 flops.
 FLOP_MODE_BIN = 75
 FLOP_BIN = 25
-# The implementation's own count of what the kernels execute, reported beside it: the
-# phase series' Horner is replaced by the exact recurrence, and per (walker, mode, bin) it
-# adds the segment offset (1), the t_coal ramp (2) and the table-plus-polynomial phasor
-# (18) and spends 24 on the complex products = 95 flops; per (walker, bin) f_j (2) and
-# the integrand (27) = 29 flops.
-IMPL_FLOP_MODE_BIN = 48 + 1 + 2 + 18 + 2 + 24
+# The implementations' own counts, reported beside it.  The FP64 dense kernel runs in 64-bit
+# fixed point on the integer units: about 185 multiply-adds of two 32-bit integers per
+# (walker, mode, bin) (ncu's opcode counts over the launch's units), of which an SM does 56
+# a clock (measured; a 32 x 32 -> 64 multiply-add).  The split kernel, per (walker, m, bin)
+# with 4 values of m for 6 modes: quadratics of A T (24 flops), phasor (17), complex
+# multiply-add (24), and the re-expansion of the quartics per 8 bins (14); per (walker, bin)
+# the integrand (29).
+INT_MAD_MODE_BIN = 185
+INT_MAD_CLK_SM = 56
+IMPL_FLOP_MODE_BIN = (24 + 17 + 24 + 14) * 4 / 6
 IMPL_FLOP_BIN = 29
-# data bytes streamed per bin by a walker tile (w and w*d for A, E, T, FP64) and the
-# spline coefficients per segment (8 series x 4 doubles)
-BYTES_BIN = 72
+# data bytes streamed per bin by a walker tile (w and w*d for A, E, T as FP32 pairs, and
+# exponents) and the spline coefficients per segment (8 series x 4 doubles)
+BYTES_BIN = 76
 # DRAM bytes per (walker, bin) of the dense kernels from ncu captures of 32 walkers
 # (dram__bytes_read.sum + dram__bytes_write.sum over 69,589,136 walker-bins), per tile
 # shape (bins per thread, group); scaled to a launch by its walker-bins.  A shape without
 # a capture reports null.
-TRAFFIC_F64_PER_WALKER_BIN = {(8, 8): (753.79e6 + 5.11e6) / 69589136,
-                              (4, 8): (755.36e6 + 6.43e6) / 69589136}
-TRAFFIC_SPLIT_PER_WALKER_BIN = {(8, 8): (374.96e6 + 4.37e6) / 69589136}
+TRAFFIC_F64_PER_WALKER_BIN = {(8, 8): (795.31e6 + 4.97e6) / 69589136}
+TRAFFIC_SPLIT_PER_WALKER_BIN = {(8, 8): (376.44e6 + 10.92e6) / 69589136}
 
 
 def peaks():
@@ -332,9 +335,9 @@ def time_split(lisalike, LisaLike, g, th, B, args, world, stream, mode_bins, bin
                          "traffic": traffic,
                          "traffic_unit": "bytes per launch",
                          "hbm_gbs": traffic / (dense_ms * 1e-3) / 1e9 if traffic else None,
-                         "algorithmic_bytes": algo_bytes(bins, shape[1], B, coef_bytes=192, bin_bytes=36),
+                         "algorithmic_bytes": algo_bytes(bins, shape[1], B, coef_bytes=150, bin_bytes=36),
                          "traffic_over_algorithmic":
-                             traffic / algo_bytes(bins, shape[1], B, coef_bytes=192, bin_bytes=36)
+                             traffic / algo_bytes(bins, shape[1], B, coef_bytes=150, bin_bytes=36)
                              if traffic else None,
                          "units_per_launch": {"walker_mode_bins": mode_bins, "walker_bins": bins},
                          "fractions": {
@@ -342,10 +345,9 @@ def time_split(lisalike, LisaLike, g, th, B, args, world, stream, mode_bins, bin
                              "fp64": None, "mufu": None,
                              "hbm": (tpw * bins / (dense_ms * 1e-3) / 1e9 / peaks()["hbm_gbs"])
                              if (tpw and peaks().get("hbm_gbs")) else None,
-                             "note": "fp64: per-item set-up only; mufu: one log2 per chunk "
-                                     "(the phasor is a table and polynomials); ncu: issue 65 %, "
-                                     "FMA pipe 54 % of cycles (packed f32x2 Horner and "
-                                     "integrand), ALU 29 %"},
+                             "note": "fp64: none; mufu: one log2 per segment search (the "
+                                     "phasor is a table and polynomials); ncu: issue 64 %, "
+                                     "FMA pipe 48 % of cycles, ALU 36 %"},
                          "peak_source": "derived: 152 SM x 128 FP32 FMA/clk x 2 x 2.07 GHz",
                          "measured_pipes": {
                              "fp32_tflops": 2 * probe["fp32_fma_per_s"] / 1e12,
@@ -862,7 +864,7 @@ def run_rb(args, world, rank, local):
                                        "lnL_spread": float(lden.max() - lden.min())},
             "dense_fp64_ms_same_walkers": dense_ms, "fiducial_setup_s": setup_s,
             "speedup_vs_dense_fp64": dense_ms / (ms / args.steps),
-            "roofline": {"bound": "alu", "kernel": "rb_walker_kernel (+ band_kernel)",
+            "roofline": {"bound": "alu", "kernel": "rb_walker_kernel (+ source_kernel)",
                          "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak, "traffic": None,
                          "peak_source": "derived: 152 SM x 2 FP64 FMA/clk x 2 x 2.07 GHz",
@@ -888,11 +890,19 @@ def algo_bytes(walker_bins, group, B, L=6, K=1024, coef_bytes=256, bin_bytes=Non
 
 
 def impl_count(mode_bins, bins, dense_ms, peak):
-    """The dense kernel's rate by the implementation's own flop count (labelled figure
+    """The split dense kernel's rate by the implementation's own flop count (labelled figure
     beside the algorithmic one)."""
     a = (IMPL_FLOP_MODE_BIN * mode_bins + IMPL_FLOP_BIN * bins) / (dense_ms * 1e-3) / 1e12
     return {"flop_per_walker_mode_bin": IMPL_FLOP_MODE_BIN, "flop_per_walker_bin": IMPL_FLOP_BIN,
             "achieved": a, "frac": a / peak}
+
+
+def int_count(mode_bins, dense_ms):
+    """The FP64 dense kernel's rate on the integer multiply-add units."""
+    a = INT_MAD_MODE_BIN * mode_bins / (dense_ms * 1e-3) / 1e12
+    peak = 152 * INT_MAD_CLK_SM * 2.07e9 / 1e12
+    return {"int_mad_per_walker_mode_bin": INT_MAD_MODE_BIN, "achieved": a, "peak": peak,
+            "unit": "T multiply-adds/s", "frac": a / peak}
 
 
 def profile_once(lisalike, like, step):
@@ -1082,7 +1092,7 @@ def like_line(args, world, rank, local, c3):
     flops = FLOP_MODE_BIN * mode_bins + FLOP_BIN * bins
     achieved = flops / (dense_ms * 1e-3) / 1e12
     peak = fp64_peak_tflops()
-    impl = impl_count(mode_bins, bins, dense_ms, peak)
+    impl = int_count(mode_bins, dense_ms)
     tpw = TRAFFIC_F64_PER_WALKER_BIN.get(tuple(shape[:2]))
     traffic = tpw * bins if tpw else None
     probe = lisalike.probe_pipes(local)      # measured pipe rates of this device
@@ -1107,14 +1117,16 @@ def like_line(args, world, rank, local, c3):
                                    "frac_of_measured_fp64": achieved / (2 * probe["fp64_fma_per_s"] / 1e12),
                                    "source": "lisa_probe_pipes: FMA / MUFU chains on every SM"}}
     hbm_peak = peaks().get("hbm_gbs")
+    roofline["note"] = ("achieved and peak: the algorithmic FP64 flops against the FP64 pipe; above "
+                        "it because the kernel does that work in 64-bit fixed point on the integer "
+                        "units (implementation_count)")
     roofline["fractions"] = {
-        "binding": "fp64", "fp64": achieved / peak, "fp32": 0.0, "mufu": 0.0,
+        "binding": "integer multiply-add", "int_mad": impl["frac"], "fp64": None, "fp32": None,
+        "mufu": 0.0,
         "hbm": (traffic / (dense_ms * 1e-3) / 1e9 / hbm_peak) if (traffic and hbm_peak) else None,
-        "note": "fp32 and mufu: the FP64 kernel's inner loop issues neither (ncu <4,8>: FP64 "
-                "pipe 94 % busy, FMA pipe 1.0 %); hbm: measured DRAM bytes per launch over "
-                "the launch time"}
+        "note": "hbm: measured DRAM bytes per launch over the launch time"}
     if c3:
-        roofline["note"] = "stage times from one profiled call before graph replay"
+        roofline["note"] += "; stage times from one profiled call before graph replay"
     line = {"metric": METRIC, "value": value, "unit": "evals/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",

@@ -30,16 +30,6 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
                  : "memory");
 }
 
-// issue one bulk copy global -> shared that completes on a barrier armed for its bytes; dst
-// and src must be 16-byte aligned and bytes a multiple of 16
-__device__ __forceinline__ void tma_copy_1d(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_addr(dst)),
-        "l"(src), "r"(bytes), "r"(smem_addr(bar))
-        : "memory");
-}
-
 // arm the barrier for `bytes` of transaction and issue one bulk copy global -> shared.
 // dst and src must be 16-byte aligned and bytes a multiple of 16.
 __device__ __forceinline__ void tma_load_1d(void *dst, const void *src, uint32_t bytes,
