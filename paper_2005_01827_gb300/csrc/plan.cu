@@ -158,14 +158,15 @@ cudaError_t launch_plan(const StageDims &d, const StageBufs &b, int tile_bins, i
 // ---------------------------------------------------------------------------- finish
 // Per walker, the sums of its slot over its group's items: `warps` warps per walker (a block
 // holds kFinishWarps), each lane a stride of the items, then a fixed tree, so the result does not
-// depend on which block ran which item.  FP64: ln L = <d|h> - <h|h>/2 - <d|d>/2 (Eq. (2)).  Split: the parts hold sum
-// (|h|^2 - 2 Re(d h*)) and <h|h>, and ln L = -sum/2 - <d|d>/2.  A device wait that gave up
-// poisons every output with NaN.
+// depend on which block ran which item.  FP64: ln L = <d|h> - <h|h>/2 - <d|d>/2 (Eq. (2)).
+// Split: the parts hold sum (|h|^2 - 2 Re(d h*)) and <h|h>, and ln L = -sum/2 - <d|d>/2.  A
+// device wait that gave up poisons every output with NaN.
 //
 // A walker of the 1-yr grid has up to 3082 items; one thread summing them in series was
 // bound by the latency of dependent loads (620 us for five walkers, 778 us for 1024);
-// a warp per walker takes 25 us for five walkers and 29 us for 1024, eight warps 10 and 24; eight are
-// used while the walkers' blocks fit the chip at once.
+// a warp per walker takes 25 us for five walkers there and 43 for 1024, eight warps 10 and 27.  With
+// few items (one walker on 30 days: 26) one warp is faster, 6 against 8 us, so eight are used on
+// grids of more than 2^18 bins, while the walkers fit the chip at once.
 constexpr int kFinishWarps = 8;
 __global__ void __launch_bounds__(32 * kFinishWarps) finish_kernel(StageDims d, StageBufs b, int G, int split,
                                                                   int warps, double dd, double *lnL,
@@ -211,7 +212,7 @@ __global__ void __launch_bounds__(32 * kFinishWarps) finish_kernel(StageDims d, 
 
 cudaError_t launch_finish(const StageDims &d, const StageBufs &b, int group, int split, double dd,
                           double *lnL, double *dh, double *hh, cudaStream_t s) {
-    const int warps = d.B <= 8 * 152 ? kFinishWarps : 1;
+    const int warps = d.N > 1 << 18 && d.B <= 8 * 152 ? kFinishWarps : 1;
     finish_kernel<<<(d.B * warps + kFinishWarps - 1) / kFinishWarps, 32 * kFinishWarps, 0, s>>>(
         d, b, group, split, warps, dd, lnL, dh, hh);
     return cudaGetLastError();
