@@ -36,8 +36,8 @@
 // all issue slots waited for instructions: 428 ms against 219 (below).  The data rows (76 bytes
 // per bin, float pairs) are read from L2 by each walker.
 //
-// Bound by the multiply-add pipe (66 % busy: 143 integer multiply-adds per (walker, mode,
-// bin), 58 % of issue slots).  1024 walkers, six modes, 1-yr grid: 951 -> 219 ms; 37 walkers,
+// Bound by the multiply-add pipe (66 % busy: 185 integer multiply-adds per (walker, mode,
+// bin), 58 % of issue slots).  1024 walkers, six modes, 1-yr grid: 951 -> 216 ms; 37 walkers,
 // four modes, quarter-year grid: 2063 -> 917 us; one walker, (2,2), 30 days: 61 -> 35 us.
 #include "f32x2.cuh"
 #include "fixed.cuh"
@@ -380,12 +380,6 @@ __device__ __forceinline__ void phase_at(const Expand *__restrict__ e, uint32_t 
     p[3] = d3;
 }
 
-__device__ __forceinline__ void diff_next(Diff &r) {
-    r.v += r.d1;
-    r.d1 += r.d2;
-    r.d2 += r.d3;
-}
-
 // ------------------------------------------------------------------ integrand
 // x as two floats: x 2^-29 = a + b 2^-23 to 48 significant bits, |x| < 2^60
 __device__ __forceinline__ void fixed_pair(i64 x, float &a, float &b) {
@@ -702,11 +696,22 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                                         wm_.H[i][2 * c + 1][lane] = h1;
                                     }
                                 }
-                                ph[0] += ph[1];
-                                ph[1] += ph[2];
-                                ph[2] += ph[3];
+                                // only what the bins to come need: six of twelve additions
+                                if (i < kC - 1) {
+                                    ph[0] += ph[1];
 #pragma unroll
-                                for (int q = 0; q < kSer; q++) diff_next(s[q]);
+                                    for (int q = 0; q < kSer; q++) s[q].v += s[q].d1;
+                                }
+                                if (i < kC - 2) {
+                                    ph[1] += ph[2];
+#pragma unroll
+                                    for (int q = 0; q < kSer; q++) s[q].d1 += s[q].d2;
+                                }
+                                if (i < kC - 3) {
+                                    ph[2] += ph[3];
+#pragma unroll
+                                    for (int q = 0; q < kSer; q++) s[q].d2 += s[q].d3;
+                                }
                             }
                         }
                     }
