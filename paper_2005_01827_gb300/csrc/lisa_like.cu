@@ -336,26 +336,28 @@ lisa_status enqueue(lisa_like_t *h, const double *dparams, int B, double *lnL, d
         order_modes(d);
     }
     const StageBufs b = bufs_of(h, dparams);
-    const int tile = h->tune.threads * h->tune.per_thread;
     const bool split = h->precision == LISA_PREC_SPLIT;
+    DenseTune tune = h->tune;
+    if (!split && !h->rows) tune.group = 1;
+    const int tile = tune.threads * tune.per_thread;
     LCK(mark(0), "cudaEventRecord");
     LCK(split ? launch_knots_split(d, b, s) : launch_knots(d, b, s), "knot kernel launch");
     LCK(mark(1), "cudaEventRecord");
     LCK(split ? launch_spline_split(d, b, s) : launch_spline(d, b, s), "spline kernel launch");
     LCK(mark(2), "cudaEventRecord");
     if (split)
-        LCK(launch_segprep(d, b, h->segs, h->tune.per_thread, s), "segment kernel launch");
+        LCK(launch_segprep(d, b, h->segs, tune.per_thread, s), "segment kernel launch");
     else
         LCK(launch_phaseprep(d, b, h->phases, s), "segment kernel launch");
     LCK(mark(3), "cudaEventRecord");
-    LCK(launch_plan(d, b, tile, h->tune.group, s), "plan kernel launch");
+    LCK(launch_plan(d, b, tile, tune.group, s), "plan kernel launch");
     LCK(mark(4), "cudaEventRecord");
     if (split)
-        LCK(launch_dense_split(d, b, h->segs, h->bins32, h->tune, s), "dense kernel launch");
+        LCK(launch_dense_split(d, b, h->segs, h->bins32, tune, s), "dense kernel launch");
     else
-        LCK(launch_dense_f64(d, b, h->phases, h->bins, h->rows, h->tune, s), "dense kernel launch");
+        LCK(launch_dense_f64(d, b, h->phases, h->bins, h->rows, tune, s), "dense kernel launch");
     LCK(mark(5), "cudaEventRecord");
-    LCK(launch_finish(d, b, h->tune.group, split ? 1 : 0, h->dd, lnL, dh, hh, s),
+    LCK(launch_finish(d, b, tune.group, split ? 1 : 0, h->dd, lnL, dh, hh, s),
         "finish kernel launch");
     LCK(mark(6), "cudaEventRecord");
     h->last_launches = 8;  // source, knots, spline solve + coefficients, segments, plan, dense, finish
@@ -614,13 +616,22 @@ lisa_status lisa_like_set_data(lisa_like_t *h, double f0, double df, int64_t n_b
     float4 *rows = nullptr;
     const bool split = h->precision == LISA_PREC_SPLIT;
     if ((e = dalloc(&part, (size_t)items * 2)) != cudaSuccess ||
-        (split && (e = dalloc(&bins32, (size_t)kBinFloats * N)) != cudaSuccess) ||
-        (!split && (e = dalloc(&rows, (size_t)fx_chunks(N) * kFxWords)) != cudaSuccess)) {
+        (split && (e = dalloc(&bins32, (size_t)kBinFloats * N)) != cudaSuccess)) {
         if (part) cudaFree(part);
         cudaFree(bins);
         return cuda_fail(h, e, "device allocation (partial sums / dense data)");
     }
-    if ((e = split ? launch_prep_split(bins, N, bins32, s) : launch_prep_fx(bins, N, rows, s)) != cudaSuccess) {
+    // the FP64 kernel's own form of the data, where there is room for a second copy: without it
+    // rows are converted as they are used, one walker per item
+    if (!split && dalloc(&rows, (size_t)fx_chunks(N) * kFxWords) != cudaSuccess) {
+        rows = nullptr;
+        cudaGetLastError();
+    }
+    if (split)
+        e = launch_prep_split(bins, N, bins32, s);
+    else if (rows)
+        e = launch_prep_fx(bins, N, rows, s);
+    if (e != cudaSuccess) {
         cudaFree(part);
         if (bins32) cudaFree(bins32);
         if (rows) cudaFree(rows);
