@@ -127,7 +127,8 @@ cudaError_t launch_plan(const StageDims &d, const StageBufs &b, int tile_bins, i
 // 64 fractional bits of the three differences (words 4..6), which keep anchors deep
 // inside long segments exact to the FP64 value of the differences; the low 32 bits of
 // word 7 hold the first bin of the next segment (0x7fffffff for the last one), its high 32
-// bits the FP32 segment-guess constants: sc log2 f_lo in segment 0, sc = (K - 1) / log2(f_hi / f_lo) in segment 1 (0 beyond).
+// bits the FP32 segment-guess constants: sc log2 f_lo in segment 0, sc = (K - 1) /
+// log2(f_hi / f_lo) in segment 1 (0 beyond).
 constexpr int kPhaseWords = 8;
 
 // FP64 path: the phase records of all segments ([B][L][K-1][kPhaseWords]).

@@ -11,8 +11,8 @@
 //    that moves x by less than 1e-8 leaves 1e-16);
 //  * what is needed at several places or angles is evaluated in one pass, a lane for each: the
 //    ends of the peak's range, phase and slope at the band's ends and the peak, sines and cosines.
-// One walker, one mode: 80 -> 29 us (98 -> 38 with cold caches; two rounds of 31 points and up to six Newton steps in FP64, all
-// else one after another).
+// One walker, one mode: 80 -> 29 us (98 -> 38 with cold caches; before, 31 points twice and up to
+// six Newton steps in FP64 for each root, and all else one after another).
 #include "fixed.cuh"
 #include "kernels.h"
 #include "model.cuh"
@@ -296,7 +296,10 @@ __global__ void __launch_bounds__(128) source_kernel(StageDims d, StageBufs b) {
         const double gs = what == 1 ? (second ? 0.0 : h) : (second ? -2.0 * h : h);
         double o[5];
         harmonics(v, gc, gs, o);
-        double *dst = what == 0 ? c->kn[second] : what == 1 ? c->kq[second] : what == 2 ? c->wn[second] : c->un[second];
+        double *dst = what == 0   ? c->kn[second]
+                      : what == 1 ? c->kq[second]
+                      : what == 2 ? c->wn[second]
+                                  : c->un[second];
         const int n = what == 3 ? 3 : 5;
         for (int i = 0; i < n; i++) dst[i] = o[i];
     }
@@ -320,7 +323,8 @@ cudaError_t launch_source(const StageDims &d, const StageBufs &b, cudaStream_t s
 // harmonics, and the modes of equal m share all of it but their polarisation weights
 // (response.cuh), whose unit phasors and orbital angle are evaluated on the integer units and the
 // sines of small angles by series.  1024 walkers, six modes of 1024 knots: 8.4 -> 3.3 ms with the
-// source kernel (5.4 with one mode per thread, 4.0 with sincos() throughout).  One block of 128 threads per system left all but a few SMs idle in small
+// source kernel (5.4 with one mode per thread, 4.0 with sincos() throughout).  One block of 128
+// threads per system left all but a few SMs idle in small
 // calls (6 systems of 1024 knots: 246 us), hence one knot per thread.
 template <bool kSplit>
 __global__ void __launch_bounds__(128) knot_kernel(StageDims d, StageBufs b, double idf, double near) {
