@@ -61,7 +61,7 @@ constexpr int kNoScale = -10000;
 constexpr int kMinSeg = 8;
 
 // One (mode, segment) in a warp's block of bins, at the block's first bin or 3 bins before
-// the segment's (a thread's 4 bins may begin there): value and forward differences of the
+// the segment's first one (a thread's 4 bins may begin there): value and forward differences of the
 // seven series in fixed point, and (index kSer) of the phase in fractions of a turn scaled by
 // 2^64; l2, l3 and low hold the next 32 bits of the differences.
 struct __align__(16) Expand {
@@ -561,7 +561,10 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                                 const int k0 = __ldg(kb + seg);
                                 const int k1 =
                                     seg < K - 2 ? __ldg(kb + seg + 1) : s_hi[kp + u / L][d.ord[u % L]] + 1;
-                                const int org = max(Jw, k0 - (kC - 1)), nn = org - k0;
+                                // a band may begin one bin below its first knot's (1e-9 bins of
+                                // slack): no thread starts more than 3 bins before the lower of the two
+                                const int b0 = min(k0, s_lo[kp + u / L][d.ord[u % L]]);
+                                const int org = max(Jw, (seg == 0 ? b0 : k0) - (kC - 1)), nn = org - k0;
                                 e->org = org;
                                 e->kb = k0;
                                 e->next = k1;
