@@ -4,14 +4,17 @@
 // One block per (walker, mode) system; the unknowns are the second derivatives
 // M_1 .. M_{K-2} of each of the 8 series, not-a-knot eliminating M_0 and M_{K-1}.  The
 // matrix (shared by the series) has diagonal 2 (h_{i-1} + h_i) and off-diagonals h_{i-1},
-// h_i, so whatever a sweep starts from is forgotten by a factor of at least
-// h / (2 (h + h') - h c) per row, about 0.27 on the nearly even steps of log-spaced knots
-// (and below 0.36 for a step ratio up to 1.2): a row's value depends on rows kHalo = 32
-// away by less than 1e-14 of them, of the size of a sweep's own rounding.  So every thread
-// sweeps a chunk of rows of its own after kHalo rows of run-in, and a sweep of 1022 rows
-// takes 64 steps instead of 1022.  The pivots forget twice as fast and take 16 rows of
-// run-in.  (Few knots have large step ratios, up to 0.5 per row; up to K = 34 every row is
-// within the run-in of the last.)
+// h_i, so whatever a sweep starts from is forgotten by a factor of 1 / (1 + r + sqrt(1 + r + r^2))
+// a row for a step ratio r: 0.27 on the nearly even steps of many log-spaced knots.  So every
+// thread sweeps a chunk of rows of its own after a run-in of halo rows, and a sweep of 1022 rows
+// takes 64 steps instead of 1022.  The rows of the run-in grow towards low frequencies, M of the
+// phase as f^(-11/3), r^(11/3) a row: of the row's own value the run-in's start is left with
+// (r^(11/3) / (1 + r + sqrt(1 + r + r^2)))^halo.  With few knots that falls slowly (40 knots over five
+// decades: 0.7 a row), so below 192 knots the run-in is 64 rows, which is every row up to
+// K = 66, and 32 from there on: less than 4e-16 of a row's own value and 2e-15 rad of a phase of 1e5
+// rad, over up to six decades (with 32 throughout: 40 knots over four decades 6e-9 and 3e-11 rad, over five
+// 2e-6 and 8e-10 rad).  The pivots forget by r / (1 + r + sqrt(1 + r + r^2))^2, 0.07, a row and do not
+// grow: 16 rows.
 //
 // What bounds it: with few systems the latency of the sweep steps, so the series are dealt
 // to several blocks; with many systems the FP64 pipe (2 lanes per clock per SM): slopes and
@@ -29,7 +32,8 @@ namespace lisa {
 
 namespace {
 constexpr int kThreads = 256;
-constexpr int kHalo = 32;        // run-in rows of a sweep
+// run-in rows of a sweep
+__device__ __forceinline__ int sweep_halo(int K) { return K < 192 ? 64 : 32; }
 constexpr int kPivotHalo = 16;   // run-in rows of the pivots
 constexpr size_t kMaxSmem = 227 * 1024;
 }  // namespace
@@ -89,7 +93,7 @@ template <typename T>
 __device__ __forceinline__ void solve_stage(int stage, T &v, T *y, const T *h, const T *ih,
                                             const T *sd, const T *c, const Rows R, int t, int n) {
     const int C = R.mask + 1;
-    const int i0 = 1 + t * C, i1 = min(i0 + C, n - 1);
+    const int i0 = 1 + t * C, i1 = min(i0 + C, n - 1), halo = sweep_halo(n);
     if (stage == 4) {  // M_0 and M_{K-1} from their neighbours
         if (t != 0) return;
         const T h0 = h[R.at(0)], h1 = h[R.at(1)], ha = h[R.at(n - 3)], hb = h[R.at(n - 2)];
@@ -98,9 +102,9 @@ __device__ __forceinline__ void solve_stage(int stage, T &v, T *y, const T *h, c
         return;
     }
     if (i0 >= n - 1) return;
-    if (stage == 0) v = sweep_forward(y, sd, R, max(1, i0 - kHalo), i0, T(0), false);
+    if (stage == 0) v = sweep_forward(y, sd, R, max(1, i0 - halo), i0, T(0), false);
     if (stage == 1) sweep_forward(y, sd, R, i0, i1, v, true);
-    if (stage == 2) v = sweep_backward(y, c, R, i1, min(n - 1, i1 + kHalo), n, T(0), false);
+    if (stage == 2) v = sweep_backward(y, c, R, i1, min(n - 1, i1 + halo), n, T(0), false);
     if (stage == 3) sweep_backward(y, c, R, i0, i1, n, v, true);
 }
 
