@@ -337,14 +337,20 @@ __global__ void __launch_bounds__(NTH) flow_eval_kernel(FlowView f, const double
     first_weights(f, w, gen ? FC - 1 : 0);
     const int r = threadIdx.x >> 4, d = threadIdx.x & 15, row = blockIdx.x * TS + r;
     const int own = blockIdx.x * TS + threadIdx.x;  // threads 0 .. 15: one row each
+    double zz = 0.0;
     if (threadIdx.x < TS) {
         float *u = sm.u + threadIdx.x * LU;
         for (int j = 0; j < LU; j++) u[j] = 0.0f;
         if (own < n) {
-            if (gen)
-                for (int j = 0; j < FD; j++) u[j] = (float)in[(size_t)own * FD + j];
-            else
+            if (gen) {  // all of the input is read here: out may be in
+                for (int j = 0; j < FD; j++) {
+                    const double zv = in[(size_t)own * FD + j];
+                    u[j] = (float)zv;
+                    zz += zv * zv;
+                }
+            } else {
                 whiten_row(f, in + (size_t)own * FD, u);
+            }
         }
     }
     if (threadIdx.x >= NTH - 32) {
@@ -363,14 +369,7 @@ __global__ void __launch_bounds__(NTH) flow_eval_kernel(FlowView f, const double
         }
     }
     if (threadIdx.x < TS && own < n) {
-        double zz = 0.0, lq = 0.0;
-        if (gen) {
-            for (int j = 0; j < FD; j++) {
-                const double zv = in[(size_t)own * FD + j];
-                zz += zv * zv;
-            }
-            lq = -0.5 * zz - 0.5 * FD * kLog2Pi;
-        }
+        double lq = gen ? -0.5 * zz - 0.5 * FD * kLog2Pi : 0.0;
         for (int k = 0; k < FC; k++) {
             const int c = gen ? FC - 1 - k : k;
             lq -= (double)s_sum(sm.s[c][threadIdx.x], c);
