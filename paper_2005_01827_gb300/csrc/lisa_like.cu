@@ -646,6 +646,7 @@ lisa_status lisa_like_set_data(lisa_like_t *h, double f0, double df, int64_t n_b
         h->deferred.push_back(bins);
         return st;
     }
+    drop_graph(h);  // a captured graph holds the old buffers, grid and <d|d>
     if (h->bins) cudaFree(h->bins);
     if (h->bins32) cudaFree(h->bins32);
     if (h->rows) cudaFree(h->rows);
