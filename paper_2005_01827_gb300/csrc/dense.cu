@@ -14,12 +14,13 @@
 //   * the amplitude and the six transfer cubics are re-expanded in FP64 where a segment
 //     enters a warp's block of 128 bins, scaled by a power of two that bounds them over its
 //     bins there, and advance by 64-bit forward differences; A e^{i phase} T is summed over
-//     the modes in 64 bits, relative to the largest mode of the block and channel (2^-54 of
-//     it per term);
+//     the modes in 64 bits, in units of 2^-55 of the largest product of bounds of the block and
+//     channel: 2^-49 of its largest mode on most segments.  Bounds further above their values
+//     than kLoose bits are not used (dense_direct), so 2^-41 at worst;
 //   * the integrand is summed in FP32 pairs (48 bits: products with their exact errors,
 //     two-sums) over a thread's bins, and in FP64 from there up.
-// Terms are thus exact to about 1e-14 of the largest mode's, and the knots' FP64 phases
-// (1e-12 to 1e-9 rad) set the error as they did: against 64-bit sums of the same splines the
+// Terms are thus exact to about 2e-15 of the largest mode's on most segments, and the knots'
+// FP64 phases (1e-12 to 1e-9 rad) set the error as they did: against 64-bit sums of the same splines the
 // errors of ln L, <d|h> and <h|h> are those of the FP64 evaluation (1024 walkers: 7.1e-11
 // both).  Where a warp's bins hold a segment of fewer than 8 bins or more than 14 segments
 // of one mode, or a value is infinite, NaN or beyond the exponents handled, they are
@@ -59,6 +60,11 @@ constexpr int kNoScale = -10000;
 // Shortest segment for the expansions: over a bin or more per segment the differences no
 // longer fall with their order.
 constexpr int kMinSeg = 8;
+// Bits that the bounds of an amplitude and of a transfer together may lie above their values where
+// the expansion begins: the sums' unit is then at most 2^(kLoose - 53) of that product.  4 bits on most
+// segments and up to 9 from 64 knots up; with 4 to 32 knots and a few bins below the first bin
+// (f0 / df < 30) up to 17.
+constexpr int kLoose = 12;
 
 // One (mode, segment) in a warp's block of bins, at the block's first bin or 3 bins before
 // the segment's first one (a thread's 4 bins may begin there): value and forward differences of the
@@ -67,13 +73,11 @@ constexpr int kMinSeg = 8;
 struct __align__(16) Expand {
     i64 vd[kSer + 1][2];  // value, first difference
     i64 d2[kSer + 1];
-    int2 d3[kSer];        // third difference, l2
-    i64 ph3;              // third difference of the phase
-    uint32_t l3[kSer], low[3];
+    i64 d3[kSer + 1];
+    uint32_t l2[kSer], l3[kSer], low[3];
     int org, kb, next;    // origin, first bin of the segment and of the next one
-    int pad[3];
 };
-static_assert(sizeof(Expand) == 320, "16-byte loads of a series' value and first difference");
+static_assert(sizeof(Expand) == 336, "16-byte loads of a series' value and first difference");
 
 struct Phase64 {
     unsigned long long ph, d1, d2, d3;
@@ -311,11 +315,10 @@ __device__ __forceinline__ void differences(const double2 *__restrict__ c2, int 
     d[3] = 6.0 * p3;
 }
 
-// m with |v| < 2^m over 2^n1 bins, |v| <= |d0| + n |d1| + n^2/2 |d2| + n^3/6 |d3|; large enough
-// for the third difference to fit 32 bits
+// m with |v| < 2^m over 2^n1 bins, |v| <= |d0| + n |d1| + n^2/2 |d2| + n^3/6 |d3|
 __device__ __forceinline__ int bound_of(const double d[4], int n1) {
     return max(max(exponent_of(d[0]), exponent_of(d[1]) + n1),
-               max(exponent_of(d[2]) + 2 * n1 - 1, exponent_of(d[3]) + max(3 * n1 - 2, 30))) +
+               max(exponent_of(d[2]) + 2 * n1 - 1, exponent_of(d[3]) + 3 * n1 - 2)) +
            2;
 }
 
@@ -325,41 +328,36 @@ __device__ __forceinline__ void series_put(Expand *e, int q, const double d[4], 
     e->vd[q][0] = __double_as_longlong(d[0]);
     e->vd[q][1] = __double_as_longlong(d[1]);
     e->d2[q] = __double_as_longlong(d[2]);
-    e->d3[q] = make_int2(__double2loint(d[3]), __double2hiint(d[3]));
+    e->d3[q] = __double_as_longlong(d[3]);
     e->l3[q] = (uint32_t)bound;
 }
 
 __device__ __forceinline__ void series_fix(Expand *e, int q, int s) {
-    uint32_t l2, l3;
     e->vd[q][0] = to_fixed(__longlong_as_double(e->vd[q][0]), s);
     e->vd[q][1] = to_fixed(__longlong_as_double(e->vd[q][1]), s);
-    e->d2[q] = to_fixed96(__longlong_as_double(e->d2[q]), s, l2);
-    e->d3[q] = make_int2((int)to_fixed96(__hiloint2double(e->d3[q].y, e->d3[q].x), s, l3), (int)l2);
-    e->l3[q] = l3;
+    e->d2[q] = to_fixed96(__longlong_as_double(e->d2[q]), s, e->l2[q]);
+    e->d3[q] = to_fixed96(__longlong_as_double(e->d3[q]), s, e->l3[q]);
 }
 
 struct Diff {
     i64 v, d1, d2;
-    int d3;
 };
 
 // series q n >= 0 bins from its origin; c2 = n(n-1)/2, c3 = n(n-1)(n-2)/6
 __device__ __forceinline__ Diff series_at(const Expand *__restrict__ e, int q, uint32_t n, uint32_t c2,
                                           uint32_t c3) {
     const longlong2 a = *reinterpret_cast<const longlong2 *>(e->vd[q]);
-    const i64 d2 = e->d2[q];
-    const int2 t = e->d3[q];
+    const i64 d2 = e->d2[q], d3 = e->d3[q];
     Diff r;
     i64 v = mad_u((uint32_t)a.y, n, a.x);
     v = mad_u((uint32_t)d2, c2, v);
-    v = mad_s(t.x, (int)c3, v);
-    v += (i64)(__umulhi(c2, (uint32_t)t.y) + __umulhi(c3, e->l3[q]));
-    r.v = add_hi(v, (uint32_t)(a.y >> 32) * n + (uint32_t)(d2 >> 32) * c2);
+    v = mad_u((uint32_t)d3, c3, v);
+    v += (i64)(__umulhi(c2, e->l2[q]) + __umulhi(c3, e->l3[q]));
+    r.v = add_hi(v, (uint32_t)(a.y >> 32) * n + (uint32_t)(d2 >> 32) * c2 + (uint32_t)(d3 >> 32) * c3);
     i64 d1 = mad_u((uint32_t)d2, n, a.y);
-    d1 = mad_s(t.x, (int)c2, d1);
-    r.d1 = add_hi(d1, (uint32_t)(d2 >> 32) * n);
-    r.d2 = mad_s(t.x, (int)n, d2);
-    r.d3 = t.x;
+    d1 = mad_u((uint32_t)d3, c2, d1);
+    r.d1 = add_hi(d1, (uint32_t)(d2 >> 32) * n + (uint32_t)(d3 >> 32) * c2);
+    r.d2 = add_hi(mad_u((uint32_t)d3, n, d2), (uint32_t)(d3 >> 32) * n);
     return r;
 }
 
@@ -367,7 +365,7 @@ __device__ __forceinline__ Diff series_at(const Expand *__restrict__ e, int q, u
 __device__ __forceinline__ void phase_at(const Expand *__restrict__ e, uint32_t n, uint32_t c2, uint32_t c3,
                                          i64 p[4]) {
     const longlong2 a = *reinterpret_cast<const longlong2 *>(e->vd[kSer]);
-    const i64 d2 = e->d2[kSer], d3 = e->ph3;
+    const i64 d2 = e->d2[kSer], d3 = e->d3[kSer];
     i64 v = mad_u((uint32_t)a.y, n, a.x);
     v = mad_u((uint32_t)d2, c2, v);
     v = mad_u((uint32_t)d3, c3, v);
@@ -574,7 +572,7 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                                 e->vd[kSer][0] = p.ph;
                                 e->vd[kSer][1] = p.d1;
                                 e->d2[kSer] = p.d2;
-                                e->ph3 = p.d3;
+                                e->d3[kSer] = p.d3;
                                 e->low[0] = (uint32_t)((r[4] + (i64)nn * r[5] + c2 * r[6]) >> 32);
                                 e->low[1] = (uint32_t)((r[5] + (i64)nn * r[6]) >> 32);
                                 e->low[2] = (uint32_t)(r[6] >> 32);
@@ -602,14 +600,19 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                                 const Expand *e = ex + lane;
                                 ts = (s_task[warp][lane] & 15) / L;
                                 ea = (int)e->l3[0];
-                                int top = ea;
+                                auto at0 = [&](int q) { return exponent_of(__longlong_as_double(e->vd[q][0])); };
+                                int top = ea, loose = 0;
 #pragma unroll
                                 for (int c = 0; c < 3; c++) {
                                     et[c] = max((int)e->l3[1 + 2 * c], (int)e->l3[2 + 2 * c]);
                                     top = max(top, et[c]);
+                                    if (et[c] > -1900)  // not all zero
+                                        loose = max(loose, et[c] - max(at0(1 + 2 * c), at0(2 + 2 * c)));
                                 }
-                                // a short segment, or an infinite or NaN coefficient
-                                bad = e->next - e->kb < kMinSeg || top > 900;
+                                // a short segment, an infinite or NaN coefficient, or bounds far
+                                // above the values
+                                if (ea > -1900) loose += ea - at0(0);
+                                bad = e->next - e->kb < kMinSeg || top > 900 || loose > kLoose;
                             }
                             const unsigned wrong = __ballot_sync(0xffffffffu, bad);
                             const unsigned of_next = __ballot_sync(0xffffffffu, lane < tasks && ts > sub);
@@ -713,7 +716,7 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                                 if (i < kC - 3) {
                                     ph[2] += ph[3];
 #pragma unroll
-                                    for (int q = 0; q < kSer; q++) s[q].d2 += s[q].d3;
+                                    for (int q = 0; q < kSer; q++) s[q].d2 += e->d3[q];
                                 }
                             }
                         }
