@@ -17,8 +17,10 @@
 //     the modes in 64 bits, in units of 2^-55 of the largest product of bounds of the block and
 //     channel: 2^-49 of its largest mode on most segments.  Bounds further above their values
 //     than kLoose bits are not used (dense_direct), so 2^-41 at worst;
-//   * the integrand is summed in FP32 pairs (48 bits: products with their exact errors,
-//     two-sums) over a thread's bins, and in FP64 from there up.
+//   * the integrand is summed in FP32 pairs over a thread's bins, and in FP64 from there up:
+//     h rounded to 8 units of its sum (2^-46 of the largest mode, without a bias), w and w d to 48
+//     bits; products with their errors and two-sums, what these leave summed in plain FP32
+//     (2^-45 of a thread's sum).
 // Terms are thus exact to about 2e-15 of the largest mode's on most segments, and the knots'
 // FP64 phases (1e-12 to 1e-9 rad) set the error as they did: against 64-bit sums of the same splines the
 // errors of ln L, <d|h> and <h|h> are those of the FP64 evaluation (1024 walkers: 7.1e-11
@@ -379,13 +381,17 @@ __device__ __forceinline__ void phase_at(const Expand *__restrict__ e, uint32_t 
 }
 
 // ------------------------------------------------------------------ integrand
-// x as two floats: x 2^-29 = a + b 2^-23 to 48 significant bits, |x| < 2^60
+// Sums begin at half a unit of fixed_pair, which cuts off what is below: it rounds then
+constexpr i64 kHalf = 4;
+
+// x - kHalf as two floats, x 2^-27 = a + b 2^-24 to a unit of 2^3 in x.  |x| < 2^58: a cubic stays below
+// 0.92 of its bound (bound_of), so a mode's |A T| below 1.2 2^55 units, and there are six
 __device__ __forceinline__ void fixed_pair(i64 x, float &a, float &b) {
-    const int hi = (int)(x >> 29);
+    const int hi = (int)(x >> 27);
     a = __int2float_rn(hi);
     const int rest = hi - __float2int_rn(a);  // |rest| <= 64
-    // (rest 2^29 + low 29 bits) 2^-6, below 2^30
-    const int r = (int)(((unsigned int)rest << 23) | (((unsigned int)x & 0x1fffffffu) >> 6));
+    // (rest 2^27 + low 27 bits) 2^-3, at most 2^30 + 2^24
+    const int r = (int)(((unsigned int)rest << 24) + (((unsigned int)x & 0x7ffffffu) >> 3));
     b = __int2float_rn(r);
 }
 
@@ -528,7 +534,7 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
 #pragma unroll
                     for (int i = 0; i < kC; i++)
 #pragma unroll
-                        for (int q = 0; q < 6; q++) wm_.H[i][q][lane] = 0;
+                        for (int q = 0; q < 6; q++) wm_.H[i][q][lane] = kHalf;
 #pragma unroll 1
                     for (int pos = 0; pos < L; pos++) {
                         const int unit = sub * L + pos, mi = d.ord[pos];
@@ -630,8 +636,10 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                                 if (m > E[c]) {
                                     if (pos > 0 && E[c] > kNoScale)
                                         for (int i = 0; i < kC; i++)
-                                            for (int q = 2 * c; q < 2 * c + 2; q++)
-                                                wm_.H[i][q][lane] >>= min(m - E[c], 63);
+                                            for (int q = 2 * c; q < 2 * c + 2; q++) {
+                                                i64 &h = wm_.H[i][q][lane];
+                                                h = ((h - kHalf) >> min(m - E[c], 63)) + kHalf;
+                                            }
                                     E[c] = m;
                                 }
                                 En[c] = max(En[c], mn);
@@ -778,15 +786,15 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                                     float2 x, y;  // h = x + y
                                     fixed_pair(wm_.H[i][2 * c][lane], x.x, y.x);
                                     fixed_pair(wm_.H[i][2 * c + 1][lane], x.y, y.y);
-                                    const float s23 = 1.1920928955078125e-7f;  // 2^-23
-                                    y = mul2(y, make_float2(s23, s23));
+                                    const float s24 = 5.9604644775390625e-8f;  // 2^-24
+                                    y = mul2(y, make_float2(s24, s24));
                                     const float2 wh = make_float2(q[2 * c], q[2 * c]);
                                     const float2 wl = make_float2(q[2 * c + 1], q[2 * c + 1]);
                                     const float2 eh = make_float2(q[6 + 4 * c], q[7 + 4 * c]);
                                     const float2 el = make_float2(q[8 + 4 * c], q[9 + 4 * c]);
                                     // w |h|^2
                                     const float2 p = mul2(x, x);
-                                    const float2 pe = fma2(add2(add2(x, x), y), y, fma2(x, x, neg2(p)));
+                                    const float2 pe = fma2(add2(x, x), y, fma2(y, y, fma2(x, x, neg2(p))));
                                     const float2 u = mul2(wh, p);
                                     float2 ue = fma2(wh, p, neg2(u));
                                     ue = fma2(wl, p, ue);
@@ -799,12 +807,12 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                                 }
                             }
                         }
-                        // h = (x + y) 2^(E - 26)
+                        // h = (x + y) 2^(E - 28)
 #pragma unroll
                         for (int c = 0; c < 3; c++) {
                             if (E[c] == kNoScale) continue;
-                            hh += scaled_sum(hs[c], hc[c], ew[c] + 2 * (E[c] - 26));
-                            dh += scaled_sum(ds[c], dc[c], ed[c] + E[c] - 26);
+                            hh += scaled_sum(hs[c], hc[c], ew[c] + 2 * (E[c] - 28));
+                            dh += scaled_sum(ds[c], dc[c], ed[c] + E[c] - 28);
                         }
                     } else if (mine > 0) {
                         const double2 r = dense_direct(d, b, segs, bins, w, j0, j0 + mine, s_lo[k], s_hi[k]);
