@@ -21,7 +21,11 @@
 //    34 instructions a bin and m, against 43 a bin and mode with A and T evaluated per mode;
 //  * the segment and 64-bit phase anchor of all a group's (walker, m) in a warp's bins are found
 //    by one lane each, once per item; warps with a segment's end in them, bands that end there
-//    and short segments take a general path, thread by thread.
+//    and short segments take a general path, thread by thread.  There a segment's bins alone are
+//    evaluated where it has no quartics (a chunk may hold several such segments), and segments
+//    without bins are passed over by their bounds, 4 bytes each: calls
+//    of 128 heavy walkers on a week's grid of 12036 bins, 1024 knots 4.59 -> 1.77 ms, 4096 knots
+//    21.5 -> 9.0 ms, of the 1024 walkers below 25.87 -> 25.56 ms.
 // 1024 walkers, six modes, year's grid: prior 31.3 -> 20.2 ms, posterior 14.7 -> 9.9 ms;
 // 8192 walkers 229 -> 147 ms.  128-thread blocks, four per SM: two blocks of 256 threads that
 // share a tile took 23.5 against 22.1 ms (longer barrier waits).
@@ -351,6 +355,13 @@ __device__ __forceinline__ void load_series(const GroupRec *__restrict__ r, Segm
         const float4 u = x[(i + 1) >> 1];
         o.s[i / 6][i % 6] = (i & 1) ? make_float2(u.x, u.y) : make_float2(u.z, u.w);
     }
+}
+
+// its first bin and ok alone
+__device__ __forceinline__ void load_head(const GroupRec *__restrict__ r, Segment &o) {
+    const int2 v = __ldg(reinterpret_cast<const int2 *>(&r->kb0));
+    o.kb0 = v.x;
+    o.ok = v.y;
 }
 
 // forward differences of the segment's phase moved from its first bin to bin n, which may
@@ -738,21 +749,24 @@ __global__ void __launch_bounds__(128, 4) dense_split_kernel(StageDims d, StageB
                 s = min(max(s, 0), K - 2);
                 const GroupRec *rec = record_at(b.coef, base + s);
                 SegPhase q = load_phase(rec);
-                load_series(rec, r);
-                // the record of the guessed segment is loaded with the bounds that check it,
-                // so a right guess (the usual case) costs no dependent load
+                load_head(rec, r);
+                // the record of the guessed segment is fetched with the bounds that check it (its
+                // other cache line ahead of its use, which a segment without quartics has none for),
+                // so a right guess (the usual case) costs no load from L2 after another
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(&rec->s[1][4]));
                 if ((s > 0 && r.kb0 > ja) || seg_next(q) <= ja) {  // the guess missed: search
                     const int *kb = b.kb + ((size_t)w * d.L + d.ord[s_first[mi]]) * K;
                     s = seg_guess(kb, K, ja, fa, s_flo[k][mi], s_scl[k][mi]);
                     rec = record_at(b.coef, base + s);
                     q = load_phase(rec);
-                    load_series(rec, r);
+                    load_head(rec, r);
                 }
                 r.next = seg_next(q);
                 p = phase_at(q, j0 - r.kb0);
                 for (;;) {  // the chunk's segments, usually one
                     const int to = min(jb, r.next);
                     if (r.ok) {
+                        load_series(rec, r);
                         expand_at(r, (float)(j0 - r.kb0) + 0.5f * (C - 1), e);
 #pragma unroll
                         for (int i = 0; i < C; i++) bin(i, j0 + i >= ja && j0 + i < to);
@@ -765,24 +779,28 @@ __global__ void __launch_bounds__(128, 4) dense_split_kernel(StageDims d, StageB
 #pragma unroll
                             for (int i = 0; i < C; i++) {
                                 const int j = j0 + i;
-                                const float t = (float)(j - r.kb0) * o.invw;
-                                const bool in = j >= ja && j < to;
-                                float amp;
-                                float2 tr[3];
-                                eval_series(o, make_float2(t, t), amp, tr);
-                                float zr, zi;
-                                phasor(pm.ph, tab, zr, zi);
-                                add_mode(in ? zr * amp : 0.0f, in ? zi * amp : 0.0f, tr, hr[i], hm[i]);
+                                if (j >= ja && j < to) {
+                                    const float t = (float)(j - r.kb0) * o.invw;
+                                    float amp;
+                                    float2 tr[3];
+                                    eval_series(o, make_float2(t, t), amp, tr);
+                                    float zr, zi;
+                                    phasor(pm.ph, tab, zr, zi);
+                                    add_mode(zr * amp, zi * amp, tr, hr[i], hm[i]);
+                                }
                                 phase_next(pm);
                             }
                         }
                     }
                     ja = max(ja, to);
                     if (ja >= jb) break;
-                    s++;
+                    const int *kb = b.kb + ((size_t)w * d.L + d.ord[s_first[mi]]) * K;
+                    do
+                        s++;
+                    while (s < K - 2 && __ldg(kb + s + 1) <= ja);  // segments without bins
                     rec = record_at(b.coef, base + s);
                     q = load_phase(rec);
-                    load_series(rec, r);
+                    load_head(rec, r);
                     r.next = seg_next(q);
                     p = phase_at(q, j0 - r.kb0);
                 }
