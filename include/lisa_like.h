@@ -78,7 +78,10 @@ lisa_status lisa_like_create(const lisa_like_config *cfg, lisa_like_t **out);
  *   f0 > 0, df > 0: the grid f_j = f0 + j df, j = 0 .. n_bins-1, 1 <= n_bins < 2^31.
  *   d   host double[3][n_bins][2], the A, E, T data d~(f_j); NULL means d = 0.
  *   psd host double[3][n_bins], one-sided S_n^{A,E,T}(f_j) > 0 and finite.
- * Stores w = 4 df / S and w d on the device and computes <d|d> (FP64).
+ * Stores w = 4 df / S and w d on the device and computes <d|d> (FP64).  An FP64 handle keeps a
+ * second copy in the dense kernel's own form (76 bytes a bin) where the device has room for it and
+ * as much again; without it calls run one walker per work item and convert the data as they go.
+ * The copy is given back when a later set_data or template needs its room.
  * Errors: LISA_ERR_ARG (NULL psd, non-finite value, S <= 0, bad grid). */
 lisa_status lisa_like_set_data(lisa_like_t *h, double f0, double df, int64_t n_bins,
                                const double *d, const double *psd);
@@ -191,13 +194,14 @@ lisa_status lisa_like_set_graphs(lisa_like_t *h, int on);
 /* Tile shape of the fused dense kernel: tiles of 128 x per_thread bins and `group` walkers
  * per work item.
  * Supported: (8,8), (4,8), (16,8) in split precision only, (8,1).  LISA_ERR_ARG
- * otherwise.  out[3] of get_tune: per_thread, group, persistent blocks. */
+ * otherwise.  out[3] of get_tune: per_thread, group, persistent blocks, as calls run now (group 1
+ * in an FP64 handle without its second copy of the data, see lisa_like_set_data). */
 lisa_status lisa_like_set_tune(lisa_like_t *h, int per_thread, int group);
 lisa_status lisa_like_get_tune(const lisa_like_t *h, int *out);
 
 /* Autotuner: times every supported tile shape on the full call for these B host
  * walkers (a representative sample is enough), keeps the fastest, and caches the
- * choice per (n_bins, n_knots, precision) in the handle; later calls with the same
+ * choice per (n_bins, n_knots, precision, second copy or not) in the handle; later calls with the same
  * key reuse it without timing.  out[3] (or NULL) receives the chosen shape.
  * Requires set_data. */
 lisa_status lisa_like_autotune(lisa_like_t *h, const double *params, int B, int *out);

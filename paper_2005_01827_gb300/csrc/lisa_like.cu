@@ -75,8 +75,8 @@ struct lisa_like {
     const void *g_key[4] = {nullptr, nullptr, nullptr, nullptr};
     int g_launches = 0;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
-    // tile shapes chosen by lisa_like_autotune, per (n_bins, K, precision)
-    std::map<std::tuple<int, int, int>, DenseTune> tuned;
+    // tile shapes chosen by lisa_like_autotune, per (n_bins, K, precision, rows)
+    std::map<std::tuple<int, int, int, bool>, DenseTune> tuned;
     bool profiling = false;
     unsigned wait_test_polls = 0;      // lisa_like_test_device_wait
     lisa::RbState *rb = nullptr;       // relative binning (lisa_like_set_fiducial)
@@ -109,7 +109,12 @@ lisa_status cuda_fail(lisa_like_t *h, cudaError_t e, const char *what) {
 template <typename T>
 cudaError_t dalloc(T **p, size_t n) {
     if (getenv("LISA_LIKE_INJECT_OOM")) return cudaErrorMemoryAllocation;
-    return cudaMalloc((void **)p, n * sizeof(T) + 16);
+    const cudaError_t e = cudaMalloc((void **)p, n * sizeof(T) + 16);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();  // the caller reports it; the next launch has not failed
+    }
+    return e;
 }
 
 void free_batch(lisa_like_t *h) {
@@ -262,6 +267,13 @@ bool make_tune(const lisa_like_t *h, int per_thread, int group, DenseTune *t) {
     return true;
 }
 
+// the shape that runs: without the second copy of the data the FP64 kernel takes one walker per item
+DenseTune tune_of(const lisa_like_t *h) {
+    DenseTune t = h->tune;
+    if (h->precision != LISA_PREC_SPLIT && h->have_data && !h->rows) t.group = 1;
+    return t;
+}
+
 lisa_status enqueue(lisa_like_t *h, const double *dparams, int B, double *lnL, double *dh,
                     double *hh, cudaStream_t s, bool profile, unsigned mode_mask = 0);
 
@@ -269,6 +281,54 @@ void drop_graph(lisa_like_t *h) {
     if (h->gexec) cudaGraphExecDestroy(h->gexec);
     h->gexec = nullptr;
     h->g_B = 0;
+}
+
+// The data in the FP64 dense kernel's own form, on stream s, where there is room for a second copy and
+// as much again (it only makes calls faster: what the handle, samplers and other users of the
+// device allocate later comes first); NULL otherwise.  LISA_LIKE_ONE_COPY=1: never (for tests).
+cudaError_t make_rows(const double *bins, int N, float4 **rows, cudaStream_t s) {
+    const size_t n = (size_t)fx_chunks(N) * kFxWords;
+    size_t room = 0, total = 0;
+    *rows = nullptr;
+    if (getenv("LISA_LIKE_ONE_COPY") || cudaMemGetInfo(&room, &total) != cudaSuccess ||
+        room < 2 * n * sizeof(float4) || dalloc(rows, n) != cudaSuccess)
+        return cudaSuccess;
+    const cudaError_t e = launch_prep_fx(bins, N, *rows, s);
+    if (e != cudaSuccess) {
+        cudaFree(*rows);
+        *rows = nullptr;
+    }
+    return e;
+}
+
+// device memory that comes before the second copy of the data: where there is none left, the copy
+// is given back
+template <typename T>
+cudaError_t dalloc_first(lisa_like_t *h, T **p, size_t n) {
+    cudaError_t e = dalloc(p, n);
+    if (e == cudaErrorMemoryAllocation && h->rows) {
+        cudaFree(h->rows);  // after all work in flight
+        h->rows = nullptr;
+        drop_graph(h);
+        e = dalloc(p, n);
+    }
+    return e;
+}
+
+lisa_status rows_back(lisa_like_t *h, bool had, lisa_status st) {
+    if (!had || h->rows || (st != LISA_OK && st != LISA_ERR_OOM)) return st;
+    float4 *rows = nullptr;
+    const std::string err = h->err;
+    if (make_rows(h->bins, h->N, &rows, h->stream) == cudaSuccess && rows) {
+        if (wait_for(h, h->stream) == LISA_OK) {
+            h->rows = rows;
+            drop_graph(h);
+        } else {
+            h->deferred.push_back(rows);
+        }
+    }
+    h->err = err;
+    return st;
 }
 
 lisa_status run_all(lisa_like_t *h, const double *dparams, int B, double *lnL, double *dh,
@@ -337,8 +397,7 @@ lisa_status enqueue(lisa_like_t *h, const double *dparams, int B, double *lnL, d
     }
     const StageBufs b = bufs_of(h, dparams);
     const bool split = h->precision == LISA_PREC_SPLIT;
-    DenseTune tune = h->tune;
-    if (!split && !h->rows) tune.group = 1;
+    const DenseTune tune = tune_of(h);
     const int tile = tune.threads * tune.per_thread;
     LCK(mark(0), "cudaEventRecord");
     LCK(split ? launch_knots_split(d, b, s) : launch_knots(d, b, s), "knot kernel launch");
@@ -536,9 +595,8 @@ lisa_status lisa_like_create(const lisa_like_config *cfg, lisa_like_t **out) {
     return LISA_OK;
 }
 
-lisa_status lisa_like_set_data(lisa_like_t *h, double f0, double df, int64_t n_bins,
-                               const double *d, const double *psd) {
-    if (!h) return LISA_ERR_ARG;
+static lisa_status set_data(lisa_like_t *h, double f0, double df, int64_t n_bins, const double *d,
+                            const double *psd) {
     if (!psd) return fail(h, LISA_ERR_ARG, "psd must not be NULL");
     if (!(f0 > 0.0) || !std::isfinite(f0) || !(df > 0.0) || !std::isfinite(df))
         return fail(h, LISA_ERR_ARG, "grid needs finite f0 > 0 and df > 0");
@@ -558,10 +616,11 @@ lisa_status lisa_like_set_data(lisa_like_t *h, double f0, double df, int64_t n_b
         if (bins) cudaFree(bins);
     };
     cudaError_t e;
-    if ((e = dalloc(&psd_dev, (size_t)3 * N)) != cudaSuccess ||
-        (d && (e = dalloc(&dd_dev, (size_t)6 * N)) != cudaSuccess) ||
-        (e = dalloc(&bins, (size_t)kBinDoubles * N)) != cudaSuccess ||
-        (e = dalloc(&ddpart, (size_t)nblk)) != cudaSuccess || (e = dalloc(&bad, 1)) != cudaSuccess) {
+    if ((e = dalloc_first(h, &psd_dev, (size_t)3 * N)) != cudaSuccess ||
+        (d && (e = dalloc_first(h, &dd_dev, (size_t)6 * N)) != cudaSuccess) ||
+        (e = dalloc_first(h, &bins, (size_t)kBinDoubles * N)) != cudaSuccess ||
+        (e = dalloc_first(h, &ddpart, (size_t)nblk)) != cudaSuccess ||
+        (e = dalloc_first(h, &bad, 1)) != cudaSuccess) {
         cleanup();
         return cuda_fail(h, e, "device allocation (data)");
     }
@@ -615,22 +674,14 @@ lisa_status lisa_like_set_data(lisa_like_t *h, double f0, double df, int64_t n_b
     float *bins32 = nullptr;
     float4 *rows = nullptr;
     const bool split = h->precision == LISA_PREC_SPLIT;
-    if ((e = dalloc(&part, (size_t)items * 2)) != cudaSuccess ||
+    if ((e = dalloc_first(h, &part, (size_t)items * 2)) != cudaSuccess ||
         (split && (e = dalloc(&bins32, (size_t)kBinFloats * N)) != cudaSuccess)) {
         if (part) cudaFree(part);
         cudaFree(bins);
         return cuda_fail(h, e, "device allocation (partial sums / dense data)");
     }
-    // the FP64 kernel's own form of the data, where there is room for a second copy: without it
-    // rows are converted as they are used, one walker per item
-    if (!split && dalloc(&rows, (size_t)fx_chunks(N) * kFxWords) != cudaSuccess) {
-        rows = nullptr;
-        cudaGetLastError();
-    }
-    if (split)
-        e = launch_prep_split(bins, N, bins32, s);
-    else if (rows)
-        e = launch_prep_fx(bins, N, rows, s);
+    // (the present data stay until the new ones are ready)
+    e = split ? launch_prep_split(bins, N, bins32, s) : make_rows(bins, N, &rows, s);
     if (e != cudaSuccess) {
         cudaFree(part);
         if (bins32) cudaFree(bins32);
@@ -666,6 +717,15 @@ lisa_status lisa_like_set_data(lisa_like_t *h, double f0, double df, int64_t n_b
     h->dd = ddv;
     h->have_data = true;
     return LISA_OK;
+}
+
+lisa_status lisa_like_set_data(lisa_like_t *h, double f0, double df, int64_t n_bins,
+                               const double *d, const double *psd) {
+    if (!h) return LISA_ERR_ARG;
+    const bool had = h->rows != nullptr;
+    const lisa_status st = set_data(h, f0, df, n_bins, d, psd);
+    // with the old data gone there may be room again; after a failure the old data are still there
+    return rows_back(h, had || (st == LISA_OK && h->precision != LISA_PREC_SPLIT), st);
 }
 
 lisa_status lisa_like_loglike_device(lisa_like_t *h, const double *d_params, int B, double *d_lnL,
@@ -768,7 +828,8 @@ lisa_status lisa_like_template(lisa_like_t *h, const double *params, double *out
     lisa_status st = run_front(h, h->params, 1, s, &nl);
     if (st != LISA_OK) return st;
     double *dev = nullptr;
-    LCK(dalloc(&dev, (size_t)6 * h->N), "device allocation (template)");
+    const bool had = h->rows != nullptr;
+    LCK(dalloc_first(h, &dev, (size_t)6 * h->N), "device allocation (template)");
     cudaError_t e = launch_template(dims_of(h, 1), bufs_of(h, h->params), dev, s);
     if (!e) e = cudaMemcpyAsync(out, dev, sizeof(double) * 6 * h->N, cudaMemcpyDeviceToHost, s);
     if (e) {
@@ -780,7 +841,7 @@ lisa_status lisa_like_template(lisa_like_t *h, const double *params, double *out
         cudaFree(dev);
     else
         h->deferred.push_back(dev);
-    return st;
+    return rows_back(h, had, st);
 }
 
 lisa_status lisa_like_set_profiling(lisa_like_t *h, int on) {
@@ -845,9 +906,10 @@ lisa_status lisa_like_set_tune(lisa_like_t *h, int per_thread, int group) {
 
 lisa_status lisa_like_get_tune(const lisa_like_t *h, int *out) {
     if (!h || !out) return LISA_ERR_ARG;
-    out[0] = h->tune.per_thread;
-    out[1] = h->tune.group;
-    out[2] = h->tune.blocks;
+    const DenseTune t = tune_of(h);
+    out[0] = t.per_thread;
+    out[1] = t.group;
+    out[2] = t.blocks;
     return LISA_OK;
 }
 
@@ -856,7 +918,7 @@ lisa_status lisa_like_autotune(lisa_like_t *h, const double *params, int B, int 
     if (!h->have_data) return fail(h, LISA_ERR_STATE, "set_data must be called first");
     if (B < 1 || B > h->max_batch || !params) return fail(h, LISA_ERR_ARG, "bad batch");
     LCK(cudaSetDevice(h->device), "cudaSetDevice");
-    const auto key = std::make_tuple(h->N, h->K, h->precision);
+    const auto key = std::make_tuple(h->N, h->K, h->precision, h->rows != nullptr);
     auto it = h->tuned.find(key);
     if (it == h->tuned.end()) {
         cudaStream_t s = h->stream;
@@ -896,12 +958,7 @@ lisa_status lisa_like_autotune(lisa_like_t *h, const double *params, int B, int 
     }
     h->tune = it->second;
     drop_graph(h);
-    if (out) {
-        out[0] = h->tune.per_thread;
-        out[1] = h->tune.group;
-        out[2] = h->tune.blocks;
-    }
-    return LISA_OK;
+    return out ? lisa_like_get_tune(h, out) : LISA_OK;
 }
 
 lisa_status lisa_like_mode_inner(lisa_like_t *h, const double *params, int B, double *dh_modes,
