@@ -147,6 +147,7 @@ cudaError_t launch_template(const StageDims &d, const StageBufs &b, double *out,
                             cudaStream_t s);
 cudaError_t launch_prep(const double *d, const double *psd, int N, double df, double *bins,
                         double *ddpart, int *bad, cudaStream_t s);
+constexpr int kPrepBlocks = 4096;  // at most
 int prep_blocks(int N);
 
 // Resident blocks per SM of a dense-kernel variant (0 if the variant does not exist).

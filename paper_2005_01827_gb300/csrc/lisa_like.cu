@@ -66,6 +66,7 @@ struct lisa_like {
     int64_t part_items = 0;
     double *h_params = nullptr, *h_out = nullptr;  // pinned staging
     int *h_err = nullptr;
+    double *h_dd = nullptr;  // set_data's: partial <d|d> sums and the flag of bad data
     int last_launches = 0;
     std::vector<void *> deferred;  // device buffers that in-flight work may still touch
     // CUDA graphs: one cached executable for the last (B, pointers) key
@@ -137,6 +138,8 @@ void free_batch(lisa_like_t *h) {
     if (h->h_params) cudaFreeHost(h->h_params);
     if (h->h_out) cudaFreeHost(h->h_out);
     if (h->h_err) cudaFreeHost(h->h_err);
+    if (h->h_dd) cudaFreeHost(h->h_dd);
+    h->h_dd = nullptr;
     h->h_params = h->h_out = nullptr;
     h->h_err = nullptr;
 }
@@ -286,11 +289,13 @@ void drop_graph(lisa_like_t *h) {
 // The data in the FP64 dense kernel's own form, on stream s, where there is room for a second copy and
 // as much again (it only makes calls faster: what the handle, samplers and other users of the
 // device allocate later comes first); NULL otherwise.  LISA_LIKE_ONE_COPY=1: never (for tests).
+bool one_copy() { return getenv("LISA_LIKE_ONE_COPY") != nullptr; }
+
 cudaError_t make_rows(const double *bins, int N, float4 **rows, cudaStream_t s) {
     const size_t n = (size_t)fx_chunks(N) * kFxWords;
     size_t room = 0, total = 0;
     *rows = nullptr;
-    if (getenv("LISA_LIKE_ONE_COPY") || cudaMemGetInfo(&room, &total) != cudaSuccess ||
+    if (one_copy() || cudaMemGetInfo(&room, &total) != cudaSuccess ||
         room < 2 * n * sizeof(float4) || dalloc(rows, n) != cudaSuccess)
         return cudaSuccess;
     const cudaError_t e = launch_prep_fx(bins, N, *rows, s);
@@ -624,14 +629,13 @@ static lisa_status set_data(lisa_like_t *h, double f0, double df, int64_t n_bins
         cleanup();
         return cuda_fail(h, e, "device allocation (data)");
     }
-    double *hpart = nullptr;
-    int *hbad = nullptr;
-    if ((e = cudaMallocHost(&hpart, sizeof(double) * nblk)) != cudaSuccess ||
-        (e = cudaMallocHost(&hbad, sizeof(int))) != cudaSuccess) {
-        if (hpart) cudaFreeHost(hpart);
+    if (!h->h_dd && (e = cudaMallocHost(&h->h_dd, sizeof(double) * (kPrepBlocks + 1))) != cudaSuccess) {
+        h->h_dd = nullptr;
         cleanup();
         return cuda_fail(h, e, "pinned allocation (data)");
     }
+    double *hpart = h->h_dd;
+    int *hbad = reinterpret_cast<int *>(hpart + kPrepBlocks);
     *hbad = 0;
     lisa_status st = LISA_OK;
     do {
@@ -649,21 +653,18 @@ static lisa_status set_data(lisa_like_t *h, double f0, double df, int64_t n_bins
     if (st == LISA_OK && *hbad) st = fail(h, LISA_ERR_ARG, "psd must be finite and > 0 and d finite");
     if (st == LISA_ERR_TIMEOUT || st == LISA_ERR_CUDA) {
         // the device may still be using these: release them at destroy, after a sync
-        void *keep[] = {dd_dev, psd_dev, ddpart, bad, bins, hpart, hbad};
+        void *keep[] = {dd_dev, psd_dev, ddpart, bad, bins, h->h_dd};
         for (void *p : keep)
             if (p) h->deferred.push_back(p);
+        h->h_dd = nullptr;
         return st;
     }
     if (st != LISA_OK) {
-        cudaFreeHost(hpart);
-        cudaFreeHost(hbad);
         cleanup();
         return st;
     }
     double ddv = 0.0;
     for (int i = 0; i < nblk; i++) ddv += hpart[i];
-    cudaFreeHost(hpart);
-    cudaFreeHost(hbad);
     cudaFree(psd_dev);
     if (dd_dev) cudaFree(dd_dev);
     cudaFree(ddpart);
@@ -680,8 +681,19 @@ static lisa_status set_data(lisa_like_t *h, double f0, double df, int64_t n_bins
         cudaFree(bins);
         return cuda_fail(h, e, "device allocation (partial sums / dense data)");
     }
-    // (the present data stay until the new ones are ready)
-    e = split ? launch_prep_split(bins, N, bins32, s) : make_rows(bins, N, &rows, s);
+    // (the present data stay until the new ones are ready, but for a second copy of the same size,
+    // which the new one replaces: it can be made again)
+    if (split) {
+        e = launch_prep_split(bins, N, bins32, s);
+    } else if (h->rows && fx_chunks(N) == fx_chunks(h->N) && !one_copy()) {
+        rows = h->rows;
+        h->rows = nullptr;
+        drop_graph(h);
+        e = cudaDeviceSynchronize();  // calls in flight on other streams read it
+        if (e == cudaSuccess) e = launch_prep_fx(bins, N, rows, s);
+    } else {
+        e = make_rows(bins, N, &rows, s);
+    }
     if (e != cudaSuccess) {
         cudaFree(part);
         if (bins32) cudaFree(bins32);

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const double *d, const double
 
 int prep_blocks(int N) {
     const int b = (N + 255) / 256;
-    return b < 4096 ? b : 4096;
+    return b < kPrepBlocks ? b : kPrepBlocks;
 }
 
 cudaError_t launch_prep(const double *d, const double *psd, int N, double df, double *bins,
