@@ -25,8 +25,6 @@ __host__ __device__ __forceinline__ Bal bal(i64 x) {
     return r;
 }
 
-__host__ __device__ __forceinline__ Bal neg(Bal a) { return Bal{-a.h, -a.l}; }
-
 // cross terms h l' + l h' of a product, in units of 2^32
 __host__ __device__ __forceinline__ i64 cross(Bal a, Bal b) {
     return (i64)a.h * b.l + (i64)a.l * b.h;

@@ -50,11 +50,6 @@ __host__ __device__ inline cplx cmul(cplx a, cplx b) {
 __host__ __device__ inline cplx cadd(cplx a, cplx b) { return {a.re + b.re, a.im + b.im}; }
 __host__ __device__ inline cplx csub(cplx a, cplx b) { return {a.re - b.re, a.im - b.im}; }
 __host__ __device__ inline cplx cscale(cplx a, double s) { return {a.re * s, a.im * s}; }
-__device__ inline cplx cexpi(double ph) {
-    double s, c;
-    sincos(ph, &s, &c);
-    return {c, s};
-}
 
 // Per-walker constants of the mode model (the "fitting constants" the paper
 // computes on the host; here they are derived on the device).
@@ -156,33 +151,11 @@ __device__ inline bool make_source_core(const double *th, double t0, Source &s) 
     return true;
 }
 
-// peak of f^2 A_22 (t_coal is reached there, Sec. II): bisection on the sign of its
-// log-derivative over [x_RD/4, 2 x_RD]
-__device__ inline double find_peak(const Source &s) {
-    double lo = 0.25 * s.xrd, hi = 2.0 * s.xrd;
-    if (peak_equation(s, lo) <= 0.0) return lo;
-    if (peak_equation(s, hi) >= 0.0) return hi;
-    for (int it = 0; it < 200 && hi - lo > 1e-14 * hi; it++) {
-        const double mid = 0.5 * (lo + hi);
-        if (peak_equation(s, mid) > 0.0)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    return 0.5 * (lo + hi);
-}
-
 // align the (2,2) phase at the peak: t_22(f_peak) = t_coal and phi_22(f_peak) = 0
 __device__ inline void set_peak(Source &s, double xpk) {
     s.xpk = xpk;
     s.phpk = raw_phase(s, xpk);
     s.dphpk = raw_slope(s, xpk);
-}
-
-__device__ inline bool make_source(const double *th, double t0, Source &s) {
-    if (!make_source_core(th, t0, s)) return false;
-    set_peak(s, find_peak(s));
-    return true;
 }
 
 // ---------------------------------------------------------------- harmonic modes
@@ -204,12 +177,6 @@ struct Mode {
 // mode-mapped (2,2) argument x = 2 M f / m
 __device__ inline double mapped_x(const Source &s, const Mode &md, double f) {
     return 2.0 * s.M * f / md.m;
-}
-
-// Eq. (6): t_lm(f) = t_coal - (1/2pi) dphi_lm/df = t_22(2 f / m)
-__device__ inline double mode_time(const Source &s, const Mode &md, double f) {
-    const double x = mapped_x(s, md, f);
-    return s.tc - s.M / kTwoPi * (raw_slope(s, x) - s.dphpk);
 }
 
 __device__ inline double amp_ratio(const Source &s, const Mode &md, double v) {
@@ -236,24 +203,6 @@ __device__ inline double phase_offset(const Mode &md) {
         case 5: return -0.5 * kPi;
         default: return 0.0;
     }
-}
-
-// Eq. (5): A_lm(f) of the stand-in mode model
-__device__ inline double mode_amp(const Source &s, const Mode &md, double f) {
-    const double x = mapped_x(s, md, f);
-    const double v = cbrt(kPi * x);
-    const double r = x / s.xrd;
-    const double r2 = r * r;
-    const double a22 = s.amp0 * pow(x, -7.0 / 6.0) * exp(s.al2 * v * v + s.al3 * v * v * v) /
-                       (1.0 + r2 * r2 * r2);
-    return amp_ratio(s, md, v) * a22;
-}
-
-// Eq. (5): phi_lm(f) = (m/2) phi_22(2 f / m) + const, phi_22 aligned at the peak
-__device__ inline double mode_phase(const Source &s, const Mode &md, double f) {
-    const double x = mapped_x(s, md, f);
-    const double p22 = raw_phase(s, x) - s.phpk - s.dphpk * (x - s.xpk);
-    return 0.5 * md.m * p22 + phase_offset(md);
 }
 
 // A_lm(f), phi_lm(f) and t_lm(f) together (Eqs. (5), (6)), sharing one cube root:
@@ -376,13 +325,6 @@ __device__ inline void constellation(double t, double p0[3], double q[3][3]) {
         q[i][1] = pre * (s1 - 3.0 * sbv[i]);
         q[i][2] = -2.0 * sqrt(3.0) * pre * c2;
     }
-}
-
-// SSB -> constellation-centre delay phase -2 pi f k.p0(t)
-__device__ inline double delay_phase(const Frame &fr, double f, double t) {
-    double p0[3], q[3][3];
-    constellation(t, p0, q);
-    return -kTwoPi * f * (fr.k[0] * p0[0] + fr.k[1] * p0[1] + fr.k[2] * p0[2]);
 }
 
 // TDI A, E, T transfer of one mode at (f, t), Eqs. (7)-(10).  The two directions of an
