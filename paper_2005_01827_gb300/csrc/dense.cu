@@ -40,8 +40,8 @@
 // per bin, float pairs) are read from L2 by each walker.
 //
 // Bound by the multiply-add pipe (66 % busy: 185 integer multiply-adds per (walker, mode,
-// bin), 58 % of issue slots).  1024 walkers, six modes, 1-yr grid: 951 -> 216 ms; 37 walkers,
-// four modes, quarter-year grid: 2063 -> 917 us; one walker, (2,2), 30 days: 61 -> 35 us.
+// bin), 58 % of issue slots).  1024 walkers, six modes, 1-yr grid: 951 -> 215.5 ms; 37 walkers,
+// four modes, quarter-year grid: 2063 -> 887 us; one walker, (2,2), 30 days: 61 -> 35 us.
 #include "f32x2.cuh"
 #include "fixed.cuh"
 #include "kernels.h"
@@ -71,12 +71,14 @@ constexpr int kLoose = 12;
 // One (mode, segment) in a warp's block of bins, at the block's first bin or 3 bins before
 // the segment's first one (a thread's 4 bins may begin there): value and forward differences of the
 // seven series in fixed point, and (index kSer) of the phase in fractions of a turn scaled by
-// 2^64; l2, l3 and low hold the next 32 bits of the differences.
+// 2^64; lo and low hold the next 32 bits of the differences.  A series is read by three loads, of 16, 16
+// and 8 bytes (its differences in arrays of their own, by five: 218.3 against 215.5 ms of 1024
+// walkers, 925 against 887 us of 37, and up to 15 % of calls with many short segments).
 struct __align__(16) Expand {
     i64 vd[kSer + 1][2];  // value, first difference
-    i64 d2[kSer + 1];
-    i64 d3[kSer + 1];
-    uint32_t l2[kSer], l3[kSer], low[3];
+    i64 dd[kSer + 1][2];  // second, third difference
+    uint2 lo[kSer];       // of the second and the third
+    uint32_t low[3];
     int org, kb, next;    // origin, first bin of the segment and of the next one
 };
 static_assert(sizeof(Expand) == 336, "16-byte loads of a series' value and first difference");
@@ -329,16 +331,18 @@ __device__ __forceinline__ int bound_of(const double d[4], int n1) {
 __device__ __forceinline__ void series_put(Expand *e, int q, const double d[4], int bound) {
     e->vd[q][0] = __double_as_longlong(d[0]);
     e->vd[q][1] = __double_as_longlong(d[1]);
-    e->d2[q] = __double_as_longlong(d[2]);
-    e->d3[q] = __double_as_longlong(d[3]);
-    e->l3[q] = (uint32_t)bound;
+    e->dd[q][0] = __double_as_longlong(d[2]);
+    e->dd[q][1] = __double_as_longlong(d[3]);
+    e->lo[q].x = (uint32_t)bound;
 }
 
 __device__ __forceinline__ void series_fix(Expand *e, int q, int s) {
     e->vd[q][0] = to_fixed(__longlong_as_double(e->vd[q][0]), s);
     e->vd[q][1] = to_fixed(__longlong_as_double(e->vd[q][1]), s);
-    e->d2[q] = to_fixed96(__longlong_as_double(e->d2[q]), s, e->l2[q]);
-    e->d3[q] = to_fixed96(__longlong_as_double(e->d3[q]), s, e->l3[q]);
+    uint2 lo;
+    e->dd[q][0] = to_fixed96(__longlong_as_double(e->dd[q][0]), s, lo.x);
+    e->dd[q][1] = to_fixed96(__longlong_as_double(e->dd[q][1]), s, lo.y);
+    e->lo[q] = lo;
 }
 
 struct Diff {
@@ -349,12 +353,14 @@ struct Diff {
 __device__ __forceinline__ Diff series_at(const Expand *__restrict__ e, int q, uint32_t n, uint32_t c2,
                                           uint32_t c3) {
     const longlong2 a = *reinterpret_cast<const longlong2 *>(e->vd[q]);
-    const i64 d2 = e->d2[q], d3 = e->d3[q];
+    const longlong2 dd = *reinterpret_cast<const longlong2 *>(e->dd[q]);
+    const i64 d2 = dd.x, d3 = dd.y;
+    const uint2 lo = e->lo[q];
     Diff r;
     i64 v = mad_u((uint32_t)a.y, n, a.x);
     v = mad_u((uint32_t)d2, c2, v);
     v = mad_u((uint32_t)d3, c3, v);
-    v += (i64)(__umulhi(c2, e->l2[q]) + __umulhi(c3, e->l3[q]));
+    v += (i64)(__umulhi(c2, lo.x) + __umulhi(c3, lo.y));
     r.v = add_hi(v, (uint32_t)(a.y >> 32) * n + (uint32_t)(d2 >> 32) * c2 + (uint32_t)(d3 >> 32) * c3);
     i64 d1 = mad_u((uint32_t)d2, n, a.y);
     d1 = mad_u((uint32_t)d3, c2, d1);
@@ -367,7 +373,8 @@ __device__ __forceinline__ Diff series_at(const Expand *__restrict__ e, int q, u
 __device__ __forceinline__ void phase_at(const Expand *__restrict__ e, uint32_t n, uint32_t c2, uint32_t c3,
                                          i64 p[4]) {
     const longlong2 a = *reinterpret_cast<const longlong2 *>(e->vd[kSer]);
-    const i64 d2 = e->d2[kSer], d3 = e->d3[kSer];
+    const longlong2 dd = *reinterpret_cast<const longlong2 *>(e->dd[kSer]);
+    const i64 d2 = dd.x, d3 = dd.y;
     i64 v = mad_u((uint32_t)a.y, n, a.x);
     v = mad_u((uint32_t)d2, c2, v);
     v = mad_u((uint32_t)d3, c3, v);
@@ -414,7 +421,6 @@ __device__ __forceinline__ double scaled_sum(float2 sum, float2 comp, int k) {
 
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
-// a thread's rows in shared memory, padded to an odd number of 16-byte units
 // G walkers per group; kRaw: data rows converted from the FP64 rows as they are used (callers
 // that bring their own rows) instead of read in the dense kernel's form.
 template <int G, bool kRaw>
@@ -577,8 +583,8 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                                 const i64 c2 = (i64)nn * (nn - 1) / 2;
                                 e->vd[kSer][0] = p.ph;
                                 e->vd[kSer][1] = p.d1;
-                                e->d2[kSer] = p.d2;
-                                e->d3[kSer] = p.d3;
+                                e->dd[kSer][0] = p.d2;
+                                e->dd[kSer][1] = p.d3;
                                 e->low[0] = (uint32_t)((r[4] + (i64)nn * r[5] + c2 * r[6]) >> 32);
                                 e->low[1] = (uint32_t)((r[5] + (i64)nn * r[6]) >> 32);
                                 e->low[2] = (uint32_t)(r[6] >> 32);
@@ -605,12 +611,12 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                             if (lane < tasks) {
                                 const Expand *e = ex + lane;
                                 ts = (s_task[warp][lane] & 15) / L;
-                                ea = (int)e->l3[0];
+                                ea = (int)e->lo[0].x;
                                 auto at0 = [&](int q) { return exponent_of(__longlong_as_double(e->vd[q][0])); };
                                 int top = ea, loose = 0;
 #pragma unroll
                                 for (int c = 0; c < 3; c++) {
-                                    et[c] = max((int)e->l3[1 + 2 * c], (int)e->l3[2 + 2 * c]);
+                                    et[c] = max((int)e->lo[1 + 2 * c].x, (int)e->lo[2 + 2 * c].x);
                                     top = max(top, et[c]);
                                     if (et[c] > -1900)  // not all zero
                                         loose = max(loose, et[c] - max(at0(1 + 2 * c), at0(2 + 2 * c)));
@@ -647,14 +653,14 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                             }
                             if (lane < tasks) {  // the binary scale of every series
                                 Expand *e = ex + lane;
-                                e->l3[0] = (uint32_t)(kABits - ea);
+                                e->lo[0].x = (uint32_t)(kABits - ea);
 #pragma unroll
                                 for (int q = 1; q < kSer; q++)
-                                    e->l3[q] = (uint32_t)(kTBits - (sc[(q - 1) >> 1] - ea));
+                                    e->lo[q].x = (uint32_t)(kTBits - (sc[(q - 1) >> 1] - ea));
                             }
                             __syncwarp();
                             for (int i = lane; i < tasks * kSer; i += 32)
-                                series_fix(ex + i / kSer, i % kSer, (int)ex[i / kSer].l3[i % kSer]);
+                                series_fix(ex + i / kSer, i % kSer, (int)ex[i / kSer].lo[i % kSer].x);
                             __syncwarp();
                         }
                         const int fc = s_first[warp][unit];
@@ -724,7 +730,7 @@ __global__ void __launch_bounds__(32 * kWarps, 2) dense_f64_kernel(StageDims d, 
                                 if (i < kC - 3) {
                                     ph[2] += ph[3];
 #pragma unroll
-                                    for (int q = 0; q < kSer; q++) s[q].d2 += e->d3[q];
+                                    for (int q = 0; q < kSer; q++) s[q].d2 += e->dd[q][1];
                                 }
                             }
                         }
