@@ -9,11 +9,11 @@
 // thread sweeps a chunk of rows of its own after a run-in of halo rows, and a sweep of 1022 rows
 // takes 64 steps instead of 1022.  The rows of the run-in grow towards low frequencies, M of the
 // phase as f^(-11/3), r^(11/3) a row: of the row's own value the run-in's start is left with
-// (r^(11/3) / (1 + r + sqrt(1 + r + r^2)))^halo.  With few knots that falls slowly (40 knots over five
-// decades: 0.7 a row), so below 192 knots the run-in is 64 rows, which is every row up to
-// K = 66, and 32 from there on: less than 4e-16 of a row's own value and 2e-15 rad of a phase of 1e5
-// rad, over up to six decades (with 32 throughout: 40 knots over four decades 6e-9 and 3e-11 rad, over five
-// 2e-6 and 8e-10 rad).  The pivots forget by r / (1 + r + sqrt(1 + r + r^2))^2, 0.07, a row and do not
+// (r^(11/3) / (1 + r + sqrt(1 + r + r^2)))^halo.  With few knots over several decades that falls slowly
+// (40 knots over five: 0.7 a row), so the run-in follows from r: 32 rows for 128 knots over two decades
+// or 1024 over any, 37 for 128 and 51 for 64 knots over five decades (with 32 throughout 40
+// knots were off by 6e-9 of the row's own value over four decades, 3e-11 rad of a phase of 1e5 rad, and by 2e-6
+// over five).  The pivots forget by r / (1 + r + sqrt(1 + r + r^2))^2, 0.07, a row and do not
 // grow: 16 rows.
 //
 // What bounds it: with few systems the latency of the sweep steps, so the series are dealt
@@ -32,8 +32,14 @@ namespace lisa {
 
 namespace {
 constexpr int kThreads = 256;
-// run-in rows of a sweep
-__device__ __forceinline__ int sweep_halo(int K) { return K < 192 ? 64 : 32; }
+// run-in rows of a sweep of n rows at the step ratio r = x1 / x0 of its knots: until less than 2^-53 of
+// a row's own value is left of what it started from
+__device__ __forceinline__ int sweep_halo(double x0, double x1, int n) {
+    const float r = (float)x1 / (float)x0;
+    const float lost = log2f(1.0f + r + sqrtf(fmaf(r, r, 1.0f + r))) - 11.0f / 3.0f * log2f(r);  // bits a row
+    const float rows = 54.0f / lost;
+    return lost > 0.0f && rows < (float)n ? max(32, (int)rows + 1) : n;
+}
 constexpr int kPivotHalo = 16;   // run-in rows of the pivots
 constexpr size_t kMaxSmem = 227 * 1024;
 }  // namespace
@@ -91,9 +97,9 @@ __device__ __forceinline__ T sweep_backward(T *y, const T *c, const Rows R, int 
 // entries that the neighbours' chunks overwrite, hence stages of their own.
 template <typename T>
 __device__ __forceinline__ void solve_stage(int stage, T &v, T *y, const T *h, const T *ih,
-                                            const T *sd, const T *c, const Rows R, int t, int n) {
+                                            const T *sd, const T *c, const Rows R, int t, int n, int halo) {
     const int C = R.mask + 1;
-    const int i0 = 1 + t * C, i1 = min(i0 + C, n - 1), halo = sweep_halo(n);
+    const int i0 = 1 + t * C, i1 = min(i0 + C, n - 1);
     if (stage == 4) {  // M_0 and M_{K-1} from their neighbours
         if (t != 0) return;
         const T h0 = h[R.at(0)], h1 = h[R.at(1)], ha = h[R.at(n - 3)], hb = h[R.at(n - 2)];
@@ -131,6 +137,7 @@ __global__ void __launch_bounds__(kThreads) spline_kernel(StageDims d, StageBufs
     float *ys32 = c32 + NP;  // split: [per][NP] (phase slot unused)
     const bool own32 = kSplit && !(per == 1 && q0 == 1);
     const double *x = b.fk + wm * K;
+    const int halo = sweep_halo(x[0], x[1], n);
     const double *yg = b.vals + wm * kNSeries * (size_t)K;
     const float *y32g = split_vals32(b.vals, wm, K);
 
@@ -224,9 +231,9 @@ __global__ void __launch_bounds__(kThreads) spline_kernel(StageDims d, StageBufs
     for (int stage = 0; stage < 5; stage++) {
         if (ql < per) {
             if (kSplit && q0 + ql != 1)
-                solve_stage<float>(stage, v32, ys32 + (size_t)ql * NP, h32, ih32, sd32, c32, R, t, n);
+                solve_stage<float>(stage, v32, ys32 + (size_t)ql * NP, h32, ih32, sd32, c32, R, t, n, halo);
             else
-                solve_stage<double>(stage, v64, ys + (size_t)(kSplit ? 0 : ql) * NP, h, ih, sd, c, R, t, n);
+                solve_stage<double>(stage, v64, ys + (size_t)(kSplit ? 0 : ql) * NP, h, ih, sd, c, R, t, n, halo);
         }
         __syncthreads();
     }
