@@ -47,13 +47,15 @@ WORKLOAD_C3 = ("8192 walkers with M_T log-uniform in [1e3, 1e9] Msun, 6 modes, K
 FLOP_MODE_BIN = 75
 FLOP_BIN = 25
 # The implementations' own counts, reported beside it.  The FP64 dense kernel runs in 64-bit
-# fixed point on the integer units: about 185 multiply-adds of two 32-bit integers per
-# (walker, mode, bin) (ncu's opcode counts over the launch's units), of which an SM does 56
-# a clock (measured; a 32 x 32 -> 64 multiply-add).  The split kernel, per (walker, m, bin)
+# fixed point on the integer units; its method takes 84 products of 32-bit integers per
+# (walker, mode, bin): A e^{i phase} and the three channels 42, the phasor 23 for 4 values of m of
+# 6 modes, the seven series moved to a thread's first of 4 bins 7 x 14 / 4, the phase 15 / 4 x 4 / 6.
+# An SM does 56 a clock (measured; a 32 x 32 -> 64 multiply-add).  (The kernel executes 183 instructions
+# of that opcode, moves and parts of 64-bit additions among them.)  The split kernel, per (walker, m, bin)
 # with 4 values of m for 6 modes: quadratics of A T (24 flops), phasor (17), complex
 # multiply-add (24), and the re-expansion of the quartics per 8 bins (14); per (walker, bin)
 # the integrand (29).
-INT_MAD_MODE_BIN = 185
+INT_MAD_MODE_BIN = 42 + 23 * 4 / 6 + 7 * 14 / 4 + 15 / 4 * 4 / 6
 INT_MAD_CLK_SM = 56
 IMPL_FLOP_MODE_BIN = (24 + 17 + 24 + 14) * 4 / 6
 IMPL_FLOP_BIN = 29
@@ -64,8 +66,8 @@ BYTES_BIN = 76
 # (dram__bytes_read.sum + dram__bytes_write.sum over 69,589,136 walker-bins), per tile
 # shape (bins per thread, group); scaled to a launch by its walker-bins.  A shape without
 # a capture reports null.
-TRAFFIC_F64_PER_WALKER_BIN = {(8, 8): (795.31e6 + 4.97e6) / 69589136}
-TRAFFIC_SPLIT_PER_WALKER_BIN = {(8, 8): (376.44e6 + 10.92e6) / 69589136}
+TRAFFIC_F64_PER_WALKER_BIN = {(8, 8): (793.38e6 + 4.84e6) / 69589136}
+TRAFFIC_SPLIT_PER_WALKER_BIN = {(8, 8): (376.57e6 + 4.86e6) / 69589136}
 
 
 def peaks():

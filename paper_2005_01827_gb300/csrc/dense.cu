@@ -39,8 +39,10 @@
 // all issue slots waited for instructions: 428 ms against 219 (below).  The data rows (76 bytes
 // per bin, float pairs) are read from L2 by each walker.
 //
-// Bound by the multiply-add pipe (66 % busy: 185 integer multiply-adds per (walker, mode,
-// bin), 58 % of issue slots).  1024 walkers, six modes, 1-yr grid: 951 -> 215.5 ms; 37 walkers,
+// Bound by the multiply-add pipe and the waits between dependent instructions (pipe 67 % busy,
+// 56 % of issue slots, 2.1 warps waiting per issue): per (walker, mode, bin) the method takes 84
+// products, and 183 instructions of the multiply-add's opcode are executed, moves and parts of
+// 64-bit additions among them.  1024 walkers, six modes, 1-yr grid: 951 -> 215.5 ms; 37 walkers,
 // four modes, quarter-year grid: 2063 -> 887 us; one walker, (2,2), 30 days: 61 -> 35 us.
 #include "f32x2.cuh"
 #include "fixed.cuh"

@@ -7,9 +7,10 @@ namespace lisa {
 
 constexpr int kScratchRows = 9;   // rows of K doubles per (walker, mode) in mscratch
 
-// Device layout of one bin of the uploaded data: the FP64 dense kernel reads the
-// nine doubles w_A, w_E, w_T, (w d)_A re/im, (w d)_E re/im, (w d)_T re/im
-// (w = 4 df / S, Eqs. (3) and (11)); 72 bytes, 16-byte aligned rows of 2 bins.
+// Device layout of one bin of the uploaded data: the nine doubles w_A, w_E, w_T, (w d)_A
+// re/im, (w d)_E re/im, (w d)_T re/im (w = 4 df / S, Eqs. (3) and (11)); 72 bytes, 16-byte
+// aligned rows of 2 bins.  Read by the relative-binning set-up, by the FP64 dense kernel's
+// bin-by-bin evaluation, and by that kernel throughout where it has no rows of its own form.
 constexpr int kBinDoubles = 9;
 
 struct WalkerConst;  // response.cuh

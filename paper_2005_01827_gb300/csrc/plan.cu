@@ -2,8 +2,9 @@
 //
 // Walkers are sorted by their band (the union of their modes' dense-bin ranges) and cut
 // into groups of G consecutive walkers; the group's union range is split into tiles of
-// tile_bins bins, and each (group, tile) is one work item: one bulk copy stages the
-// tile's data in shared memory and every walker of the group reuses it.  Masses that
+// tile_bins bins, and each (group, tile) is one work item.  In split precision one bulk copy
+// stages the tile's data in shared memory for every walker of the group; in FP64 the
+// walkers' warps read their rows from L2.  Masses that
 // span decades give bands of very different lengths; sorting keeps a group's bands
 // alike, and the persistent dense blocks pull items from a counter, so the uneven
 // batch stays balanced.  Everything runs on the device (no host round trip), so a

@@ -229,7 +229,7 @@ __device__ inline double block_sum(double v, double *red) {
 // the response but for their polarisation weights (response.cuh), powers of the edge frequencies
 // are tabulated, divisions by the fiducial and by the bin widths are in the stored
 // data, each ratio is formed once, and the pairs of a mode are summed before its ratio
-// multiplies them (12 operations a pair).  1024 walkers, 128 bins, six modes: 3.67 -> 1.5 ms.
+// multiplies them (12 operations a pair).  1024 walkers, 256 bins (263 edges), six modes: 3.67 -> 1.5 ms.
 __global__ void __launch_bounds__(kRbThreads, 2) rb_walker_kernel(RbDev r, StageDims d, StageBufs b,
                                                                   double *lnL, double *dh,
                                                                   double *hh) {

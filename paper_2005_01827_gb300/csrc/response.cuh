@@ -53,9 +53,10 @@ static __device__ __noinline__ double near_arm_link(double x, double g) {
     return g == 0.0 ? x : sin(x * g) / g;
 }
 
-// cos and sin of 2 pi turns on the integer units (fixed.cuh; |turns| < 2^20), with an absolute error of
-// about 2e-16, like the rounding of a cosine near 1: for unit phasors and angles, not where a small
-// sine counts.  tab: the phasor table of kFxTab entries
+// cos and sin of 2 pi turns on the integer units (fixed.cuh), with an absolute error of about
+// 2e-16 beside the rounding of `turns` itself: like the rounding of a cosine near 1, but a sine or
+// cosine near 0 has fewer correct bits than sincos() gives.  For unit phasors and angles, not
+// where a small sine counts.  tab: the phasor table of kFxTab entries
 __device__ __forceinline__ void phasor_turns(double turns, const FxTab *__restrict__ tab, double &sn, double &cs) {
     const double fr = turns - rint(turns);
     const i64 v = to_fixed(fr, 62);  // |fr| <= 1/2

@@ -13,7 +13,7 @@
 // next 23 bits give a small signed angle (|r| <= pi / 256) whose sine and cosine are
 // short FP32 polynomials.
 //
-// What bounds the dense kernel is the instruction issue (65 % of the slots, FMA pipe 51 %; the
+// What bounds the dense kernel is the instruction issue (64 % of the slots, FMA pipe 49 %; the
 // rest waits on the segment records), so the work per bin is cut to what depends on the bin:
 //  * modes of equal m share the phase, so per segment the preparation sums their A T (complex,
 //    per channel) into one quartic; a thread re-expands it to a quadratic over its chunk, and a bin
