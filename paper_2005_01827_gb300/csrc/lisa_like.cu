@@ -320,8 +320,10 @@ cudaError_t dalloc_first(lisa_like_t *h, T **p, size_t n) {
     return e;
 }
 
+// after a call that may have given the copy back: makes it again where there is room (not after a
+// device failure, with work perhaps still in flight)
 lisa_status rows_back(lisa_like_t *h, bool had, lisa_status st) {
-    if (!had || h->rows || (st != LISA_OK && st != LISA_ERR_OOM)) return st;
+    if (!had || h->rows || st == LISA_ERR_TIMEOUT || st == LISA_ERR_CUDA) return st;
     float4 *rows = nullptr;
     const std::string err = h->err;
     if (make_rows(h->bins, h->N, &rows, h->stream) == cudaSuccess && rows) {

@@ -103,3 +103,28 @@ def test_room_for_others_comes_first(pkg, orc):
     like.close()
     del hog
     torch.cuda.empty_cache()
+
+
+def test_refused_data_leave_the_second_copy(pkg, orc):
+    """Memory so short that an upload takes the second copy's room, and data that are refused
+    then: the old data, and their copy, are in use as before."""
+    import torch
+
+    LL = pkg.lisalike
+    n = 4000003
+    data, th = problem(orc, n, 2)
+    like = pkg.LisaLike(n_knots=64, t0=W.T0_C1, max_batch=2)
+    like.set_data(*data)
+    want = like.loglike(th)
+    bad = data[4].copy()
+    bad[1, n // 2] = 0.0
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    hog = torch.empty(free - (72 * n + 36 * n), dtype=torch.uint8, device="cuda")
+    with pytest.raises(pkg.lisalike.LisaError):
+        like.set_data(*data[:4], bad)
+    assert LL.lisa_like_get_tune(like.h)[1] == 8
+    assert all(np.array_equal(x, y) for x, y in zip(like.loglike(th), want))
+    like.close()
+    del hog
+    torch.cuda.empty_cache()
